@@ -123,7 +123,8 @@ typedef struct kg_options {
                               the N/C + C vectors held); the choice is reported in
                               kg_report.ckpt_every */
   int32_t tile_bits;       /* 0 = automatic; else amplitudes per tile = 2^tile_bits (6..13) */
-  int32_t ctas;            /* 0 = automatic; else CTAs cooperating on the problem */
+  int32_t ctas;            /* 0 = automatic; else CTAs cooperating on the problem.  With both 0, chains
+                              that fit one CTA's registers run there (one CTA, no device-side wait) */
   int32_t flags;           /* KG_FLAG_* */
   double dt;               /* slice length, dt > 0 */
   double breakdown_tol;    /* <= 0: 1e-12 (C128) or 1e-5 (C64); Lanczos stops when
@@ -166,7 +167,8 @@ typedef struct kg_report {
                               [1] stage 2 (stencil inside the tile), [2] group reductions
                               incl. the barrier wait, [3] recurrence scalars and broadcast,
                               [4] small exponential, [5] recombination, [6] sweep setup,
-                              [7] total; zeros otherwise */
+                              [7] total; zeros otherwise.  A single-CTA launch in registers: [0]
+                              the whole Lanczos loop, [4]-[7] as above */
 } kg_report;
 
 typedef struct kg_handle kg_handle;   /* opaque host object; owns no device memory */
@@ -222,16 +224,20 @@ kg_status kg_set_wait_limit_ns(int64_t ns);
 
 /* ---------------------------------------------------------------- batched evaluation
  * Many independent pulses (each its own chain, controls, initial state and target; shared
- * kg_options) evaluated by ONE cooperative persistent launch: the host schedules every problem
+ * kg_options) evaluated side by side.  Schedule left to the library, every L <= 16: one kernel
+ * launch per chain length, on streams of the batch's own that fork from the caller's stream and
+ * join it again; a problem runs on one CTA (L <= 12) or on one cluster of 2^(L-13) CTAs.
+ * Otherwise ONE cooperative persistent launch: the host schedules every problem
  * onto a group of CTAs (largest first, onto the least loaded CTAs); each group synchronises
  * on its own barrier, so small problems run on single CTAs without any grid-wide wait.
- * Complex64 path only (KG_PREC_C64_F64REC).  The launch is CUDA-graph capturable: all
+ * Complex64 path only (KG_PREC_C64_F64REC).  The launch is CUDA-graph capturable either way: all
  * pointers are fixed when the batch is created. */
-typedef struct kg_batch kg_batch;  /* opaque host object; owns no device memory */
+typedef struct kg_batch kg_batch;  /* opaque host object; owns no device memory (and its streams and events) */
 
 typedef struct kg_batch_schedule {
-  int32_t ctas;           /* CTAs of the launch; 0 = every CTA that fits co-resident */
-  int32_t tiles_per_cta;  /* 1 or 2 (0 = 2): a problem of T tiles gets ceil(T/tiles_per_cta) CTAs */
+  int32_t ctas;           /* CTAs of the cooperative launch; 0 = every CTA that fits co-resident */
+  int32_t tiles_per_cta;  /* 1 or 2 (0 = 2): a problem of T tiles gets ceil(T/tiles_per_cta) CTAs.
+                             Both 0: the schedule is left to the library (see above) */
   int32_t reserved0;      /* must be 0 */
   int32_t reserved1;      /* must be 0 */
 } kg_batch_schedule;
@@ -249,15 +255,16 @@ kg_status kg_batch_create(kg_batch** batch, int32_t B, const kg_chain* chains, c
                           const void* const* target, double* fid, double* const* grad, void* workspace,
                           size_t bytes, void* cuda_stream);
 
-/* Enqueue one evaluation of every problem of the batch on the batch's stream (a 64-byte
- * memset of the control block plus one cooperative kernel; capturable in a CUDA graph). */
+/* Enqueue one evaluation of every problem of the batch on the batch's stream (a memset of the
+ * control block, then one kernel per chain length or one cooperative kernel; capturable in a CUDA
+ * graph).  Work enqueued on the stream afterwards waits for every problem. */
 kg_status kg_batch_launch(kg_batch* batch);
 
 /* Wait for the stream and return the device status (as kg_sync). ctas_used (nullable) receives
- * the grid size of the launch. */
+ * the number of CTAs launched. */
 kg_status kg_batch_sync(kg_batch* batch, int32_t* ctas_used);
 
-/* Destroy (host memory only). NULL is a no-op. */
+/* Destroy (host memory, streams and events; launches in flight complete). NULL is a no-op. */
 kg_status kg_batch_destroy(kg_batch* batch);
 
 /* Size of the library's fixed device scratch array used by kg_evaluate_static. */

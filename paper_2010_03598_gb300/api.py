@@ -197,7 +197,8 @@ def fidelity(u: torch.Tensor, engine: KGrape, psi0: torch.Tensor, target: torch.
 
 
 class KGrapeBatch:
-    """Many independent pulses evaluated by one cooperative launch (complex64 path).
+    """Many independent pulses evaluated side by side (complex64 path): one launch per chain length, or, with
+    ``ctas`` or ``tiles_per_cta`` given or a chain above 16 spins, one cooperative launch.
 
     ``chains`` (one ChainSpec per problem) and shared ``opts``; ``u``, ``psi0``, ``target`` are
     lists of device tensors (kept referenced).  ``fid`` (B) and ``grads`` (B x N) are device

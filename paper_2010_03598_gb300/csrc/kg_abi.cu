@@ -190,6 +190,19 @@ kg_status configure_handle(const kg_chain* chain, const kg_options* opts, const 
   const int t = default_tile_bits(chain, opts);
   const int ntiles = 1 << (chain->L - t);
   cudaError_t e;
+  // Schedule left to the library: one tile in registers per CTA where that kernel covers the chain.
+  const bool autosched = opts->tile_bits == 0 && opts->ctas == 0 && !(opts->flags & KG_FLAG_FULL_REORTH);
+  if (autosched && kg::tile_kernel_covers(opts->prec, chain->L)) {
+    h->chain = *chain;
+    h->opts = *opts;
+    if (!(h->opts.breakdown_tol > 0.0)) h->opts.breakdown_tol = (opts->prec == KG_PREC_C128) ? 1e-12 : 1e-5;
+    h->lay = lay;
+    h->device = dev;
+    h->ctas = 1;
+    h->t_bits = chain->L;
+    h->variant = kg::kVariantTile;
+    return KG_OK;
+  }
   // Resident variant when every CTA can keep its tiles in registers/shared memory.
   int variant = kg::kVariantStreaming;
   int ctas = 0;
@@ -336,7 +349,8 @@ static kg_status enqueue(kg_handle* h, const double* u, const void* psi0, const 
   p.prof = (o.flags & KG_FLAG_PHASE_TIMING) ? (long long*)(ws + h->lay.prof) : nullptr;
   cudaError_t e = cudaMemsetAsync(ws + h->lay.ctrl, 0, kg::kCtrlBytes, h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(control block)");
-  e = kg::launch_eval_kernel(o.prec, h->variant, p, h->ctas, h->stream);
+  e = (h->variant == kg::kVariantTile) ? kg::launch_tile_kernel(o.prec, p, h->stream)
+                                       : kg::launch_eval_kernel(o.prec, h->variant, p, h->ctas, h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "cooperative launch of the evaluation kernel");
   h->launches = 1;
   return KG_OK;
@@ -376,7 +390,8 @@ kg_status kg_sync(kg_handle* h, kg_report* rep) {
     rep->launches = h->launches;
     rep->ctas = h->ctas;
     rep->tile_bits = h->t_bits;
-    rep->threads = kg::eval_kernel_threads(h->opts.prec, h->variant, h->t_bits);
+    rep->threads = (h->variant == kg::kVariantTile) ? kg::tile_kernel_threads(h->opts.prec, h->chain.L)
+                                                    : kg::eval_kernel_threads(h->opts.prec, h->variant, h->t_bits);
     rep->ckpt_every = h->opts.ckpt_every;
     rep->reserved0 = 0;
     long long pc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -531,6 +546,12 @@ extern "C" kg_status kg_evaluate_static(const kg_chain* chain, const kg_options*
 }
 
 // ---------------------------------------------------------------- batched evaluation
+// The problems of one chain length: `n` of them from `first` on in the problem table, by clusters of
+// `size` CTAs (0: one tile in registers per CTA).
+struct BatchClass {
+  int L = 0, first = 0, n = 0, size = 0;
+};
+
 struct kg_batch {
   int B = 0;
   kg_options opts{};
@@ -541,12 +562,21 @@ struct kg_batch {
   int ctas = 0;
   size_t clear_off = 0, clear_bytes = 0;  // control block + barrier counters, zeroed per launch
   kg::BatchParams bp{};
+  // Schedule left to the library: one launch per chain length, side by side on streams of the batch's
+  // own, forked from the caller's stream and joined to it.  Empty: the cooperative launch.
+  std::vector<BatchClass> classes;
+  std::vector<cudaStream_t> streams;   // [classes - 1]: the first class runs on the caller's stream
+  std::vector<cudaEvent_t> done;
+  cudaEvent_t fork = nullptr;
 };
 
 namespace {
 
+constexpr size_t kIRingBytes = sizeof(unsigned long long) * 4 * kg::kIRing;
+constexpr int kBatchClassMaxL = 16;  // longest chain of a class: 16 tiles, a cluster of 8
+
 struct BatchLayout {
-  size_t ctrl = 0, bars = 0, reds = 0, probs = 0, item_off = 0, items = 0, total = 0;
+  size_t ctrl = 0, bars = 0, irings = 0, clear = 0, reds = 0, probs = 0, item_off = 0, items = 0, total = 0;
   std::vector<size_t> prob;  // start of each problem's own workspace
   size_t max_items = 0;
 };
@@ -561,8 +591,11 @@ BatchLayout make_batch_layout(int B, const kg_chain* chains, const kg_options* o
     off = align_up(off + bytes);
     return at;
   };
-  l.ctrl = take(64 + sizeof(unsigned long long) * (size_t)B);  // ctrl words, then barrier counters
+  // ctrl words, barrier counters, then (256-byte aligned) the sum rings: one memset
+  l.ctrl = take(align_up(64 + sizeof(unsigned long long) * (size_t)B) + kIRingBytes * (size_t)B);
   l.bars = l.ctrl + 64;
+  l.irings = l.ctrl + align_up(64 + sizeof(unsigned long long) * (size_t)B);
+  l.clear = l.irings + kIRingBytes * (size_t)B - l.ctrl;
   l.reds = take(sizeof(double) * kg::kBatchRedPerGroup * (size_t)B);
   l.probs = take(sizeof(kg::EvalParams) * (size_t)B);
   l.item_off = take(sizeof(int) * (size_t)(kg::kMaxCtas + 1));
@@ -616,6 +649,7 @@ kg_status kg_batch_create(kg_batch** batch, int32_t B, const kg_chain* chains, c
   kg_batch_schedule sc{0, 0, 0, 0};
   if (sched) sc = *sched;
   if (sc.reserved0 || sc.reserved1) return fail(KG_ERR_INVALID_ARG, "schedule reserved fields must be 0");
+  const bool explicit_tiles = sc.tiles_per_cta != 0;
   if (sc.tiles_per_cta == 0) sc.tiles_per_cta = 2;
   if (sc.tiles_per_cta != 1 && sc.tiles_per_cta != 2) return fail(KG_ERR_INVALID_ARG, "tiles_per_cta must be 1 or 2");
   if (sc.ctas < 0 || sc.ctas > kg::kMaxCtas) return fail(KG_ERR_INVALID_ARG, "ctas must be 0..2048");
@@ -638,7 +672,23 @@ kg_status kg_batch_create(kg_batch** batch, int32_t B, const kg_chain* chains, c
   int ctas = sc.ctas > 0 ? std::min(sc.ctas, maxc) : maxc;
   if (ctas < 1) return fail(KG_ERR_UNSUPPORTED, "batch kernel does not fit on this device");
 
-  // ---- schedule: largest problems first, each onto the least loaded CTAs it needs
+  // ---- schedule left to the library: the longest chains first, one class per length
+  std::vector<BatchClass> classes;
+  std::vector<int> order_of(B);  // problem table position -> problem
+  for (int b = 0; b < B; ++b) order_of[b] = b;
+  int max_L = 0;
+  for (int b = 0; b < B; ++b) max_L = std::max(max_L, (int)chains[b].L);
+  if (sc.ctas == 0 && !explicit_tiles && max_L <= kBatchClassMaxL) {
+    std::stable_sort(order_of.begin(), order_of.end(), [&](int a, int c) { return chains[a].L > chains[c].L; });
+    for (int i = 0; i < B; ++i) {
+      const int L = chains[order_of[i]].L;
+      if (classes.empty() || classes.back().L != L)
+        classes.push_back(BatchClass{L, i, 0, kg::tile_kernel_covers(opts->prec, L) ? 0 : 1 << (L - 13)});
+      classes.back().n++;
+    }
+  }
+
+  // ---- else: largest problems first, each onto the least loaded CTAs it needs
   struct Job {
     int b, g;
     double cost;
@@ -682,11 +732,12 @@ kg_status kg_batch_create(kg_batch** batch, int32_t B, const kg_chain* chains, c
   // ---- problem table
   char* ws = (char*)workspace;
   std::vector<kg::EvalParams> probs(B);
-  for (int b = 0; b < B; ++b) {
+  for (int i = 0; i < B; ++i) {
+    const int b = order_of[i];
     const kg_chain& ch = chains[b];
     const Layout pl = make_layout(&ch, opts);
     char* w = ws + lay.prob[b];
-    kg::EvalParams& p = probs[b];
+    kg::EvalParams& p = probs[i];
     p = kg::EvalParams{};
     p.L = ch.L;
     p.N = opts->N;
@@ -722,6 +773,11 @@ kg_status kg_batch_create(kg_batch** batch, int32_t B, const kg_chain* chains, c
     p.Gi = nullptr;
     p.tint = nullptr;
     p.prof = nullptr;
+    p.ctrl = (int*)(ws + lay.ctrl);
+    p.bar = (unsigned long long*)(ws + lay.bars) + b;
+    p.iring = (unsigned long long*)(ws + lay.irings) + (size_t)b * 4 * kg::kIRing;
+    p.red = (double*)(ws + lay.reds) + (size_t)b * kg::kBatchRedPerGroup;
+    p.red_stride = kg::kBatchMaxGroup;
   }
   if ((e = cudaMemcpy(ws + lay.probs, probs.data(), sizeof(kg::EvalParams) * B, cudaMemcpyHostToDevice)) ||
       (e = cudaMemcpy(ws + lay.item_off, item_off.data(), sizeof(int) * (ctas + 1), cudaMemcpyHostToDevice)) ||
@@ -737,13 +793,30 @@ kg_status kg_batch_create(kg_batch** batch, int32_t B, const kg_chain* chains, c
   h->device = dev;
   h->ctas = ctas;
   h->clear_off = lay.ctrl;
-  h->clear_bytes = 64 + sizeof(unsigned long long) * (size_t)B;
+  h->clear_bytes = lay.clear;
   h->bp.probs = (const kg::EvalParams*)(ws + lay.probs);
   h->bp.item_off = (const int*)(ws + lay.item_off);
   h->bp.items = (const kg::BatchItem*)(ws + lay.items);
   h->bp.bars = (unsigned long long*)(ws + lay.bars);
   h->bp.reds = (double*)(ws + lay.reds);
   h->bp.ctrl = (int*)(ws + lay.ctrl);
+  h->classes = classes;
+  if (!classes.empty()) {
+    h->ctas = 0;
+    for (const BatchClass& c : classes) h->ctas += c.n * std::max(c.size, 1);
+    e = cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming);
+    for (size_t i = 1; i < classes.size() && e == cudaSuccess; ++i) {
+      cudaStream_t s = nullptr;
+      cudaEvent_t ev = nullptr;
+      if ((e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking)) == cudaSuccess) h->streams.push_back(s);
+      if (e == cudaSuccess && (e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) == cudaSuccess)
+        h->done.push_back(ev);
+    }
+    if (e != cudaSuccess) {
+      kg_batch_destroy(h);
+      return cuda_fail(e, "streams of the batch");
+    }
+  }
   *batch = h;
   return KG_OK;
 }
@@ -752,6 +825,22 @@ kg_status kg_batch_launch(kg_batch* b) {
   if (!b) return fail(KG_ERR_INVALID_ARG, "batch must not be NULL");
   cudaError_t e = cudaMemsetAsync(b->ws + b->clear_off, 0, b->clear_bytes, b->stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(batch control block)");
+  if (!b->classes.empty()) {
+    const size_t n = b->classes.size();
+    if (n > 1 && (e = cudaEventRecord(b->fork, b->stream)) != cudaSuccess) return cuda_fail(e, "cudaEventRecord(batch)");
+    for (size_t i = 0; i < n; ++i) {
+      const BatchClass& c = b->classes[i];
+      cudaStream_t s = (i == 0) ? b->stream : b->streams[i - 1];
+      if (i > 0 && (e = cudaStreamWaitEvent(s, b->fork, 0)) != cudaSuccess) return cuda_fail(e, "cudaStreamWaitEvent(batch)");
+      const kg::EvalParams* list = b->bp.probs + c.first;
+      e = (c.size == 0) ? kg::launch_tile_list(c.L, b->opts.m, list, c.n, s) : kg::launch_cluster_list(c.size, list, c.n, s);
+      if (e != cudaSuccess) return cuda_fail(e, "launch of a batch class");
+      if (i > 0 && ((e = cudaEventRecord(b->done[i - 1], s)) != cudaSuccess ||
+                    (e = cudaStreamWaitEvent(b->stream, b->done[i - 1], 0)) != cudaSuccess))
+        return cuda_fail(e, "join of a batch class");
+    }
+    return KG_OK;
+  }
   e = kg::launch_batch_kernel(b->bp, b->ctas, b->stream);
   if (e != cudaSuccess) return cuda_fail(e, "cooperative launch of the batch kernel");
   return KG_OK;
@@ -773,6 +862,11 @@ kg_status kg_batch_sync(kg_batch* b, int32_t* ctas_used) {
 }
 
 kg_status kg_batch_destroy(kg_batch* b) {
+  if (b) {
+    for (cudaEvent_t ev : b->done) cudaEventDestroy(ev);
+    for (cudaStream_t s : b->streams) cudaStreamDestroy(s);
+    if (b->fork) cudaEventDestroy(b->fork);
+  }
   delete b;
   return KG_OK;
 }

@@ -892,4 +892,120 @@ __device__ __forceinline__ void tridiag_expv_e1_ff(const double* alpha, const do
   c_im = ff_to_double(yi);
 }
 
+// ---------------------------------------------------------------- float-float square root, reciprocal
+// The FP32 estimate refined by one Newton step carried out in float-float (the residual a - s^2, or
+// 1 - b y, formed exactly with an FMA), about 44 bits.
+__device__ __forceinline__ FF ff_sqrt(FF a) {
+  if (!(a.hi > 0.f)) return FF{0.f, 0.f};
+  const float s = sqrtf(a.hi);
+  const float p = __fmul_rn(s, s);
+  const float e = __fmaf_rn(s, s, -p);                                      // s^2 = p + e exactly
+  const float r = __fadd_rn(__fsub_rn(__fsub_rn(a.hi, p), e), a.lo);       // a - s^2
+  return ff_two_sum(s, __fdiv_rn(r, __fmul_rn(2.f, s)));
+}
+__device__ __forceinline__ FF ff_rcp(FF b) {
+  const float y = __frcp_rn(b.hi);
+  const float p = __fmul_rn(b.hi, y);
+  const float pe = __fmaf_rn(b.hi, y, -p);                                  // b.hi y = p + pe exactly
+  const float r = __fsub_rn(__fsub_rn(__fsub_rn(1.f, p), pe), __fmul_rn(b.lo, y));  // 1 - b y
+  return ff_two_sum(y, __fmul_rn(y, r));
+}
+
+// a x + b y + c z: the three products by FMA TwoProduct, their high parts by two TwoSums, one
+// renormalisation; about 44 bits, in half the dependent instructions of three ff_mul and two ff_add.
+__device__ __forceinline__ FF ff_dot3(FF a, FF x, FF b, FF y, FF c, FF z) {
+  const float p = __fmul_rn(a.hi, x.hi), q = __fmul_rn(b.hi, y.hi), r = __fmul_rn(c.hi, z.hi);
+  const float tp = __fmaf_rn(a.hi, x.lo, __fmaf_rn(a.lo, x.hi, __fmaf_rn(a.hi, x.hi, -p)));
+  const float tq = __fmaf_rn(b.hi, y.lo, __fmaf_rn(b.lo, y.hi, __fmaf_rn(b.hi, y.hi, -q)));
+  const float tr = __fmaf_rn(c.hi, z.lo, __fmaf_rn(c.lo, z.hi, __fmaf_rn(c.hi, z.hi, -r)));
+  const FF s = ff_two_sum(p, r);
+  const FF t = ff_two_sum(s.hi, q);
+  const float lo = __fadd_rn(__fadd_rn(__fadd_rn(tp, tr), tq), __fadd_rn(s.lo, t.lo));
+  const float hi = __fadd_rn(t.hi, lo);
+  return {hi, __fsub_rn(lo, __fsub_rn(hi, t.hi))};
+}
+
+// c = exp(-i tau T) e_1 as tridiag_expv_e1_ff, with T's entries handed over in float-float registers
+// (lane k: diagonal a = alpha_k, off-diagonal b = b_k that couples k - 1 and k; n <= 32): no FP64
+// instruction, and the series as A^p y and 1/p! (as the FP64 version), so that a term's weight is off
+// the chain of dependent terms.  ||A|| <= 4 keeps A^p y below 4^p and the weights above 1/28!, inside
+// the FP32 range, for tol >= 1e-14.
+#define KG_FFF(p) {(float)(1.0 / (p)), (float)(1.0 / (p) - (double)(float)(1.0 / (p)))}
+__device__ __constant__ float2 kInvFactFF[30] = {
+    KG_FFF(1.0), KG_FFF(1.0), KG_FFF(2.0), KG_FFF(6.0), KG_FFF(24.0), KG_FFF(120.0), KG_FFF(720.0), KG_FFF(5040.0),
+    KG_FFF(40320.0), KG_FFF(362880.0), KG_FFF(3628800.0), KG_FFF(39916800.0), KG_FFF(479001600.0),
+    KG_FFF(6227020800.0), KG_FFF(87178291200.0), KG_FFF(1307674368000.0), KG_FFF(20922789888000.0),
+    KG_FFF(355687428096000.0), KG_FFF(6402373705728000.0), KG_FFF(121645100408832000.0),
+    KG_FFF(2432902008176640000.0), KG_FFF(51090942171709440000.0), KG_FFF(1124000727777607680000.0),
+    KG_FFF(25852016738884976640000.0), KG_FFF(620448401733239439360000.0), KG_FFF(15511210043330985984000000.0),
+    KG_FFF(403291461126605635584000000.0), KG_FFF(10888869450418352160768000000.0),
+    KG_FFF(304888344611713860501504000000.0), KG_FFF(8841761993739701954543616000000.0)};
+#undef KG_FFF
+// `fact` is the caller's lane's entry of the table (kInvFactFF[lane], lanes 0..29): the weights come by
+// shuffles and the number of terms by a ballot, as indexed loads from constant memory and a loop over
+// the terms' bounds took three times as long as the series itself.
+__device__ __forceinline__ void tridiag_expv_e1_fff(FF a, FF b, int n, FF tau, float tol, float2 fact, FF& c_re,
+                                                    FF& c_im, float& tnorm) {
+  const int lane = threadIdx.x & 31;
+  if (lane >= n) a = FF{0.f, 0.f};
+  if (lane < 1 || lane >= n) b = FF{0.f, 0.f};
+  const FF bn = ff_shfl_down(b);  // b_{k+1}
+  const FF bh = (lane + 1 < n) ? bn : FF{0.f, 0.f};
+  float row = fabsf(tau.hi) * (fabsf(a.hi) + b.hi + bh.hi);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) row = fmaxf(row, __shfl_xor_sync(0xffffffffu, row, o));
+  tnorm = row;
+  int s = 1;
+  FF h = tau;
+  float r = row * 1.0001f;
+  if (r > 4.f) {
+    s = (int)ceilf(r * 0.25f);
+    const FF si = ff_rcp(FF{(float)s, 0.f});
+    h = ff_mul(tau, si);
+    r *= si.hi;
+  }
+  const FF ha = ff_mul(h, a), hl = ff_mul(h, b), hh = ff_mul(h, bh);  // rows of A = h T
+  // K terms: r^(K+1) / (K+1)!, the bound of the first term left out, is below tol (lane p tests p terms)
+  const float ln = __log2f(r) * (float)(lane + 1) + __log2f(__shfl_down_sync(0xffffffffu, fact.x, 1));
+  const int K = __popc(__ballot_sync(0xffffffffu, lane < 28 && ln >= __log2f(tol) - 0.01f));
+  FF yr{(lane == 0) ? 1.f : 0.f, 0.f}, yi{0.f, 0.f};
+  for (int st = 0; st < s; ++st) {
+    const bool cplx = (st > 0);
+    FF pr = yr, pi = yi;  // A^p y
+    FF ar = yr, ai = yi;  // accumulated result
+    FF tr, ti{0.f, 0.f};
+    auto term = [&](int k) {  // the k-th term's vectors, weighted
+      const FF w{__shfl_sync(0xffffffffu, fact.x, k), __shfl_sync(0xffffffffu, fact.y, k)};
+      pr = ff_dot3(hl, ff_shfl_up(pr), ha, pr, hh, ff_shfl_down(pr));
+      tr = ff_mul(w, pr);
+      if (cplx) {
+        pi = ff_dot3(hl, ff_shfl_up(pi), ha, pi, hh, ff_shfl_down(pi));
+        ti = ff_mul(w, pi);
+      }
+    };
+    // (-i)^k: -i, -1, +i, +1, applied to (tr + i ti)
+    for (int k = 1; k <= K; k += 4) {
+      term(k);
+      ai = ff_add(ai, ff_neg(tr));
+      if (cplx) ar = ff_add(ar, ti);
+      if (k + 1 > K) break;
+      term(k + 1);
+      ar = ff_add(ar, ff_neg(tr));
+      if (cplx) ai = ff_add(ai, ff_neg(ti));
+      if (k + 2 > K) break;
+      term(k + 2);
+      ai = ff_add(ai, tr);
+      if (cplx) ar = ff_add(ar, ff_neg(ti));
+      if (k + 3 > K) break;
+      term(k + 3);
+      ar = ff_add(ar, tr);
+      if (cplx) ai = ff_add(ai, ti);
+    }
+    yr = ar;
+    yi = ai;
+  }
+  c_re = yr;
+  c_im = yi;
+}
+
 }  // namespace kg

@@ -2682,6 +2682,45 @@ __global__ void __launch_bounds__(eval_threads(MODE), 1) kg_eval_kernel(const __
   cta_teardown(ss, kTmem);
 }
 
+// Many problems of one chain length on the resident loop (complex64, two 4096-amplitude tiles per
+// CTA): problem b by the cluster of `size` CTAs b size .. b size + size - 1, which the hardware places
+// together, so that no other launch can keep a member of a group off the device.
+__global__ void __launch_bounds__(kCtlThreads, 1) kg_cluster_list_kernel(const EvalParams* list, int size) {
+  extern __shared__ __align__(16) unsigned char smem_dyn[];
+  __shared__ SmemSlice ss;
+  __shared__ EvalParams p;
+  if (threadIdx.x == 0) p = list[blockIdx.x / size];
+  cta_setup(ss, true);
+  unsigned lz_count = 0u;
+  if (threadIdx.x >= kThreads) {
+    res64b_control(ss);
+  } else {
+    run_eval<float2, float, 8, 2, true, kModeResident64b>(p, blockIdx.x % size, size, ss, smem_dyn, lz_count);
+    if (threadIdx.x == 0) ss.ctl_cmd = kCtlExit;
+    nbar_arrive(kBarPost, kCtlThreads);
+  }
+  cta_teardown(ss, true);
+}
+
+cudaError_t launch_cluster_list(int size, const EvalParams* list, int n, cudaStream_t stream) {
+  cudaError_t err = cudaFuncSetAttribute(kg_cluster_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kRes64bSmemBytes);
+  if (err != cudaSuccess) return err;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n * size));
+  cfg.blockDim = dim3(kCtlThreads);
+  cfg.dynamicSmemBytes = kRes64bSmemBytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)size;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kg_cluster_list_kernel, list, size);
+}
+
 // Many independent problems (complex64) in one cooperative launch.  Every CTA walks its own
 // list of items in the order the host scheduled them; a group of CTAs forms for one problem
 // and uses its own barrier counter.  Lists are ordered consistently (a global sequence), so a

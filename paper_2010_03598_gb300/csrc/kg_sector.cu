@@ -72,23 +72,6 @@ __device__ __forceinline__ FFR operator*(FFR a, FFR b) {
   return FFR(p.hi, p.lo);
 }
 __device__ __forceinline__ FFR fma(FFR a, FFR b, FFR c) { return a * b + c; }
-// Square root and reciprocal: the FP32 estimate refined by one Newton step carried out in
-// float-float (the residual a - s^2, or 1 - b y, formed exactly with an FMA), about 44 bits.
-__device__ __forceinline__ FF ff_sqrt(FF a) {
-  if (!(a.hi > 0.f)) return FF{0.f, 0.f};
-  const float s = sqrtf(a.hi);
-  const float p = __fmul_rn(s, s);
-  const float e = __fmaf_rn(s, s, -p);                                      // s^2 = p + e exactly
-  const float r = __fadd_rn(__fsub_rn(__fsub_rn(a.hi, p), e), a.lo);       // a - s^2
-  return ff_two_sum(s, __fdiv_rn(r, __fmul_rn(2.f, s)));
-}
-__device__ __forceinline__ FF ff_rcp(FF b) {
-  const float y = __frcp_rn(b.hi);
-  const float p = __fmul_rn(b.hi, y);
-  const float pe = __fmaf_rn(b.hi, y, -p);                                  // b.hi y = p + pe exactly
-  const float r = __fsub_rn(__fsub_rn(__fsub_rn(1.f, p), pe), __fmul_rn(b.lo, y));  // 1 - b y
-  return ff_two_sum(y, __fmul_rn(y, r));
-}
 // Scalar operations, once per Lanczos step: comparisons on (hi, lo) in order.
 __device__ __forceinline__ bool ffr_less(FFR a, FFR b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
 __device__ __forceinline__ FFR operator/(FFR a, FFR b) {

@@ -1,0 +1,1211 @@
+// K-GRAPE evaluation with one tile of amplitudes per CTA, held in registers: the forward Krylov
+// sweep, target overlap, co-state sweep and gradient of one pulse, in one launch.
+//
+// For chains whose amplitudes fit the registers of one CTA (or, complex128, of the co-resident CTAs
+// with one tile each) an evaluation is a chain of short Krylov steps, whose cost is latency: block
+// barriers, warp sums, the recurrence's scalars and the small exponential.  This kernel is laid out
+// for that chain.  A CTA has as many threads as its tile needs (a thread owns APT amplitudes
+// li = tid + NT j), one barrier per Lanczos step, and no FP64 instruction on the complex64 path
+// between the first slice and the last: one FP64 instruction occupies a quarter of the SM's FP64
+// unit for 64 cycles whatever the number of active lanes, so padding warps and scalar chains in
+// FP64 are what small chains spend their time on otherwise.
+//
+// One Lanczos step (App. A, Alg. "Lanczos", Paige's order), v_k in shared memory for the neighbours:
+//   W_{k+1} = H v_k - b_k v_{k-1},   H v = diag v + (Jxy/2) sum_{antiparallel bonds} v[partner] (+ control)
+//   alpha_k = <v_k|W_{k+1}>,  b_{k+1}^2 = ||W_{k+1}||^2 - 2 alpha_k <v_k|W_{k+1}> + alpha_k^2 ||v_k||^2
+//   v_{k+1} = (W_{k+1} - alpha_k v_k) / b_{k+1}
+// with two block barriers (the sums, v_{k+1}); every warp adds up the warps' partial sums and forms the
+// scalars for itself.  v_{k-1}, v_k and W stay in registers; the basis holds the v_k (shared memory if
+// it fits, else global).
+//
+// Several CTAs (complex128): the stencil acts on the raw vector W_k, which needs none of the step's
+// scalars, so that it runs while the group's sums are under way:
+//   v_k = (W_k - alpha_{k-1} v_{k-1}) / b_k,   H v_k = (H W_k - alpha_{k-1} H v_{k-1}) / b_k.
+// (On one CTA the waits it would hide are short, and H v_k by its recurrence carries more rounding.)  The tiles' W_k are exchanged through global memory.  A control warp posts
+// the CTA's sums and the group's barrier in one message, a 16-byte {value, sequence number} per sum:
+// every CTA polls the other CTAs' messages and adds them up in the same order, so that one trip
+// through L2 both closes the step and carries its sums.
+#include <cuda_runtime.h>
+
+#include "kg_device.cuh"
+#include "kg_launch.h"
+
+namespace kg {
+namespace {
+
+// ---------------------------------------------------------------- per-precision arithmetic
+// Sum of a reduction, scalar of the recurrence (complex64: float-float sums, FP32 scalars).
+template <class V> struct Prec;
+template <> struct Prec<float2> {
+  using R = float;
+  using S = FF;
+  static constexpr bool F32 = true;
+};
+template <> struct Prec<double2> {
+  using R = double;
+  using S = double;
+  static constexpr bool F32 = false;
+};
+
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ double2 vadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 vmul(float a, float2 x) { return __fmul2_rn(make_float2(a, a), x); }
+__device__ __forceinline__ double2 vmul(double a, double2 x) { return make_double2(a * x.x, a * x.y); }
+__device__ __forceinline__ float2 vfma(float a, float2 x, float2 y) { return __ffma2_rn(make_float2(a, a), x, y); }
+__device__ __forceinline__ double2 vfma(double a, double2 x, double2 y) {
+  return make_double2(fma(a, x.x, y.x), fma(a, x.y, y.y));
+}
+// y + (a + ib) x, the part with b first: a is the larger one where the rounding counts (slot 0)
+__device__ __forceinline__ float2 vcfma(float a, float b, float2 x, float2 y) {
+  return make_float2(fmaf(a, x.x, fmaf(-b, x.y, y.x)), fmaf(a, x.y, fmaf(b, x.x, y.y)));
+}
+__device__ __forceinline__ double2 vcfma(double a, double b, double2 x, double2 y) {
+  return make_double2(fma(a, x.x, fma(-b, x.y, y.x)), fma(a, x.y, fma(b, x.x, y.y)));
+}
+
+__device__ __forceinline__ FF sfrom(double d, FF) { return ff_from_double(d); }
+__device__ __forceinline__ double sfrom(double d, double) { return d; }
+__device__ __forceinline__ double sdouble(FF a) { return ff_to_double(a); }
+__device__ __forceinline__ double sdouble(double a) { return a; }
+__device__ __forceinline__ float sround(FF a) { return __fadd_rn(a.hi, a.lo); }
+__device__ __forceinline__ double sround(double a) { return a; }
+__device__ __forceinline__ bool sfinite(FF a) { return isfinite(a.hi); }
+__device__ __forceinline__ bool sfinite(double a) { return isfinite(a); }
+
+// A sum kept in 8 bytes of a double array (G, nrm) between slices; read back by whoever needs it.
+__device__ __forceinline__ double spack(FF a) {
+  return __hiloint2double(__float_as_int(a.hi), __float_as_int(a.lo));
+}
+__device__ __forceinline__ double spack(double a) { return a; }
+__device__ __forceinline__ FF sunpack(double d, FF) {
+  return FF{__int_as_float(__double2hiint(d)), __int_as_float(__double2loint(d))};
+}
+__device__ __forceinline__ double sunpack(double d, double) { return d; }
+
+__device__ __forceinline__ float sinv(FF n) {
+  const float f = sround(n);
+  return (f > 0.f) ? __frcp_rn(f) : 0.f;
+}
+__device__ __forceinline__ double sinv(double n) { return (n > 0.0) ? 1.0 / n : 0.0; }
+// ||x|| and 1/||x|| from ||x||^2.
+__device__ __forceinline__ void snorm(FF n2, FF& n, float& inv) {
+  n = ff_sqrt(n2);
+  inv = sinv(n);
+}
+__device__ __forceinline__ void snorm(double n2, double& n, double& inv) {
+  n = sqrt(fmax(n2, 0.0));
+  inv = (n > 0.0) ? 1.0 / n : 0.0;
+}
+
+// b^2 = n + a^2 (q - 2), b and 1/b
+__device__ __forceinline__ FF sb2(FF a, FF n, FF q) { return ff_add(n, ff_mul(ff_mul(a, a), ff_add(q, FF{-2.f, 0.f}))); }
+__device__ __forceinline__ double sb2(double a, double n, double q) { return fma(a * a, q - 2.0, n); }
+__device__ __forceinline__ bool scancels(FF b2, FF n) { return b2.hi < 1e-3f * n.hi; }
+__device__ __forceinline__ bool scancels(double b2, double n) { return b2 < 1e-3 * n; }
+// b and 1/b from b^2: the FP32 estimate of 1/sqrt refined by one step of Newton's iteration (complex64:
+// the residual 1 - b^2 y^2 formed exactly, so that both results are rounded once) or of Halley's (FP64:
+// cubic convergence, 2^-22 -> below 2^-60), then b = b^2 / b.
+__device__ __forceinline__ void sroot(FF b2, float& b, float& inv) {
+  const float x = b2.hi;
+  if (!(x > 1e-30f)) {
+    b = __fsqrt_rn(fmaxf(sround(b2), 0.f));
+    inv = (b > 0.f) ? __frcp_rn(b) : 0.f;
+    return;
+  }
+  const float y = rsqrtf(x);
+  const float p = __fmul_rn(x, y);
+  const float e = __fmaf_rn(x, y, -p) + b2.lo * y;  // b2 y = p + e
+  const float r = __fmaf_rn(-p, y, 1.f) - e * y;
+  inv = fmaf(0.5f * r, y, y);
+  const float c = x * inv;
+  b = fmaf(0.5f * inv, fmaf(-c, c, x) + b2.lo, c);
+}
+__device__ __forceinline__ void sroot(double b2, double& b, double& inv) {
+  if (!(b2 > 1e-30 && b2 < 1e30)) {
+    inv = (b2 > 0.0) ? rsqrt(b2) : 0.0;
+    b = fmax(b2, 0.0) * inv;
+    return;
+  }
+  const double y = (double)rsqrtf((float)b2);
+  const double r = fma(-b2 * y, y, 1.0);
+  inv = fma(y, r * fma(0.375, r, 0.5), y);
+  b = b2 * inv;
+}
+
+constexpr int kTileSums = 3;  // values of one reduction
+
+struct TileSmem {
+  float red_f[2][16][4];     // warp partials (complex64: FP32 sums), by reduction parity
+  double red_d[2][16][4];    // warp partials (complex128, and the FP64 overlaps of complex64)
+  double tot[2][4];          // group totals (several CTAs), by parity
+  float2 al_ff[kMaxM], b2_ff[kMaxM];  // complex64: alpha_k, b_{k+1}^2 of the slice (float-float)
+  double al[kMaxM], be[kMaxM + 1];    // complex128: alpha_k, b_{k+1}
+  double coef_re[3][kMaxM], coef_im[3][kMaxM];
+  float coef_re_f[3][kMaxM], coef_im_f[3][kMaxM];
+  float2 tau_ff[3];          // complex64: dt and the interior quadrature nodes s_a, s_b of a slice
+  float err_max;
+  int breakdowns;
+  int cmd, ok;               // control warp: hand-over and answer
+  long long prof_last, prof_acc[8];
+};
+
+// ---------------------------------------------------------------- messages between CTAs
+// 16-byte accesses at one point of the memory system: value and sequence number travel together.
+__device__ __forceinline__ void st_msg(ulonglong2* p, unsigned long long v, unsigned long long seq) {
+  asm volatile("{\n .reg .b128 q;\n mov.b128 q, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], q;\n}" ::"l"(p), "l"(v), "l"(seq)
+               : "memory");
+}
+__device__ __forceinline__ ulonglong2 ld_msg(const ulonglong2* p) {
+  ulonglong2 r;
+  asm volatile("{\n .reg .b128 q;\n ld.relaxed.gpu.global.b128 q, [%2];\n mov.b128 {%0, %1}, q;\n}"
+               : "=l"(r.x), "=l"(r.y)
+               : "l"(p)
+               : "memory");
+  return r;
+}
+
+constexpr int kTileBarPost = 2, kTileBarGroup = 3;
+constexpr int kTileCmdSums = 1, kTileCmdExit = 2;
+
+template <class V, int NT, int APT, bool SB, bool MULTI>
+struct Tile {
+  using P = Prec<V>;
+  using R = typename P::R;
+  using S = typename P::S;
+  static constexpr bool F32 = P::F32;
+  static constexpr int NW = NT / 32;
+  static constexpr int LT = (NT == 32) ? 5 : (NT == 64) ? 6 : (NT == 128) ? 7 : (NT == 256) ? 8 : 9;
+  static constexpr int LA = (APT == 1) ? 0 : (APT == 2) ? 1 : (APT == 4) ? 2 : (APT == 8) ? 3 : 4;
+  static constexpr int T = NT * APT;
+  static constexpr bool RAW = MULTI || APT == 16;  // the stencil acts on the raw vectors
+  static_assert((1 << LT) == NT && (1 << LA) == APT, "powers of two");
+
+  const EvalParams& p;
+  TileSmem& sm;
+  V* sw;        // [2][T] the neighbours' vector, by the parity of the step; SB: [m][T], the basis itself
+  V* ring;      // MULTI: [slots][T] partner blocks of W_k
+  int tid, wid, rank, D1;  // D1: amplitudes of the tile that exist (T, or fewer for chains below 5 spins)
+  size_t base, D;
+  int nb;       // bonds inside the tile
+  int par;      // parity of the next reduction
+  R hxy;
+  R dj[APT];           // diagonal of H_j
+  R cx;                // Sx control weight of the slice
+  double hca;          // hc_amp, times 1/2 for an Sx control
+  unsigned bonds_hi;   // MULTI: active bonds with both bits above the tile, bit b
+  V wo[APT];           // own W_k
+  float2 fact;         // complex64: this lane's entry of kInvFactFF
+  float w1[kTileSums];  // one warp, complex64: its sums
+  S nrm;               // ||W_0||
+  R inv;               // 1 / ||W_0||
+
+  __device__ __forceinline__ void mark(int ph) {
+    if (p.prof != nullptr && rank == 0 && tid == 0) {
+      const long long now = clock64();
+      sm.prof_acc[ph] += now - sm.prof_last;
+      sm.prof_last = now;
+    }
+  }
+
+  __device__ __forceinline__ void sync() {
+    if constexpr (MULTI) asm volatile("barrier.sync 1, %0;" ::"n"(NT) : "memory");
+    else if constexpr (NW == 1) __syncwarp();
+    else asm volatile("barrier.sync 0;" ::: "memory");  // lanes of warp 0 may arrive apart
+  }
+
+  // -------------------------------------------------------------- sums over the block / the group
+  // post: this thread's values into the warp partials (and, MULTI, the hand-over to the control
+  // warp); collect (after the barrier that follows): the totals, the same bits in every thread.
+  __device__ __forceinline__ void post(const R (&v)[kTileSums]) {
+    const int lane = tid & 31, warp = tid >> 5;
+    if constexpr (F32) {
+      float s[kTileSums];
+#pragma unroll
+      for (int i = 0; i < kTileSums; ++i) s[i] = warp_sum(v[i]);
+      if constexpr (NW == 1) {
+        w1[0] = s[0], w1[1] = s[1], w1[2] = s[2];
+        return;
+      }
+      if (lane < kTileSums) sm.red_f[par][warp][lane] = (lane == 0) ? s[0] : (lane == 1) ? s[1] : s[2];
+    } else {
+      // transposed butterfly: a lane ends up with one of four values, six additions instead of fifteen
+      const bool o1 = lane & 1, o2 = lane & 2;
+      const double a0 = o1 ? v[1] : v[0], g0 = o1 ? v[0] : v[1];
+      const double a1 = o1 ? 0.0 : v[2], g1 = o1 ? v[2] : 0.0;
+      const double s0 = a0 + __shfl_xor_sync(0xffffffffu, g0, 1);
+      const double s1 = a1 + __shfl_xor_sync(0xffffffffu, g1, 1);
+      double s = (o2 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, o2 ? s0 : s1, 2);
+#pragma unroll
+      for (int o = 4; o <= 16; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane < kTileSums) sm.red_d[par][warp][lane] = s;  // lane 0: v0, 1: v1, 2: v2
+    }
+    if constexpr (MULTI) {
+      if (tid == 0) sm.cmd = kTileCmdSums | (par << 2);
+      nbar_arrive(kTileBarPost, NT + 32);
+    }
+  }
+  __device__ __forceinline__ bool collect(S (&out)[kTileSums]) {
+    const int lane = tid & 31;
+    if constexpr (MULTI) {
+      nbar_sync(kTileBarGroup, NT + 32);
+#pragma unroll
+      for (int i = 0; i < kTileSums; ++i) out[i] = sfrom(sm.tot[par][i], S());
+      par ^= 1;
+      return sm.ok != 0;
+    } else if constexpr (F32 && NW == 1) {
+#pragma unroll
+      for (int i = 0; i < kTileSums; ++i) out[i] = FF{w1[i], 0.f};
+    } else if constexpr (F32) {
+#pragma unroll
+      for (int i = 0; i < kTileSums; ++i) {
+        FF s{sm.red_f[par][lane & (NW - 1)][i], 0.f};
+#pragma unroll
+        for (int o = 1; o < NW; o <<= 1)
+          s = ff_add(s, FF{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)});
+        out[i] = s;
+      }
+      par ^= 1;
+    } else {
+      // lane = 4 w + i adds value i over the warps w
+      double s = sm.red_d[par][(lane >> 2) & (NW - 1)][lane & 3];
+#pragma unroll
+      for (int o = 1; o < NW; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, 4 * o);
+#pragma unroll
+      for (int i = 0; i < kTileSums; ++i) out[i] = __shfl_sync(0xffffffffu, s, i);
+      par ^= 1;
+    }
+    return true;
+  }
+  // Sums of FP64 values whatever the path (overlap with the complex128 target): twice an evaluation.
+  __device__ __forceinline__ bool sum_fp64(const double (&v)[kTileSums], double (&out)[kTileSums]) {
+    const int lane = tid & 31, warp = tid >> 5;
+    if constexpr (!F32) {
+      post(v);
+      if constexpr (!MULTI) sync();
+      return collect(out);
+    } else {
+#pragma unroll
+      for (int i = 0; i < kTileSums; ++i) {
+        const double s = warp_sum(v[i]);
+        if (lane == 0) sm.red_d[par][warp][i] = s;
+      }
+      sync();
+#pragma unroll
+      for (int i = 0; i < kTileSums; ++i) {
+        double s = sm.red_d[par][lane & (NW - 1)][i];
+#pragma unroll
+        for (int o = 1; o < NW; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        out[i] = s;
+      }
+      par ^= 1;
+      return true;
+    }
+  }
+
+  // -------------------------------------------------------------- setup
+  __device__ __forceinline__ int li(int j) const { return tid + j * NT; }
+  __device__ __forceinline__ void init() {
+    wid = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    hxy = (R)(0.5 * p.Jxy);
+    hca = (p.hc_kind == KG_HC_SX_SITE) ? 0.5 * p.hc_amp : p.hc_amp;
+    nb = MULTI ? LT + LA - 1 : min(p.L - 1, LT + LA - 1);
+    bonds_hi = 0u;
+    fact = kInvFactFF[min(tid & 31, 29)];
+    if (F32 && tid == 0) {
+      const double s = 0.5 * p.dt * (1.0 - 0.4472135954999579);  // 1/sqrt(5)
+      const FF t[3] = {ff_from_double(p.dt), ff_from_double(s), ff_from_double(p.dt - s)};
+      for (int i = 0; i < 3; ++i) sm.tau_ff[i] = make_float2(t[i].hi, t[i].lo);
+    }
+    if constexpr (MULTI)
+      bonds_hi = (unsigned)((base ^ (base >> 1)) & ((1u << (p.L - 1)) - 1u)) & ~((1u << (LT + LA)) - 1u);
+  }
+  // Diagonal of Hc = hc_amp sum Sz over the mask, in units of hc_amp.
+  __device__ __forceinline__ R zdiag(int j) const {
+    const unsigned mk = (unsigned)p.hc_mask, gi = (unsigned)(base + li(j));
+    return (R)(0.5f * (float)(__popc(mk) - 2 * __popc(gi & mk)));
+  }
+  __device__ __forceinline__ void set_control(double uj) {
+    const bool sx = (p.hc_kind == KG_HC_SX_SITE);
+    const R c = (R)(uj * hca);
+    cx = sx ? c : (R)0;
+    const unsigned maskL1 = (p.L >= 2) ? ((1u << (p.L - 1)) - 1u) : 0u;
+    const R qz = (R)(0.25 * p.Jz);
+#pragma unroll
+    for (int j = 0; j < APT; ++j) {
+      const unsigned gi = (unsigned)(base + li(j));
+      dj[j] = qz * (R)((p.L - 1) - 2 * __popc((gi ^ (gi >> 1)) & maskL1));
+      if (!sx) dj[j] = fma(c, zdiag(j), dj[j]);
+    }
+  }
+
+  // -------------------------------------------------------------- H x inside the tile
+  // s: the tile's vector in shared memory; x: the own amplitudes of the same vector.
+  __device__ __forceinline__ void stencil(const V* s, const V (&x)[APT], V (&h)[APT]) {
+#pragma unroll
+    for (int j = 0; j < APT; ++j) h[j] = vmake<V>(0, 0);
+    const unsigned xt = (unsigned)(tid ^ (tid >> 1));
+    // Bonds with a bit inside the warp: every lane loads its partner and adds it times 0 or 1, so that
+    // no branch separates the loads (with the loads under the lane's condition each bond's latency was
+    // waited for by itself: 24.2 us a slice at L = 10, m = 16 instead of 22.2).
+#pragma unroll
+    for (int b = 0; b < (LT - 1 < 5 ? LT - 1 : 5); ++b) {
+      if (b < nb) {
+        const V* q = s + (tid ^ (3 << b));
+        const R on = (R)(float)((xt >> b) & 1u);
+#pragma unroll
+        for (int j = 0; j < APT; ++j) h[j] = vfma(on, q[j * NT], h[j]);
+      }
+    }
+#pragma unroll
+    for (int b = 5; b < LT - 1; ++b) {  // both bits in the warp's number: the same for all lanes
+      if (((wid >> (b - 5)) ^ (wid >> (b - 4))) & 1) {
+        const V* q = s + (tid ^ (3 << b));
+#pragma unroll
+        for (int j = 0; j < APT; ++j) h[j] = vadd(h[j], q[j * NT]);
+      }
+    }
+    if constexpr (APT > 1) {
+      const int tt = (tid >> (LT - 1)) & 1;  // top bit of tid against bit 0 of j
+#pragma unroll
+      for (int j = 0; j < APT; ++j)
+        if (tt != (j & 1)) h[j] = vadd(h[j], s[(tid ^ (NT / 2)) + (j ^ 1) * NT]);
+#pragma unroll
+      for (int c = 0; c + 1 < LA; ++c)  // both bits in j: registers
+#pragma unroll
+        for (int j = 0; j < APT; ++j)
+          if (((j >> c) ^ (j >> (c + 1))) & 1) h[j] = vadd(h[j], x[j ^ (3 << c)]);
+    }
+#pragma unroll
+    for (int j = 0; j < APT; ++j) h[j] = vfma(dj[j], x[j], vmul(hxy, h[j]));
+    if (p.hc_kind == KG_HC_SX_SITE && p.hc_site < LT + LA) {
+#pragma unroll
+      for (int j = 0; j < APT; ++j) h[j] = vfma(cx, s[li(j) ^ (1 << p.hc_site)], h[j]);
+    }
+  }
+
+  // MULTI: partner blocks of W_k from the other tiles, through this thread's own slots of the ring.
+  // Slot 0: the bond between the tile's top bit and the lowest bit above it (half of the amplitudes);
+  // then the bonds above the tile that are antiparallel for the whole tile; then an Sx control above it.
+  __device__ __forceinline__ bool top_active(int j) const {
+    constexpr int b = LT + LA - 1;
+    return ((unsigned)(li(j) >> b) ^ (unsigned)(base >> (b + 1))) & 1u;
+  }
+  __device__ __forceinline__ void cross_issue(const V* w) {
+    constexpr int b0 = LT + LA - 1;
+    int s = 1;
+#pragma unroll
+    for (int j = 0; j < APT; ++j)
+      if (top_active(j)) cross_copy(ring + li(j), w + ((base + li(j)) ^ ((size_t)3 << b0)));
+    for (unsigned act = bonds_hi; act; act &= act - 1, ++s) {
+      const V* q = w + (base ^ ((size_t)3 << (__ffs(act) - 1)));
+#pragma unroll
+      for (int j = 0; j < APT; ++j) cross_copy(ring + s * T + li(j), q + li(j));
+    }
+    if (p.hc_kind == KG_HC_SX_SITE && p.hc_site > b0) {
+      const V* q = w + (base ^ ((size_t)1 << p.hc_site));
+#pragma unroll
+      for (int j = 0; j < APT; ++j) cross_copy(ring + s * T + li(j), q + li(j));
+    }
+    cp_async_commit();
+  }
+  __device__ __forceinline__ static void cross_copy(V* dst, const V* src) {
+    static_assert(!MULTI || sizeof(V) == 16, "the ring moves 16-byte amplitudes");
+    cp_async16(dst, src);
+  }
+  __device__ __forceinline__ void cross_add(V (&h)[APT]) {
+    constexpr int b0 = LT + LA - 1;
+    cp_async_wait<0>();
+    V x[APT];
+#pragma unroll
+    for (int j = 0; j < APT; ++j) x[j] = top_active(j) ? ring[li(j)] : vmake<V>(0, 0);
+    int s = 1;
+    for (unsigned act = bonds_hi; act; act &= act - 1, ++s)
+#pragma unroll
+      for (int j = 0; j < APT; ++j) x[j] = vadd(x[j], ring[s * T + li(j)]);
+#pragma unroll
+    for (int j = 0; j < APT; ++j) h[j] = vfma(hxy, x[j], h[j]);
+    if (p.hc_kind == KG_HC_SX_SITE && p.hc_site > b0)
+#pragma unroll
+      for (int j = 0; j < APT; ++j) h[j] = vfma(cx, ring[s * T + li(j)], h[j]);
+  }
+
+  __device__ __forceinline__ V* sbasis(int k) const { return sw + k * T; }  // SB: v_k
+  __device__ __forceinline__ V* gbasis(int k) const { return (V*)p.basis + (size_t)(k - 1) * D + base; }
+  __device__ __forceinline__ V* gw(int k) const { return (V*)p.wbuf + (size_t)(k & 1) * D; }
+
+  __device__ __forceinline__ void fail_nonfinite() {
+    if (tid == 0) {
+      atomicCAS(p.ctrl + kCtrlStatus, 0, (int)KG_ERR_NONFINITE);
+      atomicExch(p.ctrl + kCtrlAbort, 1);
+    }
+  }
+
+  // Lanczos basis of the slice from wo (||wo|| = nrm): v_k in the basis, alpha_k and b_{k+1} in shared
+  // memory, the number of vectors, whether the basis ended early, b_m.  false: aborted.
+  __device__ __forceinline__ bool lanczos(int& meff, bool& broke, R& beta_m) {
+    const int m = p.m;
+    V vp[APT], v[APT], w[APT];
+    V* s = sw;  // v_k
+#pragma unroll
+    for (int j = 0; j < APT; ++j) {
+      vp[j] = vmake<V>(0, 0);
+      v[j] = vmul(inv, wo[j]);
+      s[li(j)] = v[j];
+    }
+    R alpha = 0, bk = 0, ib = 0, amax = 0, bmax = 0;
+    const R tol = (R)p.bd_tol;
+    meff = (sround(nrm) > 0) ? m : 0;
+    broke = false;
+    beta_m = 0;
+    for (int k = 0; k < meff; ++k) {
+      const bool last = (k == m - 1);
+      sync();  // v_k is in shared memory
+      stencil(s, v, w);
+      R acc[3] = {0, 0, 0};
+#pragma unroll
+      for (int j = 0; j < APT; ++j) {
+        w[j] = vfma(-bk, vp[j], w[j]);
+        acc[0] = fma(v[j].x, w[j].x, fma(v[j].y, w[j].y, acc[0]));
+        acc[1] = fma(w[j].x, w[j].x, fma(w[j].y, w[j].y, acc[1]));
+        acc[2] = fma(v[j].x, v[j].x, fma(v[j].y, v[j].y, acc[2]));
+      }
+      post(acc);
+      sync();
+      S o[kTileSums];
+      if (!collect(o)) return false;
+      if (!step_scalars(k, last, o, v, w, tol, amax, bmax, alpha, bk, ib, broke)) return false;
+      if (last) beta_m = bk;
+      if (last || broke) {
+        meff = k + 1;
+        break;
+      }
+      s = SB ? sw + (k + 1) * T : sw + ((k + 1) & 1) * T;
+#pragma unroll
+      for (int j = 0; j < APT; ++j) {
+        const V vn = vmul(ib, vfma(-alpha, v[j], w[j]));
+        vp[j] = v[j];
+        v[j] = vn;
+        s[li(j)] = vn;
+        if constexpr (!SB) stv(gbasis(k + 1) + li(j), vn);
+      }
+    }
+    return true;
+  }
+  // The same by the raw vectors (several CTAs, or 16 amplitudes a thread, where the other arrangement's
+  // third vector does not fit the registers); src is W_0 in global memory.
+  __device__ __forceinline__ bool lanczos_raw(const V* src, int& meff, bool& broke, R& beta_m) {
+    const int m = p.m;
+    V vp[APT], hp[APT];
+#pragma unroll
+    for (int j = 0; j < APT; ++j) vp[j] = hp[j] = vmake<V>(0, 0);
+    R ap = 0, ib = inv, bk = 0, amax = 0, bmax = 0;
+    const R tol = (R)p.bd_tol;
+    meff = (sround(nrm) > 0) ? m : 0;
+    broke = false;
+    beta_m = 0;
+    for (int k = 0; k < meff; ++k) {
+      const bool last = (k == m - 1);
+      V h[APT];
+      stencil(sw + (k & 1) * T, wo, h);
+      if (k > 0) {  // alpha_{k-1}, b_k from the sums of step k - 1
+        S o[kTileSums];
+        if (!collect(o)) return false;
+        if constexpr (MULTI) cross_issue(gw(k));
+        if (!step_scalars(k - 1, false, o, vp, wo, tol, amax, bmax, ap, bk, ib, broke)) return false;
+        if (broke) {
+          meff = k;
+          if constexpr (MULTI) cp_async_wait<0>();
+          break;
+        }
+      } else if constexpr (MULTI) {
+        cross_issue(src);
+      }
+      if constexpr (MULTI) cross_add(h);
+      R acc[3] = {0, 0, 0};
+      V* sn = sw + ((k + 1) & 1) * T;
+      V* vslot = (k > 0) ? gbasis(k) : nullptr;
+#pragma unroll
+      for (int j = 0; j < APT; ++j) {
+        const V v = vmul(ib, vfma(-ap, vp[j], wo[j]));
+        const V hv = vmul(ib, vfma(-ap, hp[j], h[j]));
+        const V w = vfma(-bk, vp[j], hv);  // b_0 counts as 0: v_{-1} = 0
+        acc[0] = fma(v.x, w.x, fma(v.y, w.y, acc[0]));
+        acc[1] = fma(w.x, w.x, fma(w.y, w.y, acc[1]));
+        acc[2] = fma(v.x, v.x, fma(v.y, v.y, acc[2]));
+        vp[j] = v;
+        hp[j] = hv;
+        wo[j] = w;
+        if (!last) {
+          sn[li(j)] = w;
+          if constexpr (MULTI) stv(gw(k + 1) + base + li(j), w);
+        }
+        if (k > 0) stv(vslot + li(j), v);
+      }
+      post(acc);
+      sync();
+    }
+    if (meff > 0 && !broke) {  // the last step's sums: alpha_{m-1}, b_m of the error indicator
+      S o[kTileSums];
+      if (!collect(o)) return false;
+      bool unused = false;
+      if (!step_scalars(m - 1, true, o, vp, wo, tol, amax, bmax, ap, beta_m, ib, unused)) return false;
+    }
+    return true;
+  }
+
+  // One slice, x (own amplitudes in wo) -> exp(-+i dt H_j) x in wo, written to dst.  back: the co-state
+  // sweep, whose sums carry Im <dst|Hc|other>.  lob 1: the interior quadrature
+  // states of a forward slice go to tint; 2: the sums carry the overlap with the interior states of
+  // a backward slice.  On return the new vector's sums are posted (collect gives ||dst||^2 and the
+  // overlaps); false: aborted (in every thread alike).
+  __device__ __forceinline__ bool slice(bool back, V* dst, const V* src, const V* other, int lob, V* tint) {
+    int meff;
+    bool broke;
+    R beta_m;
+    if constexpr (RAW) {
+      if (!lanczos_raw(src, meff, broke, beta_m)) return false;
+    } else {
+      if (!lanczos(meff, broke, beta_m)) return false;
+    }
+    mark(0);
+    // ---- the other vector of the overlap and the newest basis vectors are fetched while the small
+    // exponential runs
+    V q[APT];
+    if (back) load_partner(other, q);
+    if (lob) sync();  // thread 0 wrote alpha and b; its warp alone reads them unless lob
+    else __syncwarp();
+    coefficients(back, meff, broke, beta_m, lob);
+    sync();
+    mark(4);
+    // ---- recombination
+    R pgi = 0;
+#pragma unroll 1
+    for (int a = lob ? 2 : 0; a >= 0; --a) {
+      recombine(a, meff, src, wo);
+      if (a == 0) break;
+      V* t = tint + (size_t)(a - 1) * D;
+      if (lob == 1) {
+#pragma unroll
+        for (int j = 0; j < APT; ++j)
+          if (li(j) < D1) stv(t + base + li(j), wo[j]);
+      } else {
+        V z[APT];
+        load_partner(t, z);
+        pgi += hc_overlap(wo, z);
+      }
+    }
+    publish(dst);
+    R pn = 0;
+#pragma unroll
+    for (int j = 0; j < APT; ++j) pn = fma(wo[j].x, wo[j].x, fma(wo[j].y, wo[j].y, pn));
+    const R vals[3] = {pn, back ? hc_overlap(wo, q) : (R)0, pgi};
+    post(vals);
+    sync();
+    mark(5);
+    return true;
+  }
+
+  // wo is the next slice's initial vector: into the trajectory (and, RAW, W_0 in shared memory).
+  __device__ __forceinline__ void publish(V* dst) {
+#pragma unroll
+    for (int j = 0; j < APT; ++j) {
+      if constexpr (RAW) sw[li(j)] = wo[j];
+      if (li(j) < D1) stv(dst + base + li(j), wo[j]);
+    }
+  }
+
+  // The amplitudes of vector v that Hc couples to the own ones (Sx: the flipped site; Sz: the same).
+  __device__ __forceinline__ void load_partner(const V* v, V (&q)[APT]) const {
+    const size_t flip = (p.hc_kind == KG_HC_SX_SITE) ? (size_t)1 << p.hc_site : 0;
+#pragma unroll
+    for (int j = 0; j < APT; ++j) q[j] = (li(j) < D1) ? ldv(v + ((base + li(j)) ^ flip)) : vmake<V>(0, 0);
+  }
+
+  // This thread's share of Im <y|Hc|q> (q already at the partner index for an Sx control).
+  __device__ __forceinline__ R hc_overlap(const V (&y)[APT], const V (&q)[APT]) {
+    const bool sx = (p.hc_kind == KG_HC_SX_SITE);
+    const R amp = (R)p.hc_amp;
+    R g = 0;
+#pragma unroll
+    for (int j = 0; j < APT; ++j) {
+      const R w = sx ? (R)0.5 : zdiag(j);
+      g = fma(w, fma(y[j].x, q[j].y, -(y[j].y * q[j].x)), g);
+    }
+    return amp * g;
+  }
+
+  // Scalars after step k from its sums o = (<v|W>, ||W||^2, ||v||^2): alpha_k, b_{k+1}, 1/b_{k+1};
+  // near an invariant subspace b_{k+1}^2 = ||W_{k+1} - alpha_k v_k||^2 formed explicitly.  broke:
+  // b_{k+1} vanishes (Alg. "Lanczos", b_j > 0 with a tolerance).  false: not finite, or aborted.
+  __device__ __forceinline__ bool step_scalars(int k, bool last, const S (&o)[kTileSums], const V (&v)[APT],
+                                               const V (&w)[APT], R tol,
+                                               R& amax, R& bmax, R& alpha, R& beta, R& inv_b, bool& broke) {
+    alpha = sround(o[0]);
+    S b2 = sb2(o[0], o[1], o[2]);
+    sroot(b2, beta, inv_b);
+    const bool usual = !scancels(b2, o[1]) && sfinite(o[0]) && sfinite(o[1]) && beta > tol * fmax((R)1, fmax(amax, fabs(alpha)) + bmax);
+    if (!usual) {
+      if (!sfinite(o[0]) || !sfinite(o[1])) {
+        fail_nonfinite();
+        return false;
+      }
+      if (!last && scancels(b2, o[1])) {
+        R e[3] = {0, 0, 0};
+#pragma unroll
+        for (int j = 0; j < APT; ++j) {
+          const V d = vfma(-alpha, v[j], w[j]);
+          e[0] = fma(d.x, d.x, fma(d.y, d.y, e[0]));
+        }
+        post(e);
+        if constexpr (!MULTI) sync();
+        S oe[kTileSums];
+        if (!collect(oe)) return false;
+        b2 = oe[0];
+        sroot(b2, beta, inv_b);
+      }
+      if (!last) broke = beta <= tol * fmax((R)1, fmax(amax, fabs(alpha)) + bmax);
+    }
+    amax = fmax(amax, fabs(alpha));
+    bmax = fmax(bmax, beta);
+    if (tid == 0) {
+      if constexpr (F32) {
+        sm.al_ff[k] = make_float2(o[0].hi, o[0].lo);
+        sm.b2_ff[k] = make_float2(b2.hi, b2.lo);
+      } else {
+        sm.al[k] = o[0];
+        sm.be[k + 1] = beta;
+      }
+    }
+    return true;
+  }
+
+  // Small exponentials: c = exp(-+i t T) e_1 for the slice end (0) and, with lob, the interior
+  // quadrature nodes (1, 2), one warp each; times ||x|| for the normalised basis vectors (slot 0 is x).
+  __device__ __forceinline__ void coefficients(bool back, int meff, bool broke, R beta_m, int lob) {
+    const int lane = tid & 31, warp = tid >> 5;
+    const int nc = lob ? 3 : 1;
+    for (int a = warp; a < nc; a += NW) {
+      R cr = 0, ci = 0;
+      float tnorm = 0.f;
+      if constexpr (F32) {
+        const float2 a2 = (lane < meff) ? sm.al_ff[lane] : make_float2(0.f, 0.f);
+        const float2 b2 = (lane >= 1 && lane < meff) ? sm.b2_ff[lane - 1] : make_float2(0.f, 0.f);
+        FF fr{0.f, 0.f}, fi{0.f, 0.f};
+        // forward exp(-i s T); backward exp(+i (dt - s) T), where dt - s_a = s_b
+        const float2 t2 = sm.tau_ff[back && a > 0 ? 3 - a : a];
+        const FF t = back ? FF{-t2.x, -t2.y} : FF{t2.x, t2.y};
+        if (meff > 0) tridiag_expv_e1_fff(FF{a2.x, a2.y}, ff_sqrt(FF{b2.x, b2.y}), meff, t, 1e-13f, fact, fr, fi, tnorm);
+        const FF f = (lane == 0) ? FF{1.f, 0.f} : nrm;
+        cr = sround(ff_mul(fr, f));
+        ci = sround(ff_mul(fi, f));
+        if (lane < meff) {
+          sm.coef_re_f[a][lane] = cr;
+          sm.coef_im_f[a][lane] = ci;
+        }
+      } else {
+        // FP32 copies for the exponential's norm bound
+        if (lane < meff) {
+          sm.coef_re_f[a][lane] = (float)sm.al[lane];
+          sm.coef_im_f[a][lane] = (lane >= 1) ? (float)sm.be[lane] : 0.f;
+        }
+        __syncwarp();
+        double dr = 0.0, di = 0.0, t = p.dt;
+        if (a > 0) t = 0.5 * p.dt * (1.0 + ((a == 1) != back ? -0.4472135954999579 : 0.4472135954999579));  // 1/sqrt(5)
+        if (back) t = -t;
+        if (meff > 0)
+          tridiag_expv_e1(sm.al, sm.be, sm.coef_re_f[a], sm.coef_im_f[a], meff, t, (float)t, 1e-18, dr, di, tnorm);
+        const double f = (lane == 0) ? 1.0 : nrm;
+        cr = dr * f;
+        ci = di * f;
+        if (lane < meff) {
+          sm.coef_re[a][lane] = cr;
+          sm.coef_im[a][lane] = ci;
+        }
+      }
+      if (a == 0 && lane == meff - 1) {
+        // a-posteriori indicator ||x|| b_m |c_{m-1}|; where the Taylor series stopped before index
+        // m - 1, ||x|| b_m ||tau T||^(m-1)/(m-1)! bounds it
+        const float n0 = (float)sround(nrm);
+        const float re = (float)cr, im = (float)ci;
+        float cm = sqrtf(re * re + im * im);
+        if (lane == 0) cm *= n0;
+        if (cm == 0.f) {
+          cm = n0;
+          for (int i = 1; i < meff; ++i) cm *= tnorm * kInvFF[i].x;
+        }
+        if (broke) sm.breakdowns += 1;
+        else sm.err_max = fmaxf(sm.err_max, (float)beta_m * cm);
+      }
+    }
+  }
+
+  // y = sum_k coef[a]_k (basis vector k), own amplitudes; the small terms (large k) first, so that the
+  // sum is rounded at full size only where the largest term, psi's, comes last.
+  __device__ __forceinline__ void recombine(int a, int meff, const V* src, V (&y)[APT]) {
+    const R* cre = F32 ? (const R*)sm.coef_re_f[a] : (const R*)sm.coef_re[a];
+    const R* cim = F32 ? (const R*)sm.coef_im_f[a] : (const R*)sm.coef_im[a];
+#pragma unroll
+    for (int j = 0; j < APT; ++j) y[j] = vmake<V>(0, 0);
+    if constexpr (SB) {
+      V x[APT];
+#pragma unroll
+      for (int j = 0; j < APT; ++j) x[j] = (li(j) < D1) ? ldv(src + base + li(j)) : vmake<V>(0, 0);
+      for (int k = meff - 1; k >= 1; --k) {
+        const R c0 = cre[k], c1 = cim[k];
+        const V* q = sbasis(k);
+#pragma unroll
+        for (int j = 0; j < APT; ++j) y[j] = vcfma(c0, c1, q[li(j)], y[j]);
+      }
+      if (meff > 0) {
+        const R c0 = cre[0], c1 = cim[0];
+#pragma unroll
+        for (int j = 0; j < APT; ++j) y[j] = vcfma(c0, c1, x[j], y[j]);
+      }
+    } else {
+      // several basis vectors' loads in flight
+      constexpr int KB = (sizeof(V) * APT > 64) ? 2 : 4;
+      for (int k0 = meff - 1; k0 >= 0; k0 -= KB) {
+        V q[KB][APT];
+#pragma unroll
+        for (int u = 0; u < KB; ++u) {
+          const int k = k0 - u;
+          const V* s = (k == 0) ? src + base : gbasis(k);
+#pragma unroll
+          for (int j = 0; j < APT; ++j) q[u][j] = (k >= 0) ? ldv(s + li(j)) : vmake<V>(0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < KB; ++u) {
+          const int k = k0 - u;
+          const R c0 = (k >= 0) ? cre[k] : (R)0, c1 = (k >= 0) ? cim[k] : (R)0;
+#pragma unroll
+          for (int j = 0; j < APT; ++j) y[j] = vcfma(c0, c1, q[u][j], y[j]);
+        }
+      }
+    }
+  }
+
+  // The new vector's sums: its norm (for the next slice) and the overlaps.
+  __device__ __forceinline__ bool finish(S& g, S& gi) {
+    S o[kTileSums];
+    if (!collect(o)) return false;
+    if (!sfinite(o[0])) {
+      fail_nonfinite();
+      return false;
+    }
+    snorm(o[0], nrm, inv);
+    g = o[1];
+    gi = o[2];
+    return true;
+  }
+
+  __device__ __forceinline__ V* fwd_slot(int j) const {  // storage of psi_j (see kg_abi.cu's layout)
+    V* traj = (V*)p.traj;
+    const int C = p.ckpt;
+    if (C == 0) return traj + (size_t)j * D;
+    if (j % C == 0) return traj + (size_t)(j / C) * D;
+    if (j == p.N) return traj + (size_t)(p.N / C + 1) * D;
+    return (V*)p.seg + (size_t)(C - 1 + (j & 1)) * D;
+  }
+
+  // The next slice starts from a stored vector.
+  __device__ __forceinline__ void load_state(const V* v) {
+#pragma unroll
+    for (int j = 0; j < APT; ++j) {
+      wo[j] = (li(j) < D1) ? ldv(v + base + li(j)) : vmake<V>(0, 0);
+      if constexpr (RAW) sw[li(j)] = wo[j];
+    }
+  }
+
+  __device__ __forceinline__ bool run() {
+    init();
+    S g, gi;
+    // ---- psi_0
+    {
+      double acc[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int j = 0; j < APT; ++j) {
+        wo[j] = vmake<V>(0, 0);
+        if (li(j) < D1) {
+          const double2 a = reinterpret_cast<const double2*>(p.psi0)[base + li(j)];
+          wo[j] = vmake<V>((R)a.x, (R)a.y);
+          acc[0] += (double)wo[j].x * wo[j].x + (double)wo[j].y * wo[j].y;
+        }
+      }
+      publish(fwd_slot(0));
+      double o[3];
+      if (!sum_fp64(acc, o)) return false;
+      if (!isfinite(o[0])) {
+        fail_nonfinite();
+        return false;
+      }
+      const double n = sqrt(fmax(o[0], 0.0));
+      nrm = sfrom(n, S());
+      inv = (n > 0.0) ? (R)(1.0 / n) : (R)0;
+    }
+    const bool lead = (rank == 0 && tid == 0);
+    if (lead) p.nrm[0] = spack(nrm);
+    const bool exact = (p.grad_mode == KG_GRAD_EXACT);
+    mark(6);
+    // The slices in order: the forward sweep, then segment by segment (one segment without
+    // checkpoints) the recomputation of psi_{a+1..b-1} and the co-state sweep.  One loop, one copy of
+    // the slice's code: three copies miss the instruction cache at every change of direction.
+    V* chi[2] = {(V*)p.chi, (V*)p.chi + D};
+    const int C = p.ckpt;
+    enum { kForward, kRecompute, kBackward };
+    int kind = kForward, j = 1, a = 0, b = p.N, cur = 0;
+    S nchi = nrm;
+    R ichi = inv;
+    for (;;) {
+      const V* src;
+      const V* other = nullptr;
+      V* dst;
+      if (kind == kForward) {
+        src = fwd_slot(j - 1);
+        dst = fwd_slot(j);
+      } else if (kind == kRecompute) {
+        src = seg_slot(a, j - 1);
+        dst = (V*)p.seg + (size_t)(j - a - 1) * D;
+      } else {
+        src = chi[cur];
+        dst = chi[cur ^ 1];
+        other = (C == 0) ? (V*)p.traj + (size_t)(j - 1) * D : seg_slot(a, j - 1);
+      }
+      set_control(p.u[j - 1]);
+      const bool back = kind == kBackward;
+      const int lob = !exact ? 0 : back ? 2 : 1;
+      if (!slice(back, dst, src, other, lob, exact ? (V*)p.tint + (size_t)2 * (j - 1) * D : nullptr))
+        return false;
+      if (!finish(g, gi)) return false;
+      // ---- what follows the slice
+      if (kind == kForward) {
+        if (lead) p.nrm[j] = spack(nrm);
+        if (j < p.N) {
+          ++j;
+          continue;
+        }
+        if (!turn(lead, chi[0])) return false;
+        if (p.grad_mode == KG_GRAD_NONE) break;
+        mark(6);
+        a = (C > 0) ? (p.N - 1) / C * C : 0;
+      } else if (kind == kRecompute) {
+        if (j + 1 < b) {
+          ++j;
+          continue;
+        }
+        sync();  // every warp is done with W_0 in shared memory
+        load_state(chi[cur]);
+        nrm = nchi;
+        inv = ichi;
+        sync();
+        kind = kBackward;
+        j = b;
+        continue;
+      } else {
+        if (lead) {
+          p.G[j - 1] = spack(g);
+          if (exact) p.Gi[j - 1] = spack(gi);  // both interior nodes of slice j
+        }
+        cur ^= 1;
+        if (j - 1 > a) {
+          --j;
+          continue;
+        }
+        if (a == 0) break;
+        b = a;
+        a -= C;
+      }
+      // ---- the next segment (a, b]
+      kind = kBackward;
+      j = b;
+      if (C > 0 && b - a > 1) {
+        nchi = nrm;
+        ichi = inv;
+        sync();
+        load_state(seg_slot(a, a));
+        nrm = sunpack(__ldcg(p.nrm + a), S());
+        inv = sinv(nrm);
+        sync();
+        kind = kRecompute;
+        j = a + 1;
+      }
+    }
+    // ---- outputs (rank 0)
+    if (rank == 0) {
+      sync();
+      if (p.grad_mode != KG_GRAD_NONE) {
+        const double f = 2.0 * p.dt;
+        for (int j = tid; j < p.N; j += NT) {
+          const double gl = f * sdouble(sunpack(__ldcg(p.G + j), S())), gr = f * sdouble(sunpack(__ldcg(p.G + j + 1), S()));
+          if (exact)  // Gauss-Lobatto weights 1/12, 5/12, 5/12, 1/12
+            p.grad[j] = (gl + gr) / 12.0 + 5.0 * (f * sdouble(sunpack(__ldcg(p.Gi + j), S()))) / 12.0;
+          else
+            p.grad[j] = (p.grad_mode == KG_GRAD_ZEROTH) ? gr : 0.5 * (gl + gr);
+        }
+      }
+      if (tid == 0) {
+        p.scal[kScErrMax] = (double)sm.err_max;
+        p.scal[kScBreakdowns] = (double)sm.breakdowns;
+      }
+    }
+    return true;
+  }
+
+  // psi_j of the segment that starts at checkpoint a.
+  __device__ __forceinline__ V* seg_slot(int a, int j) const {
+    return (j == a) ? (V*)p.traj + (size_t)(a / p.ckpt) * D : (V*)p.seg + (size_t)(j - 1 - a) * D;
+  }
+
+  // The end of the forward sweep: beta = <f|psi_N> (FP64) and F; with a gradient chi_N = beta f (into
+  // wo and chi), its norm, and G_N = 2 dt Im <chi_N|Hc|psi_N>.
+  __device__ __forceinline__ bool turn(bool lead, V* chi) {
+    const double2* f = reinterpret_cast<const double2*>(p.target) + base;
+    double acc[3] = {0.0, 0.0, 0.0}, o[3];
+#pragma unroll
+    for (int j = 0; j < APT; ++j) {
+      if (li(j) < D1) {
+        const double2 t = f[li(j)];
+        const double yr = (double)wo[j].x, yi = (double)wo[j].y;
+        acc[0] += t.x * yr + t.y * yi;
+        acc[1] += t.x * yi - t.y * yr;
+      }
+    }
+    if (!sum_fp64(acc, o)) return false;
+    const double br = o[0], bi = o[1];
+    if (lead) {
+      p.scal[kScBetaRe] = br;
+      p.scal[kScBetaIm] = bi;
+      p.scal[kScNormFinal] = sdouble(nrm);
+      p.fid[0] = br * br + bi * bi;
+    }
+    if (p.grad_mode == KG_GRAD_NONE) return true;
+    V z[APT];
+    load_partner(fwd_slot(p.N), z);
+    acc[0] = acc[1] = 0.0;
+#pragma unroll
+    for (int j = 0; j < APT; ++j) {
+      wo[j] = vmake<V>(0, 0);
+      if (li(j) < D1) {
+        const double2 t = f[li(j)];
+        wo[j] = vmake<V>((R)(br * t.x - bi * t.y), (R)(br * t.y + bi * t.x));
+        acc[0] += (double)wo[j].x * wo[j].x + (double)wo[j].y * wo[j].y;
+      }
+    }
+    publish(chi);
+    const bool sx = (p.hc_kind == KG_HC_SX_SITE);
+#pragma unroll
+    for (int j = 0; j < APT; ++j) {
+      const R w = (R)p.hc_amp * (sx ? (R)0.5 : zdiag(j));
+      acc[1] += (double)(w * (wo[j].x * z[j].y - wo[j].y * z[j].x));
+    }
+    if (!sum_fp64(acc, o)) return false;
+    const double n = sqrt(fmax(o[0], 0.0));
+    nrm = sfrom(n, S());
+    inv = (n > 0.0) ? (R)(1.0 / n) : (R)0;
+    if (lead) p.G[p.N] = spack(sfrom(o[1], S()));
+    return true;
+  }
+};
+
+// The control warp of a CTA that is one of several (threads NT .. NT + 31): for every reduction it takes
+// the workers' warp partials, makes the CTA's stores visible and posts the CTA's sums with the
+// reduction's number, then reads every CTA's message (lane l those of CTAs l, l + 32, ...) until it
+// carries that number, adds them up and answers the workers.  Two sets of slots, by the number's
+// parity: a CTA posts reduction n + 2 only after every CTA has posted n + 1, so has read n.
+template <int NT>
+__device__ __forceinline__ void tile_control(const EvalParams& p, TileSmem& sm, int rank, int size) {
+  constexpr int NW = NT / 32;
+  const int lane = threadIdx.x & 31;
+  unsigned long long seq = 0;
+  for (;;) {
+    nbar_sync(kTileBarPost, NT + 32);
+    const int cmd = sm.cmd;
+    if ((cmd & 3) == kTileCmdExit) return;
+    const int par = (cmd >> 2) & 1;
+    ++seq;
+    ulonglong2* slots = reinterpret_cast<ulonglong2*>(p.red) + (size_t)(seq & 1) * size * kNRed;
+    double s = sm.red_d[par][(lane >> 2) & (NW - 1)][lane & 3];
+#pragma unroll
+    for (int o = 1; o < NW; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, 4 * o);
+    __threadfence();  // the workers' stores, ordered before this warp by the named barrier
+    const bool skip = rank == 0 && ((p.debug_fault == 1 && seq == 1) || (p.debug_fault == 2 && seq == 2));
+    if (lane < kTileSums && !skip) st_msg(slots + rank * kNRed + lane, (unsigned long long)__double_as_longlong(s), seq);
+    double t[kTileSums] = {0.0, 0.0, 0.0};
+    bool ok = true;
+    unsigned long long t0 = 0;
+    unsigned polls = 0;
+    for (int r = lane; r < size && ok; r += 32) {
+      ulonglong2 q[kTileSums];
+      for (;;) {
+        bool all = true;
+#pragma unroll
+        for (int i = 0; i < kTileSums; ++i) {
+          q[i] = ld_msg(slots + r * kNRed + i);
+          all = all && q[i].y == seq;
+        }
+        if (all) break;
+        if ((++polls & 31u) == 0u) {
+          if (ld_volatile_i32(p.ctrl + kCtrlAbort)) { ok = false; break; }
+          const unsigned long long now = globaltimer_ns();
+          if (t0 == 0) {
+            t0 = now;
+          } else if ((long long)(now - t0) > p.wait_limit_ns) {
+            atomicCAS(p.ctrl + kCtrlStatus, 0, (int)KG_ERR_TIMEOUT);
+            atomicExch(p.ctrl + kCtrlAbort, 1);
+            ok = false;
+            break;
+          }
+        }
+      }
+      if (ok)
+#pragma unroll
+        for (int i = 0; i < kTileSums; ++i) t[i] += __longlong_as_double((long long)q[i].x);
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    __threadfence();  // what the workers read after the barrier was stored before the messages
+    // transposed butterfly over the lanes, as in Tile::post
+    const bool o1 = lane & 1, o2 = lane & 2;
+    const double s0 = (o1 ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, o1 ? t[0] : t[1], 1);
+    const double s1 = (o1 ? 0.0 : t[2]) + __shfl_xor_sync(0xffffffffu, o1 ? t[2] : 0.0, 1);
+    double x = (o2 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, o2 ? s0 : s1, 2);
+#pragma unroll
+    for (int o = 4; o <= 16; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (lane < kTileSums) sm.tot[par][lane] = x;
+    if (lane == 0) sm.ok = ok ? 1 : 0;
+    __syncwarp();
+    nbar_arrive(kTileBarGroup, NT + 32);
+  }
+}
+
+template <class V, int NT, int APT, bool SB, bool MULTI>
+__device__ __forceinline__ void tile_cta(const EvalParams& p, TileSmem& sm, V* sw, int rank) {
+  using TileT = Tile<V, NT, APT, SB, MULTI>;
+  const long long t0 = clock64();
+  if (threadIdx.x == 0) {
+    sm.err_max = 0.f;
+    sm.breakdowns = 0;
+    sm.ok = 1;
+    for (int i = 0; i < 8; ++i) sm.prof_acc[i] = 0;
+    sm.prof_last = t0;
+  }
+  __syncthreads();
+  if (MULTI && threadIdx.x >= NT) {
+    tile_control<NT>(p, sm, rank, (int)gridDim.x);
+    return;
+  }
+  TileT t{p, sm, sw, sw + 2 * TileT::T};
+  t.tid = (int)threadIdx.x;
+  t.rank = rank;
+  t.D = (size_t)1 << p.L;
+  t.base = (size_t)rank * TileT::T;
+  t.D1 = (int)min((size_t)TileT::T, t.D);
+  t.par = 0;
+  t.run();
+  if constexpr (MULTI) {
+    if (threadIdx.x == 0) sm.cmd = kTileCmdExit;
+    nbar_arrive(kTileBarPost, NT + 32);
+  }
+  if (p.prof != nullptr && rank == 0 && threadIdx.x == 0) {
+    for (int i = 0; i < 7; ++i) p.prof[i] = sm.prof_acc[i];
+    p.prof[7] = clock64() - t0;
+  }
+}
+
+template <class V, int NT, int APT, bool SB, bool MULTI>
+__global__ void __launch_bounds__(MULTI ? NT + 32 : NT, 1) kg_tile_kernel(const __grid_constant__ EvalParams p) {
+  extern __shared__ __align__(16) unsigned char tile_dyn[];
+  __shared__ TileSmem sm;
+  tile_cta<V, NT, APT, SB, MULTI>(p, sm, reinterpret_cast<V*>(tile_dyn), MULTI ? (int)blockIdx.x : 0);
+}
+
+// Many problems of one chain length, one CTA each.
+template <class V, int NT, int APT, bool SB>
+__global__ void __launch_bounds__(NT, 1) kg_tile_list_kernel(const EvalParams* list) {
+  extern __shared__ __align__(16) unsigned char tile_dyn[];
+  __shared__ TileSmem sm;
+  __shared__ EvalParams p;
+  if (threadIdx.x == 0) p = list[blockIdx.x];
+  __syncthreads();
+  tile_cta<V, NT, APT, SB, false>(p, sm, reinterpret_cast<V*>(tile_dyn), 0);
+}
+
+// ---------------------------------------------------------------- launch selection
+struct TileKernel {
+  const void* fn = nullptr;    // one problem (EvalParams by value)
+  const void* list = nullptr;  // complex64: a list of problems
+  int threads = 0, tile_bits = 0;
+  size_t smem = 0;
+};
+
+// Basis in shared memory up to this size.
+constexpr size_t kTileSmemBasis = 100 * 1024;
+
+template <class V, int NT, int APT, bool SB>
+TileKernel tile_choice(size_t smem) {
+  TileKernel k{reinterpret_cast<const void*>(&kg_tile_kernel<V, NT, APT, SB, false>), nullptr, NT,
+               __builtin_ctz(NT * APT), smem};
+  if constexpr (sizeof(V) == 8) k.list = reinterpret_cast<const void*>(&kg_tile_list_kernel<V, NT, APT, SB>);
+  return k;
+}
+template <class V, int NT, int APT>
+TileKernel tile_single(int m) {
+  constexpr size_t vec = (size_t)NT * APT * sizeof(V);
+  if constexpr (APT < 16)
+    if (m * vec <= kTileSmemBasis) return tile_choice<V, NT, APT, true>(m * vec);
+  return tile_choice<V, NT, APT, false>(2 * vec);
+}
+
+// Threads x amplitudes by chain length.  More threads shorten every thread's chain of shared-memory
+// loads, fewer make the block's sums cheaper; measured (us per slice, m = 16, complex64):
+//   L = 7: 64 x 2 12.7, 32 x 4 12.3;  8: 128 x 2 14.1, 32 x 8 15.3, 64 x 4 15.7;  9: 256 x 2 17.3, 128 x 4
+//   17.7, 64 x 8 18.5;  10: 128 x 8 22.2, 256 x 4 22.6;  11: 256 x 8 29.7, 512 x 4 34.8;
+//   12: 256 x 16 (raw vectors) 47.7, 512 x 8 61.0 (128 registers).
+// The kernels that ran these chains before took 100 (L = 5) to 148 us (L = 11) and 77 us (L = 12).
+// complex128 is bound by the FP64 units, one quarter in each quarter of the SM: one warp per quarter
+// as soon as there are amplitudes for it (L = 8: 128 x 2 76, 64 x 4 113, 256 x 1 91; 9: 128 x 4 125,
+// 256 x 2 140).  Before: 351 us (L = 5, m = 20) to 620 us (L = 10); now 54 to 280.
+TileKernel pick_tile(int prec, int L, int m) {
+  if (prec == KG_PREC_C64_F64REC) {
+    if (L <= 5) return tile_single<float2, 32, 1>(m);
+    if (L == 6) return tile_single<float2, 32, 2>(m);
+    if (L == 7) return tile_single<float2, 64, 2>(m);
+    if (L == 8) return tile_single<float2, 128, 2>(m);
+    if (L == 9) return tile_single<float2, 256, 2>(m);
+    if (L == 10) return tile_single<float2, 128, 8>(m);
+    if (L == 11) return tile_single<float2, 256, 8>(m);
+    if (L == 12) return tile_single<float2, 256, 16>(m);
+  }
+  if (prec == KG_PREC_C128) {
+    if (L <= 5) return tile_single<double2, 32, 1>(m);
+    if (L == 6) return tile_single<double2, 64, 1>(m);
+    if (L == 7) return tile_single<double2, 128, 1>(m);
+    if (L == 8) return tile_single<double2, 128, 2>(m);
+    if (L == 9) return tile_single<double2, 128, 4>(m);
+    if (L == 10) return tile_single<double2, 128, 8>(m);
+  }
+  return {};
+}
+
+}  // namespace
+
+bool tile_kernel_covers(int prec, int L) { return pick_tile(prec, L, 1).fn != nullptr; }
+int tile_kernel_threads(int prec, int L) { return pick_tile(prec, L, 1).threads; }
+
+cudaError_t launch_tile_kernel(int prec, const EvalParams& p, cudaStream_t stream) {
+  const TileKernel k = pick_tile(prec, p.L, p.m);
+  if (!k.fn) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {const_cast<EvalParams*>(&p)};
+  return cudaLaunchKernel(k.fn, dim3(1), dim3(k.threads), args, k.smem, stream);
+}
+
+cudaError_t launch_tile_list(int L, int m, const EvalParams* list, int n, cudaStream_t stream) {
+  const TileKernel k = pick_tile(KG_PREC_C64_F64REC, L, m);
+  if (!k.list) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(k.list, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {const_cast<EvalParams**>(&list)};
+  return cudaLaunchKernel(k.list, dim3(n), dim3(k.threads), args, k.smem, stream);
+}
+
+}  // namespace kg

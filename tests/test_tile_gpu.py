@@ -1,0 +1,103 @@
+"""The kernel that holds one tile of amplitudes per CTA in registers, against the oracle.
+
+It serves single evaluations whose schedule is left to the library on short chains.  Sizes: every
+block shape (chains with fewer amplitudes than a warp, one warp, several, the largest), every bond
+position and control site that has code of its own, basis sizes around the switch between shared
+and global memory, breakdowns, an invariant subspace, checkpoints and every gradient mode.
+Tolerances are those of test_parity_gpu.py: 1e-10 (complex128), 1e-5 / 1e-4 (complex64).
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2010_03598_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+TOL = {"c128": (1e-10, 1e-10), "c64": (1e-5, 1e-4)}
+
+
+def evaluate(spec, opts, u, psi0, f):
+    from paper_2010_03598_gb300 import api as A
+    dev = torch.device("cuda", 0)
+    eng = A.KGrape(A.ChainSpec(**spec), A.Options(**opts))
+    fid, grad = eng.evaluate(torch.tensor(u, device=dev), torch.tensor(psi0, device=dev), torch.tensor(f, device=dev))
+    rep = eng.sync()
+    out = float(fid.item()), (grad.cpu().numpy().copy() if opts["grad"] != "none" else None), rep
+    eng.close()
+    return out
+
+
+def problem(L, N, seed, hc):
+    rng = np.random.default_rng(seed)
+    u = rng.uniform(-1, 1, N)
+    # a target with a healthy overlap: relative errors are then those of the arithmetic (complex64
+    # rounding of an overlap far below a typical one would be amplified)
+    psi0 = rng.standard_normal(1 << L) + 1j * rng.standard_normal(1 << L)
+    psi0 /= np.linalg.norm(psi0)
+    f = psi0 + 0.8 * W.draw_target(rng, 1 << L)
+    f /= np.linalg.norm(f)
+    spec = dict(L=L, Jxy=1.0, Jz=0.7, hc_amp=0.9)
+    if hc == "sz":
+        mask = 1 | (1 << (L - 1))
+        return u, psi0, f, dict(spec, hc_kind="sz", hc_mask=mask), oracle.Chain(L, 1.0, 0.7, "sz", hc_mask=mask, hc_amp=0.9)
+    return u, psi0, f, dict(spec, hc_site=hc), oracle.Chain(L, 1.0, 0.7, "sx", hc_site=hc, hc_amp=0.9)
+
+
+def check(prec, F, g, F_ref, g_ref):
+    assert abs(F - F_ref) <= TOL[prec][0] * abs(F_ref), (F, F_ref)
+    if g is not None:
+        assert np.linalg.norm(g - g_ref) <= TOL[prec][1] * np.linalg.norm(g_ref)
+
+
+CASES = [(L, hc, m, mode) for L, hc, m, mode in [
+    (1, 0, 4, "centered"), (2, 1, 6, "exact"), (3, "sz", 8, "zeroth"), (4, 3, 12, "centered"), (5, 0, 1, "centered"),
+    (5, 4, 20, "exact"), (6, 5, 9, "none"), (6, "sz", 16, "centered"), (7, 6, 13, "exact"), (7, 0, 32, "zeroth"),
+    (8, 0, 12, "centered"), (8, 7, 32, "exact"), (8, 4, 2, "zeroth"), (9, 8, 20, "exact"), (9, "sz", 24, "centered"),
+    (10, 0, 11, "exact"), (10, 9, 10, "zeroth"), (10, 6, 25, "none"), (11, "sz", 13, "exact"), (11, 10, 12, "centered"),
+    (12, 0, 16, "exact"), (12, 11, 12, "centered"), (12, 8, 5, "zeroth")]]
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("L,hc,m,mode", CASES)
+def test_every_block_shape_and_mode_vs_oracle(L, hc, m, mode, prec):
+    N, dt = 7, 0.06
+    u, psi0, f, spec, ch = problem(L, N, 700 + L, hc)
+    F_ref, g_ref, _ = oracle.evaluate(ch, u, dt, m, psi0, f, "centered" if mode == "none" else mode)
+    F, g, rep = evaluate(spec, dict(N=N, dt=dt, m=m, prec=prec, grad=mode), u, psi0, f)
+    check(prec, F, g, F_ref, g_ref)
+    assert rep["status"] == 0 and abs(rep["norm_final"] - 1.0) < (1e-12 if prec == "c128" else 1e-5)
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("L,N,C", [(4, 9, 2), (8, 11, 4), (9, 6, 1), (11, 10, 9), (7, 5, 7)])
+def test_checkpoints_are_bitwise_equal_to_the_full_trajectory(L, N, C, prec):
+    u, psi0, f, spec, ch = problem(L, N, 800 + L, 0)
+    full = evaluate(spec, dict(N=N, dt=0.05, m=10, prec=prec, grad="centered"), u, psi0, f)
+    part = evaluate(spec, dict(N=N, dt=0.05, m=10, prec=prec, grad="centered", ckpt_every=C), u, psi0, f)
+    assert full[0] == part[0] and np.array_equal(full[1], part[1])
+    F_ref, g_ref, _ = oracle.evaluate(ch, u, 0.05, 10, psi0, f, "centered")
+    check(prec, full[0], full[1], F_ref, g_ref)
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("L", [6, 8, 11])
+def test_invariant_and_nearly_invariant_subspaces(L, prec):
+    # |0...0> is an eigenstate of H0 and of the Sz control: the basis ends after one vector.  With 1 %
+    # of a random state the identity for b_1 cancels, and b_1 is formed explicitly, in every slice.
+    N, m, dt, D = 5, 10, 0.05, 1 << L
+    u, psi0, f, spec, ch = problem(L, N, 900 + L, "sz")
+    for share in (0.0, 0.01):
+        p = share * psi0
+        p[0] += 1.0
+        p /= np.linalg.norm(p)
+        g = 0.5 * psi0 + 0.1 * f
+        g[0] += 1.0
+        g /= np.linalg.norm(g)
+        F_ref, g_ref, _ = oracle.evaluate(ch, u, dt, m, p, g, "centered")
+        F, gr, rep = evaluate(spec, dict(N=N, dt=dt, m=m, prec=prec, grad="centered"), u, p, g)
+        assert abs(F - F_ref) <= TOL[prec][0] * F_ref
+        # G_j = 2 dt Im <chi|Hc|psi> is the imaginary part of an overlap of modulus below 1 (exactly 0 in
+        # the eigenstate): its rounding is that of the overlap, held to the tolerance on F
+        assert np.linalg.norm(gr - g_ref) <= TOL[prec][0] * 2 * dt * np.sqrt(N)
+        assert rep["status"] == 0 and rep["breakdowns"] >= (N if share == 0.0 else 0)
