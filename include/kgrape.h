@@ -124,7 +124,8 @@ typedef struct kg_options {
                               kg_report.ckpt_every */
   int32_t tile_bits;       /* 0 = automatic; else amplitudes per tile = 2^tile_bits (6..13) */
   int32_t ctas;            /* 0 = automatic; else CTAs cooperating on the problem.  With both 0, chains
-                              that fit one CTA's registers run there (one CTA, no device-side wait) */
+                              that fit the registers of one CTA, or (complex128, L <= 18) of one
+                              tile per CTA, run there */
   int32_t flags;           /* KG_FLAG_* */
   double dt;               /* slice length, dt > 0 */
   double breakdown_tol;    /* <= 0: 1e-12 (C128) or 1e-5 (C64); Lanczos stops when
@@ -167,7 +168,7 @@ typedef struct kg_report {
                               [1] stage 2 (stencil inside the tile), [2] group reductions
                               incl. the barrier wait, [3] recurrence scalars and broadcast,
                               [4] small exponential, [5] recombination, [6] sweep setup,
-                              [7] total; zeros otherwise.  A single-CTA launch in registers: [0]
+                              [7] total; zeros otherwise.  One tile in registers per CTA: [0]
                               the whole Lanczos loop, [4]-[7] as above */
 } kg_report;
 

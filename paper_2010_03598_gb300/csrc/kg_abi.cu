@@ -198,8 +198,8 @@ kg_status configure_handle(const kg_chain* chain, const kg_options* opts, const 
     if (!(h->opts.breakdown_tol > 0.0)) h->opts.breakdown_tol = (opts->prec == KG_PREC_C128) ? 1e-12 : 1e-5;
     h->lay = lay;
     h->device = dev;
-    h->ctas = 1;
-    h->t_bits = chain->L;
+    h->ctas = kg::tile_kernel_ctas(opts->prec, chain->L);
+    h->t_bits = kg::tile_kernel_bits(opts->prec, chain->L);
     h->variant = kg::kVariantTile;
     return KG_OK;
   }
@@ -347,7 +347,11 @@ static kg_status enqueue(kg_handle* h, const double* u, const void* psi0, const 
   p.wait_limit_ns = g_wait_limit_ns.load();
   p.debug_fault = g_debug_fault.exchange(0);
   p.prof = (o.flags & KG_FLAG_PHASE_TIMING) ? (long long*)(ws + h->lay.prof) : nullptr;
-  cudaError_t e = cudaMemsetAsync(ws + h->lay.ctrl, 0, kg::kCtrlBytes, h->stream);
+  // the reduction slots follow the control block: one memset clears both
+  static_assert(kg::kCtrlBytes % kg::kAlign == 0, "reduction slots right behind the control block");
+  size_t clear = kg::kCtrlBytes;
+  if (h->variant == kg::kVariantTile) clear += kg::tile_kernel_clear_bytes(o.prec, ch.L);
+  cudaError_t e = cudaMemsetAsync(ws + h->lay.ctrl, 0, clear, h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(control block)");
   e = (h->variant == kg::kVariantTile) ? kg::launch_tile_kernel(o.prec, p, h->stream)
                                        : kg::launch_eval_kernel(o.prec, h->variant, p, h->ctas, h->stream);

@@ -29,10 +29,14 @@ int eval_kernel_threads(int prec, int variant, int t_bits);
 int max_tile_bits(int prec);
 int resident_tiles_per_cta(int prec);
 
-// Evaluation with one tile of amplitudes per CTA (kg_tile.cu): whether it covers a chain, its threads
-// per CTA and tile size (log2 amplitudes), and the launch.
+// Evaluation with one tile of amplitudes per CTA (kg_tile.cu): whether it covers a chain on the current
+// device, its threads per CTA, tile size (log2 amplitudes) and CTAs, the bytes at the start of the
+// reduction slots that have to be zero at launch, and the launch.
 bool tile_kernel_covers(int prec, int L);
 int tile_kernel_threads(int prec, int L);
+int tile_kernel_bits(int prec, int L);
+int tile_kernel_ctas(int prec, int L);
+size_t tile_kernel_clear_bytes(int prec, int L);
 cudaError_t launch_tile_kernel(int prec, const EvalParams& p, cudaStream_t stream);
 // n complex64 problems of one chain length and basis size (device array), one CTA each.
 cudaError_t launch_tile_list(int L, int m, const EvalParams* list, int n, cudaStream_t stream);

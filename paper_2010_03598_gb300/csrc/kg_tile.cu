@@ -183,7 +183,7 @@ struct Tile {
   const EvalParams& p;
   TileSmem& sm;
   V* sw;        // [2][T] the neighbours' vector, by the parity of the step; SB: [m][T], the basis itself
-  V* ring;      // MULTI: [slots][T] partner blocks of W_k
+  V* ring;      // MULTI: [RD][T] partner blocks of W_k
   int tid, wid, rank, D1;  // D1: amplitudes of the tile that exist (T, or fewer for chains below 5 spins)
   size_t base, D;
   int nb;       // bonds inside the tile
@@ -390,43 +390,57 @@ struct Tile {
     constexpr int b = LT + LA - 1;
     return ((unsigned)(li(j) >> b) ^ (unsigned)(base >> (b + 1))) & 1u;
   }
-  __device__ __forceinline__ void cross_issue(const V* w) {
-    constexpr int b0 = LT + LA - 1;
-    int s = 1;
-#pragma unroll
-    for (int j = 0; j < APT; ++j)
-      if (top_active(j)) cross_copy(ring + li(j), w + ((base + li(j)) ^ ((size_t)3 << b0)));
-    for (unsigned act = bonds_hi; act; act &= act - 1, ++s) {
-      const V* q = w + (base ^ ((size_t)3 << (__ffs(act) - 1)));
-#pragma unroll
-      for (int j = 0; j < APT; ++j) cross_copy(ring + s * T + li(j), q + li(j));
-    }
-    if (p.hc_kind == KG_HC_SX_SITE && p.hc_site > b0) {
-      const V* q = w + (base ^ ((size_t)1 << p.hc_site));
-#pragma unroll
-      for (int j = 0; j < APT; ++j) cross_copy(ring + s * T + li(j), q + li(j));
-    }
-    cp_async_commit();
+  static constexpr int RD = (T <= 1024) ? 6 : 4;  // slots of the ring
+  __device__ __forceinline__ int cross_count() const {
+    return 1 + __popc(bonds_hi) + ((p.hc_kind == KG_HC_SX_SITE && p.hc_site >= LT + LA) ? 1 : 0);
   }
-  __device__ __forceinline__ static void cross_copy(V* dst, const V* src) {
-    static_assert(!MULTI || sizeof(V) == 16, "the ring moves 16-byte amplitudes");
-    cp_async16(dst, src);
+  // Copies of block n into slot n % RD; `act`: the active bonds from block n on.  One commit group per
+  // block, empty past the last.
+  __device__ __forceinline__ void cross_copy(const V* w, int n, int count, unsigned& act) {
+    if constexpr (MULTI) {
+      V* r = ring + (n % RD) * T;
+      if (n == 0) {
+#pragma unroll
+        for (int j = 0; j < APT; ++j)
+          if (top_active(j)) cp_async16(r + li(j), w + ((base + li(j)) ^ ((size_t)3 << (LT + LA - 1))));
+      } else if (n < count) {
+        const V* q = w + (base ^ (act ? (size_t)3 << (__ffs(act) - 1) : (size_t)1 << p.hc_site));
+        act &= act - 1;
+#pragma unroll
+        for (int j = 0; j < APT; ++j) cp_async16(r + li(j), q + li(j));
+      }
+      cp_async_commit();
+    }
   }
-  __device__ __forceinline__ void cross_add(V (&h)[APT]) {
-    constexpr int b0 = LT + LA - 1;
-    cp_async_wait<0>();
+  __device__ __forceinline__ void cross_issue(const V* w, unsigned& act) {
+    act = bonds_hi;
+    const int count = cross_count();
+#pragma unroll
+    for (int n = 0; n < RD; ++n) cross_copy(w, n, count, act);
+  }
+  __device__ __forceinline__ void cross_add(const V* w, unsigned act, V (&h)[APT]) {
+    const int count = cross_count(), nb1 = 1 + __popc(bonds_hi);
     V x[APT];
 #pragma unroll
-    for (int j = 0; j < APT; ++j) x[j] = top_active(j) ? ring[li(j)] : vmake<V>(0, 0);
-    int s = 1;
-    for (unsigned act = bonds_hi; act; act &= act - 1, ++s)
+    for (int j = 0; j < APT; ++j) x[j] = vmake<V>(0, 0);
+    for (int n = 0; n < count; ++n) {
+      cp_async_wait<RD - 1>();
+      const V* r = ring + (n % RD) * T;
+      if (n == 0) {
 #pragma unroll
-      for (int j = 0; j < APT; ++j) x[j] = vadd(x[j], ring[s * T + li(j)]);
+        for (int j = 0; j < APT; ++j)
+          if (top_active(j)) x[j] = r[li(j)];
+      } else if (n < nb1) {
+#pragma unroll
+        for (int j = 0; j < APT; ++j) x[j] = vadd(x[j], r[li(j)]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < APT; ++j) h[j] = vfma(cx, r[li(j)], h[j]);
+      }
+      cross_copy(w, n + RD, count, act);
+    }
 #pragma unroll
     for (int j = 0; j < APT; ++j) h[j] = vfma(hxy, x[j], h[j]);
-    if (p.hc_kind == KG_HC_SX_SITE && p.hc_site > b0)
-#pragma unroll
-      for (int j = 0; j < APT; ++j) h[j] = vfma(cx, ring[s * T + li(j)], h[j]);
   }
 
   __device__ __forceinline__ V* sbasis(int k) const { return sw + k * T; }  // SB: v_k
@@ -506,11 +520,13 @@ struct Tile {
     for (int k = 0; k < meff; ++k) {
       const bool last = (k == m - 1);
       V h[APT];
+      const V* wk = (k > 0) ? gw(k) : src;
+      unsigned act = 0u;
       stencil(sw + (k & 1) * T, wo, h);
       if (k > 0) {  // alpha_{k-1}, b_k from the sums of step k - 1
         S o[kTileSums];
         if (!collect(o)) return false;
-        if constexpr (MULTI) cross_issue(gw(k));
+        if constexpr (MULTI) cross_issue(wk, act);
         if (!step_scalars(k - 1, false, o, vp, wo, tol, amax, bmax, ap, bk, ib, broke)) return false;
         if (broke) {
           meff = k;
@@ -518,9 +534,9 @@ struct Tile {
           break;
         }
       } else if constexpr (MULTI) {
-        cross_issue(src);
+        cross_issue(wk, act);
       }
-      if constexpr (MULTI) cross_add(h);
+      if constexpr (MULTI) cross_add(wk, act, h);
       R acc[3] = {0, 0, 0};
       V* sn = sw + ((k + 1) & 1) * T;
       V* vslot = (k > 0) ? gbasis(k) : nullptr;
@@ -1101,6 +1117,7 @@ __device__ __forceinline__ void tile_cta(const EvalParams& p, TileSmem& sm, V* s
   t.par = 0;
   t.run();
   if constexpr (MULTI) {
+    cp_async_wait<0>();  // an abandoned evaluation may have copies under way
     if (threadIdx.x == 0) sm.cmd = kTileCmdExit;
     nbar_arrive(kTileBarPost, NT + 32);
   }
@@ -1134,6 +1151,7 @@ struct TileKernel {
   const void* list = nullptr;  // complex64: a list of problems
   int threads = 0, tile_bits = 0;
   size_t smem = 0;
+  int ctas = 1;
 };
 
 // Basis in shared memory up to this size.
@@ -1154,6 +1172,15 @@ TileKernel tile_single(int m) {
   return tile_choice<V, NT, APT, false>(2 * vec);
 }
 
+// One of several CTAs: two W_k buffers and the ring of partner blocks.
+template <class V, int NT, int APT>
+TileKernel tile_multi(int L) {
+  using TileT = Tile<V, NT, APT, false, true>;
+  const int t = __builtin_ctz(NT * APT);
+  return {reinterpret_cast<const void*>(&kg_tile_kernel<V, NT, APT, false, true>), nullptr, NT + 32, t,
+          (size_t)(2 + TileT::RD) * TileT::T * sizeof(V), 1 << (L - t)};
+}
+
 // Threads x amplitudes by chain length.  More threads shorten every thread's chain of shared-memory
 // loads, fewer make the block's sums cheaper; measured (us per slice, m = 16, complex64):
 //   L = 7: 64 x 2 12.7, 32 x 4 12.3;  8: 128 x 2 14.1, 32 x 8 15.3, 64 x 4 15.7;  9: 256 x 2 17.3, 128 x 4
@@ -1161,8 +1188,12 @@ TileKernel tile_single(int m) {
 //   12: 256 x 16 (raw vectors) 47.7, 512 x 8 61.0 (128 registers).
 // The kernels that ran these chains before took 100 (L = 5) to 148 us (L = 11) and 77 us (L = 12).
 // complex128 is bound by the FP64 units, one quarter in each quarter of the SM: one warp per quarter
-// as soon as there are amplitudes for it (L = 8: 128 x 2 76, 64 x 4 113, 256 x 1 91; 9: 128 x 4 125,
-// 256 x 2 140).  Before: 351 us (L = 5, m = 20) to 620 us (L = 10); now 54 to 280.
+// as soon as there are amplitudes for it, and as many CTAs as there are SMs (us per slice, m = 16):
+//   L = 8: 128 x 2 76, 64 x 4 113, 256 x 1 91;  9: 4 CTAs of 128 x 1 76, 2 of 128 x 2 88, one CTA 125;
+//   10: 8 CTAs 79, 4 92, one CTA 222;  12: 32 CTAs 100, 16 111, 8 149;  14: 128 CTAs 123, 64 127;
+//   15: 128 x 2 146, 256 x 1 162;  16: 128 x 4 180, 256 x 2 219, 64 CTAs 299;  17: 256 x 4 313, 128 x 8 328;
+//   18: 256 x 8 588.
+// The streaming kernel takes 281 (L = 5) to 496 us (L = 10) for these, 776 at L = 16 and 833 at L = 18.
 TileKernel pick_tile(int prec, int L, int m) {
   if (prec == KG_PREC_C64_F64REC) {
     if (L <= 5) return tile_single<float2, 32, 1>(m);
@@ -1179,16 +1210,36 @@ TileKernel pick_tile(int prec, int L, int m) {
     if (L == 6) return tile_single<double2, 64, 1>(m);
     if (L == 7) return tile_single<double2, 128, 1>(m);
     if (L == 8) return tile_single<double2, 128, 2>(m);
-    if (L == 9) return tile_single<double2, 128, 4>(m);
-    if (L == 10) return tile_single<double2, 128, 8>(m);
+    if (L <= 14) return tile_multi<double2, 128, 1>(L);
+    if (L == 15) return tile_multi<double2, 128, 2>(L);
+    if (L == 16) return tile_multi<double2, 128, 4>(L);
+    if (L == 17) return tile_multi<double2, 256, 4>(L);
+    if (L == 18) return tile_multi<double2, 256, 8>(L);
   }
   return {};
 }
 
 }  // namespace
 
-bool tile_kernel_covers(int prec, int L) { return pick_tile(prec, L, 1).fn != nullptr; }
+bool tile_kernel_covers(int prec, int L) {
+  const TileKernel k = pick_tile(prec, L, 1);
+  if (!k.fn || k.ctas == 1) return k.fn != nullptr;
+  // the CTAs of a group wait for one another: all of them have to be resident at once
+  int per_sm = 0, dev = 0, sms = 0;
+  if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, k.smem) != cudaSuccess ||
+      cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return false;
+  return per_sm * sms >= k.ctas;
+}
 int tile_kernel_threads(int prec, int L) { return pick_tile(prec, L, 1).threads; }
+int tile_kernel_bits(int prec, int L) { return L < 5 ? L : pick_tile(prec, L, 1).tile_bits; }
+int tile_kernel_ctas(int prec, int L) { return pick_tile(prec, L, 1).ctas; }
+size_t tile_kernel_clear_bytes(int prec, int L) {
+  const int n = pick_tile(prec, L, 1).ctas;
+  return n > 1 ? (size_t)2 * n * kNRed * sizeof(ulonglong2) : 0;
+}
 
 cudaError_t launch_tile_kernel(int prec, const EvalParams& p, cudaStream_t stream) {
   const TileKernel k = pick_tile(prec, p.L, p.m);
@@ -1196,6 +1247,7 @@ cudaError_t launch_tile_kernel(int prec, const EvalParams& p, cudaStream_t strea
   cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<EvalParams*>(&p)};
+  if (k.ctas > 1) return cudaLaunchCooperativeKernel(k.fn, dim3(k.ctas), dim3(k.threads), args, k.smem, stream);
   return cudaLaunchKernel(k.fn, dim3(1), dim3(k.threads), args, k.smem, stream);
 }
 

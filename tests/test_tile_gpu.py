@@ -69,6 +69,51 @@ def test_every_block_shape_and_mode_vs_oracle(L, hc, m, mode, prec):
     assert rep["status"] == 0 and abs(rep["norm_final"] - 1.0) < (1e-12 if prec == "c128" else 1e-5)
 
 
+@pytest.mark.parametrize("L,hc,m,mode", [(13, 12, 9, "exact"), (14, 13, 6, "centered"), (15, "sz", 8, "zeroth"), (15, 7, 7, "none"),
+                                         (16, 8, 8, "centered"), (16, 9, 6, "exact"), (17, 16, 6, "centered"), (18, 0, 6, "zeroth")])
+def test_complex128_over_several_ctas_vs_oracle(L, hc, m, mode):
+    # 64 to 128 CTAs with one tile each: tiles of 128 to 2048 amplitudes, the control inside the tile, on
+    # its top bit (L = 16: bit 8) and above it
+    N, dt = 2, 0.05
+    u, psi0, f, spec, ch = problem(L, N, 750 + L, hc)
+    F_ref, g_ref, _ = oracle.evaluate(ch, u, dt, m, psi0, f, "centered" if mode == "none" else mode)
+    F, g, rep = evaluate(spec, dict(N=N, dt=dt, m=m, prec="c128", grad=mode), u, psi0, f)
+    check("c128", F, g, F_ref, g_ref)
+    assert rep["status"] == 0 and rep["ctas"] > 1
+
+
+def test_group_that_a_member_never_joins_times_out_cleanly():
+    # CTA 0 does not post its first sums (host-side fault injection): every wait runs out, the launch ends
+    # with KG_ERR_TIMEOUT, and the next launch on the same engine is clean and deterministic.
+    from paper_2010_03598_gb300 import _abi
+    from paper_2010_03598_gb300 import api as A
+    L, N = 12, 3
+    u, psi0, f, spec, ch = problem(L, N, 77, 0)
+    dev = torch.device("cuda", 0)
+    eng = A.KGrape(A.ChainSpec(**spec), A.Options(N, 0.05, 8, prec="c128"))
+    t = [torch.tensor(x, device=dev) for x in (u, psi0, f)]
+    for kind in (1, 2):
+        try:
+            A.set_wait_limit_ns(50_000_000)
+            _abi.check(_abi.lib().kg_debug_set_fault(kind), "kg_debug_set_fault")
+            eng.evaluate(*t)
+            with pytest.raises(_abi.KGrapeError) as ei:
+                eng.sync()
+            assert ei.value.status == _abi.KG_ERR_TIMEOUT
+        finally:
+            A.set_wait_limit_ns(2_000_000_000)
+            _abi.lib().kg_debug_set_fault(0)
+    got = []
+    for _ in range(2):
+        fid, grad = eng.evaluate(*t)
+        assert eng.sync()["ctas"] > 1
+        got.append((float(fid.item()), grad.cpu().numpy().copy()))
+    eng.close()
+    assert got[0][0] == got[1][0] and np.array_equal(got[0][1], got[1][1])
+    F_ref, g_ref, _ = oracle.evaluate(ch, u, 0.05, 8, psi0, f, "centered")
+    check("c128", *got[0], F_ref, g_ref)
+
+
 @pytest.mark.parametrize("prec", ["c64", "c128"])
 @pytest.mark.parametrize("L,N,C", [(4, 9, 2), (8, 11, 4), (9, 6, 1), (11, 10, 9), (7, 5, 7)])
 def test_checkpoints_are_bitwise_equal_to_the_full_trajectory(L, N, C, prec):
