@@ -892,6 +892,51 @@ __device__ __forceinline__ void tridiag_expv_e1_ff(const double* alpha, const do
   c_im = ff_to_double(yi);
 }
 
+// ---------------------------------------------------------------- sums of three values
+// Transposed butterflies: after the first two exchanges a lane carries one of four values (the fourth is
+// 0), so that three sums over a warp take six additions and six shuffles (float) instead of fifteen.
+__device__ __forceinline__ float vx_shfl(float a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ double vx_shfl(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ FF vx_shfl(FF a, int o) {
+  return FF{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ float vx_add(float a, float b) { return a + b; }
+__device__ __forceinline__ double vx_add(double a, double b) { return a + b; }
+__device__ __forceinline__ FF vx_add(FF a, FF b) { return ff_add(a, b); }
+__device__ __forceinline__ float vx_sel(bool c, float a, float b) { return c ? a : b; }
+__device__ __forceinline__ double vx_sel(bool c, double a, double b) { return c ? a : b; }
+__device__ __forceinline__ FF vx_sel(bool c, FF a, FF b) { return FF{c ? a.hi : b.hi, c ? a.lo : b.lo}; }
+__device__ __forceinline__ float vx_bcast(float a, int l) { return __shfl_sync(0xffffffffu, a, l); }
+__device__ __forceinline__ double vx_bcast(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
+__device__ __forceinline__ FF vx_bcast(FF a, int l) {
+  return FF{__shfl_sync(0xffffffffu, a.hi, l), __shfl_sync(0xffffffffu, a.lo, l)};
+}
+// Over the warp: lane l gets the sum of value l % 4.
+template <class T>
+__device__ __forceinline__ T warp_sum3(T v0, T v1, T v2) {
+  const int lane = threadIdx.x & 31;
+  const bool o1 = lane & 1, o2 = lane & 2;
+  const T zero = T();
+  const T s0 = vx_add(vx_sel(o1, v1, v0), vx_shfl(vx_sel(o1, v0, v1), 1));
+  const T s1 = vx_add(vx_sel(o1, zero, v2), vx_shfl(vx_sel(o1, v2, zero), 1));
+  T s = vx_add(vx_sel(o2, s1, s0), vx_shfl(vx_sel(o2, s0, s1), 2));
+#pragma unroll
+  for (int o = 4; o <= 16; o <<= 1) s = vx_add(s, vx_shfl(s, o));
+  return s;
+}
+// Over NW warps' partials (at(w, i): value i of warp w), in every lane: lane 4 w + i adds value i of the
+// warps w, w + 8.
+template <int NW, class T, class F>
+__device__ __forceinline__ void warps_sum3(F at, T (&out)[3]) {
+  const int lane = threadIdx.x & 31;
+  T s = at((lane >> 2) & (NW - 1), lane & 3);
+  if constexpr (NW == 16) s = vx_add(s, at(((lane >> 2) & 7) + 8, lane & 3));
+#pragma unroll
+  for (int o = 1; o < (NW < 8 ? NW : 8); o <<= 1) s = vx_add(s, vx_shfl(s, 4 * o));
+#pragma unroll
+  for (int i = 0; i < 3; ++i) out[i] = vx_bcast(s, i);
+}
+
 // ---------------------------------------------------------------- float-float square root, reciprocal
 // The FP32 estimate refined by one Newton step carried out in float-float (the residual a - s^2, or
 // 1 - b y, formed exactly with an FMA), about 44 bits.

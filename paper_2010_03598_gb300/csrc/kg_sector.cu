@@ -14,18 +14,23 @@
 // phi(t) = +1 for the smaller member of its orbit, p for the mirrored one (parity 0: one state per
 // orbit).  Row r' therefore needs H0 applied to the single state s_r': its diagonal
 // (Jz/4)(L-1 - 2 popcount((s ^ s>>1) & mask)), computed on the fly, and one term Jxy/2 per
-// antiparallel bond, landing in orbit r(t) with the factor sqrt(n_r'/n_r(t)) phi(t).  The host
-// tabulates those terms per row as 16-bit entries (13 bits: column r(t); 3 bits: one of the
-// factor classes 1, sqrt 2, 1/sqrt 2, -1, 0) in an ELL layout [entry][row], which the CTA keeps in
-// shared memory.  Hc is diagonal (mirror-symmetric Sz mask): hc_amp (popcount(mask) -
-// 2 popcount(s & mask))/2.
+// antiparallel bond, landing in orbit r(t) with the factor sqrt(n_r'/n_r(t)) phi(t), one of 1, sqrt 2,
+// 1/sqrt 2 and -1.  The host splits those terms by weight, so that the kernel decodes no weight: list A
+// holds the columns of weight Jxy/2, in an ELL layout [entry][row]; list B those of a second weight
+// (even parity: Jxy/(2 sqrt 2), a sqrt 2 listed twice; odd: -Jxy/2), which few rows have, in one ELL
+// slice per 32 rows.  Padding points at a zero element behind the vector.  Columns are 16 bits, two
+// in a word; the CTA keeps both lists in shared memory.  Hc is diagonal
+// (mirror-symmetric Sz mask): hc_amp (popcount(mask) - 2 popcount(s & mask))/2.
 //
-// One Lanczos step (App. A, Alg. "Lanczos", Paige's order), thread t owning rows t + NT i:
-//   w       = H v_k - b_k v_{k-1}                      (gather from shared memory)
+// One Lanczos step (App. A, Alg. "Lanczos", Paige's order), thread t owning rows t + NT i, v_{k-1}, v_k
+// and w in registers, v_k in shared memory for the gather:
+//   w       = H v_k - b_k v_{k-1}
 //   alpha_k = <v_k|w>,  b_{k+1}^2 = ||w||^2 - 2 alpha_k <v_k|w> + alpha_k^2 ||v_k||^2   (one block reduction)
 //   v_{k+1} = (w - alpha_k v_k) / b_{k+1}               (into shared memory and the basis)
-// Complex64 path: vectors and partial sums in FP32, cross-warp sums in float-float, the
-// tridiagonal T in FP64 (warp 0, once per slice).  Complex128 path: FP64 throughout.
+// with two block barriers: every warp adds up the warps' partial sums and forms the scalars for itself.
+// Complex64 path: vectors and partial sums in FP32, cross-warp sums, the tridiagonal T and its
+// exponential in float-float (warp 0, once per slice): no FP64 instruction between the first slice and
+// the last.  Complex128 path: FP64 throughout.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -72,38 +77,52 @@ __device__ __forceinline__ FFR operator*(FFR a, FFR b) {
   return FFR(p.hi, p.lo);
 }
 __device__ __forceinline__ FFR fma(FFR a, FFR b, FFR c) { return a * b + c; }
-// Scalar operations, once per Lanczos step: comparisons on (hi, lo) in order.
-__device__ __forceinline__ bool ffr_less(FFR a, FFR b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
-__device__ __forceinline__ FFR operator/(FFR a, FFR b) {
-  const FF q = ff_rcp(FF{b.hi, b.lo});
-  return a * FFR(q.hi, q.lo);
+// 1/sqrt(a) and sqrt(a): the FP32 estimate y refined by r/2 + 3 r^2 / 8, r = 1 - a y^2 formed exactly.
+__device__ __forceinline__ void ff_rsqrt(FF a, FF& root, FF& inv) {
+  if (!(a.hi > 1e-30f)) {
+    root = ff_sqrt(a);
+    inv = (root.hi > 0.f) ? ff_rcp(root) : FF{0.f, 0.f};
+    return;
+  }
+  const float y = rsqrtf(a.hi);
+  const float p = __fmul_rn(a.hi, y), e = __fmaf_rn(a.hi, y, -p);
+  const float q = __fmul_rn(p, y), f = __fmaf_rn(p, y, -q);
+  const float r = __fsub_rn(__fsub_rn(__fsub_rn(1.f, q), f), __fmul_rn(__fmaf_rn(a.lo, y, e), y));
+  inv = ff_two_sum(y, __fmul_rn(__fmul_rn(y, r), __fmaf_rn(0.375f, r, 0.5f)));
+  root = ff_mul(a, inv);
 }
-__device__ __forceinline__ bool operator<=(FFR a, FFR b) { return !ffr_less(b, a); }
-__device__ __forceinline__ FFR fmax(FFR a, FFR b) { return ffr_less(a, b) ? b : a; }
-__device__ __forceinline__ FFR fabs(FFR a) { return (a.hi < 0.f) ? -a : a; }
-__device__ __forceinline__ FFR sqrt(FFR a) {
-  const FF s = ff_sqrt(FF{a.hi, a.lo});
-  return FFR(s.hi, s.lo);
+// Unevaluated sum of many float-float terms: the high parts by TwoSum, everything below them in one FP32
+// accumulator; ff_close renormalises once at the end.
+__device__ __forceinline__ void ff_acc(FF& a, FFR v) {
+  const FF s = ff_two_sum(a.hi, v.hi);
+  a.hi = s.hi;
+  a.lo = __fadd_rn(a.lo, __fadd_rn(s.lo, v.lo));
 }
-// the float and double functions stay visible beside these overloads inside namespace kg
-using ::fma;
-using ::fmax;
-using ::fabs;
-using ::sqrt;
+__device__ __forceinline__ void ff_acc_mul(FF& a, FFR x, FFR y) {  // a += x y
+  const float p = __fmul_rn(x.hi, y.hi);
+  const float t = __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, __fmaf_rn(x.hi, y.hi, -p)));
+  const FF s = ff_two_sum(a.hi, p);
+  a.hi = s.hi;
+  a.lo = __fadd_rn(a.lo, __fadd_rn(s.lo, t));
+}
+__device__ __forceinline__ FF ff_close(FF a) {
+  const float hi = __fadd_rn(a.hi, a.lo);
+  return {hi, __fsub_rn(a.lo, __fsub_rn(hi, a.hi))};
+}
+__device__ __forceinline__ FF ff_of(FFR a) { return FF{a.hi, a.lo}; }
+__device__ __forceinline__ FFR ffr_of(FF a) { return FFR(a.hi, a.lo); }
+using ::fma;  // the float and double functions stay visible beside the overload inside namespace kg
 template <> struct VecTraits<FFC> { using R = FFR; };
 template <> __device__ __forceinline__ FFC vmake<FFC>(FFR a, FFR b) { return FFC{a, b}; }
 
-constexpr int kSecColBits = 13;
-constexpr int kSecMaxD = 1 << kSecColBits;  // columns fit the entry's 13 bits
-constexpr int kSecClasses = 8;
-enum SecClass { kSecW1 = 0, kSecWSqrt2 = 1, kSecWInvSqrt2 = 2, kSecWMinus1 = 3, kSecWZero = 7 };
 
 struct SectorParams {
-  int D, N, m, ell, B, L1, grad_mode;
+  int D, N, m, B, L1, grad_mode;
+  int na2, rows, groups, words;  // list A: words per row, row stride; 32-row groups; words of the whole table
   unsigned maskL1, hc_mask;
   double qz, hc_amp, dt, bd_tol;
-  double wcls[kSecClasses];      // weight of each entry class: (Jxy/2) x factor
-  const unsigned short* ell_g;   // [ell][D] entries
+  double wa, wb;                 // weights of lists A and B
+  const unsigned* tab_g;         // [na2][rows] list A, [groups] (first word << 8 | words a row) of list B, list B
   const unsigned* states;        // [D] s_r
   const double* u;               // [B][N]
   const double* psi0;            // [2D] complex128
@@ -129,20 +148,19 @@ struct SectorParams {
 __device__ __forceinline__ void sec_sync() { asm volatile("barrier.sync 0;" ::: "memory"); }
 
 struct SecSmem {
-  float red_f[2][32 * 4];   // warp partials (complex64), by reduction parity
-  double red_d[2][32 * 4];  // warp partials (complex128)
-  float2 tot_f[2][4];       // float-float totals
-  double tot_d[2][4];
-  float wcls_f[kSecClasses];
-  double wcls_d[kSecClasses];
-  float2 wcls_ff[kSecClasses];  // float-float (hi, lo)
-  double alpha[kMaxM], beta[kMaxM + 1];
-  float alpha_f[kMaxM], beta_f[kMaxM + 1];
-  float2 ff_a[kMaxM], ff_n[kMaxM], ff_q[kMaxM], ff_e[kMaxM];
+  float red_f[2][16 * 4];   // warp partials by reduction parity: complex64
+  float2 red_ff[2][16 * 4]; // float-float
+  double red_d[2][16 * 4];  // complex128, and FP64 sums of every path
+  double alpha[kMaxM], beta[kMaxM + 1];    // T, FP64
+  float alpha_f[kMaxM], beta_f[kMaxM + 1]; // its FP32 copies (norm bounds, Taylor terms)
+  float2 ff_a[kMaxM], ff_n[kMaxM], ff_q[kMaxM], ff_e[kMaxM];  // the steps' sums; ff_e: b_{k+1}^2 (complex64),
+                                                              // or the explicit one (float-float)
+  float2 tau_ff[3];            // complex64: dt and the interior quadrature nodes
+  float2 diag_ff[2];           // Jz / 4 and hc_amp / 2
+  double diag_d[2];
   float coef_f[3][2][kMaxM];   // [slice end, interior node a, b][re, im][k]
   double coef_d[3][2][kMaxM];
-  double nrm_d, ex_d, tay_d, err_max;
-  float beta_m_f, inv_f;
+  float err_max;
   unsigned ff_e_set;
   int breakdowns;
   int abort;                    // the pulse in hand is abandoned (status set)
@@ -163,70 +181,38 @@ __device__ __forceinline__ void sec_mark(const SectorParams& p, SecSmem& sm, int
 }
 
 // ---------------------------------------------------------------- block reductions
-// Every thread receives the totals.  Two barriers: warp partials, then warp v sums value v.
-template <int NT, int NV>
-__device__ __forceinline__ void sec_reduce(SecSmem& sm, int& par, const float (&vals)[NV], FF (&out)[NV]) {
+// Every thread receives the three totals, the same bits in each.  One barrier: the warps' partials, then
+// every warp adds them up for itself (the partials alternate between two sets, so that the next
+// reduction's do not overwrite what a slow warp still reads).
+template <int NT>
+__device__ __forceinline__ void sec_reduce(SecSmem& sm, int& par, float v0, float v1, float v2, FF (&out)[3]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* red = sm.red_f[par];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const float x = warp_sum(vals[v]);
-    if (lane == 0) red[warp * 4 + v] = x;
-  }
-  sec_sync();
-  if (warp < NV) {
-    FF s{(lane < NT / 32) ? red[lane * 4 + warp] : 0.f, 0.f};
-    s = ff_warp_sum(s);
-    if (lane == 0) sm.tot_f[par][warp] = make_float2(s.hi, s.lo);
-  }
-  sec_sync();
-#pragma unroll
-  for (int v = 0; v < NV; ++v) out[v] = FF{sm.tot_f[par][v].x, sm.tot_f[par][v].y};
   par ^= 1;
+  const float s = warp_sum3(v0, v1, v2);
+  if (lane < 4) red[warp * 4 + lane] = s;
+  sec_sync();
+  warps_sum3<NT / 32, FF>([&](int w, int i) { return FF{red[w * 4 + i], 0.f}; }, out);
 }
-template <int NT, int NV>
-__device__ __forceinline__ void sec_reduce(SecSmem& sm, int& par, const double (&vals)[NV], double (&out)[NV]) {
+template <int NT>
+__device__ __forceinline__ void sec_reduce(SecSmem& sm, int& par, FF v0, FF v1, FF v2, FF (&out)[3]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float2* red = sm.red_ff[par];
+  par ^= 1;
+  const FF s = warp_sum3(v0, v1, v2);
+  if (lane < 4) red[warp * 4 + lane] = make_float2(s.hi, s.lo);
+  sec_sync();
+  warps_sum3<NT / 32, FF>([&](int w, int i) { return FF{red[w * 4 + i].x, red[w * 4 + i].y}; }, out);
+}
+template <int NT>
+__device__ __forceinline__ void sec_reduce(SecSmem& sm, int& par, double v0, double v1, double v2, double (&out)[3]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double* red = sm.red_d[par];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const double x = warp_sum(vals[v]);
-    if (lane == 0) red[warp * 4 + v] = x;
-  }
-  sec_sync();
-  if (warp < NV) {
-    double s = (lane < NT / 32) ? red[lane * 4 + warp] : 0.0;
-    s = warp_sum(s);
-    if (lane == 0) sm.tot_d[par][warp] = s;
-  }
-  sec_sync();
-#pragma unroll
-  for (int v = 0; v < NV; ++v) out[v] = sm.tot_d[par][v];
   par ^= 1;
-}
-
-// Float-float partial sums (KG_PREC_FF): the same two stages, warp sums by ff_add (the warp partials
-// are kept in the complex128 path's slots, two floats in each).
-template <int NT, int NV>
-__device__ __forceinline__ void sec_reduce(SecSmem& sm, int& par, const FF (&vals)[NV], FF (&out)[NV]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float2* red = reinterpret_cast<float2*>(sm.red_d[par]);
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const FF x = ff_warp_sum(vals[v]);
-    if (lane == 0) red[warp * 4 + v] = make_float2(x.hi, x.lo);
-  }
+  const double s = warp_sum3(v0, v1, v2);
+  if (lane < 4) red[warp * 4 + lane] = s;
   sec_sync();
-  if (warp < NV) {
-    FF s{0.f, 0.f};
-    if (lane < NT / 32) s = FF{red[lane * 4 + warp].x, red[lane * 4 + warp].y};
-    s = ff_warp_sum(s);
-    if (lane == 0) sm.tot_f[par][warp] = make_float2(s.hi, s.lo);
-  }
-  sec_sync();
-#pragma unroll
-  for (int v = 0; v < NV; ++v) out[v] = FF{sm.tot_f[par][v].x, sm.tot_f[par][v].y};
-  par ^= 1;
+  warps_sum3<NT / 32, double>([&](int w, int i) { return red[w * 4 + i]; }, out);
 }
 
 __device__ __forceinline__ void sec_flag(const SectorParams& p, int code) { atomicCAS(p.ctrl, 0, code); }
@@ -248,21 +234,166 @@ template <class V> __device__ __forceinline__ V vaxpy(typename VecTraits<V>::R a
   return vmake<V>(fma(a, x.x, y.x), fma(a, x.y, y.y));
 }
 
-// Scalars of step k from the reduced sums o = (<v|w>, ||w||^2, ||v||^2), computed by every thread
-// alike.  code: 0 go on, 1 the identity cancels (form ||w - alpha v||^2 explicitly), 2 non-finite.
-struct SecStep {
-  float alpha, b2;
-  int code;
+// ---------------------------------------------------------------- per-precision scalars
+// S: a step's sums; N: ||x|| between slices.
+template <class V> struct SecPrec;
+template <> struct SecPrec<float2> {
+  using S = FF;
+  using N = FF;
 };
-__device__ __forceinline__ SecStep sec_scalars(const FF (&o)[3], bool last, FF& b2ff) {
-  SecStep s;
-  s.alpha = __fadd_rn(o[0].hi, o[0].lo);
-  b2ff = ff_add(o[1], ff_mul(ff_mul(o[0], o[0]), ff_add(o[2], FF{-2.f, 0.f})));
-  s.b2 = __fadd_rn(b2ff.hi, b2ff.lo);
-  s.code = 0;
-  if (!isfinite(s.alpha) || !isfinite(o[1].hi)) s.code = 2;
-  else if (!last && b2ff.hi < 1e-3f * o[1].hi) s.code = 1;
-  return s;
+template <> struct SecPrec<FFC> {
+  using S = FF;
+  using N = double;
+};
+template <> struct SecPrec<double2> {
+  using S = double;
+  using N = double;
+};
+// Per-row partial sums: acc += x y.
+__device__ __forceinline__ void sacc(float& a, float x, float y) { a = fmaf(x, y, a); }
+__device__ __forceinline__ void sacc(double& a, double x, double y) { a = ::fma(x, y, a); }
+__device__ __forceinline__ void sacc(FF& a, FFR x, FFR y) { ff_acc_mul(a, x, y); }
+__device__ __forceinline__ float sclose(float a) { return a; }
+__device__ __forceinline__ double sclose(double a) { return a; }
+__device__ __forceinline__ FF sclose(FF a) { return ff_close(a); }
+template <class R> struct SecAcc { using T = R; };
+template <> struct SecAcc<FFR> { using T = FF; };
+
+// alpha_k, b_{k+1} and 1/b_{k+1} from a step's sums (or from an explicit b_{k+1}^2).
+__device__ __forceinline__ FF sec_b2(const FF (&o)[3]) {
+  return ff_add(o[1], ff_mul(ff_mul(o[0], o[0]), ff_add(o[2], FF{-2.f, 0.f})));
+}
+__device__ __forceinline__ double sec_b2(const double (&o)[3]) { return ::fma(o[0] * o[0], o[2] - 2.0, o[1]); }
+__device__ __forceinline__ void sec_roots(FF b2, float& b, float& ib) {
+  FF r, i;
+  ff_rsqrt(b2, r, i);
+  b = __fadd_rn(r.hi, r.lo);
+  ib = __fadd_rn(i.hi, i.lo);
+}
+__device__ __forceinline__ void sec_roots(FF b2, FFR& b, FFR& ib) {
+  FF r, i;
+  ff_rsqrt(b2, r, i);
+  b = ffr_of(r);
+  ib = ffr_of(i);
+}
+__device__ __forceinline__ void sec_roots(double b2, double& b, double& ib) {
+  if (!(b2 > 1e-30 && b2 < 1e30)) {
+    b = ::sqrt(::fmax(b2, 0.0));
+    ib = (b > 0.0) ? 1.0 / b : 0.0;
+    return;
+  }
+  const double y = (double)rsqrtf((float)b2);  // one step of Halley's iteration: 2^-22 -> below 2^-60
+  const double r = ::fma(-b2 * y, y, 1.0);
+  ib = ::fma(y, r * ::fma(0.375, r, 0.5), y);
+  b = b2 * ib;
+}
+__device__ __forceinline__ float sec_top(FF a) { return a.hi; }
+__device__ __forceinline__ double sec_top(double a) { return a; }
+// The identity for b^2 cancels: near an invariant subspace.
+__device__ __forceinline__ bool sec_cancels(FF b2, FF n) { return b2.hi < 1e-3f * n.hi; }
+__device__ __forceinline__ bool sec_cancels(double b2, double n) { return b2 < 1e-3 * n; }
+__device__ __forceinline__ float sec_real(FF a, float) { return __fadd_rn(a.hi, a.lo); }
+__device__ __forceinline__ FFR sec_real(FF a, FFR) { return ffr_of(a); }
+__device__ __forceinline__ double sec_real(double a, double) { return a; }
+__device__ __forceinline__ float sec_f32(float a) { return a; }
+__device__ __forceinline__ float sec_f32(double a) { return (float)a; }
+__device__ __forceinline__ float sec_f32(FFR a) { return a.hi; }
+// A sum kept in 8 bytes of a double array between slices.
+__device__ __forceinline__ double sec_pack(FF a) { return __hiloint2double(__float_as_int(a.hi), __float_as_int(a.lo)); }
+__device__ __forceinline__ double sec_pack(double a) { return a; }
+template <bool F32>
+__device__ __forceinline__ double sec_unpack(double d) {
+  if constexpr (F32) return (double)__int_as_float(__double2hiint(d)) + (double)__int_as_float(__double2loint(d));
+  else return d;
+}
+
+// ---------------------------------------------------------------- H in the subspace
+// h = (diagonal + H0's couplings) x - bk xp on the own rows; S holds x for the gather (element D is 0).
+// The words of list A are read row by row in step, so that every thread has its rows' loads in flight
+// together.
+template <class V, int NT, int RPT>
+__device__ __forceinline__ void sec_apply(const SectorParams& p, const V* S, const unsigned* tab,
+                                          const typename VecTraits<V>::R (&dj)[RPT], const V (&x)[RPT],
+                                          typename VecTraits<V>::R bk, const V (&xp)[RPT], V (&h)[RPT]) {
+  using R = typename VecTraits<V>::R;
+  constexpr bool FFM = std::is_same<R, FFR>::value;
+  const int tid = threadIdx.x, D = p.D;
+  const unsigned* ta = tab + min(tid, D);
+  const unsigned* meta = tab + p.na2 * p.rows;
+  const unsigned* tb = meta + p.groups + (tid & 31);
+  const R wa = (R)p.wa;
+  if constexpr (FFM) {
+    FF ax[RPT], ay[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) ax[i] = ay[i] = FF{0.f, 0.f};
+    for (int q = 0; q < p.na2; ++q) {
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        const unsigned w = (tid + NT * i <= D) ? ta[q * p.rows + NT * i] : tab[q * p.rows + D];
+        const V a = S[w & 0xffffu], b = S[w >> 16];
+        ff_acc(ax[i], a.x);
+        ff_acc(ay[i], a.y);
+        ff_acc(ax[i], b.x);
+        ff_acc(ay[i], b.y);
+      }
+    }
+    const FF wf = ff_of(wa), nb = ff_of(-bk);
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+      const FF d = ff_of(dj[i]);
+      h[i].x = ffr_of(ff_dot3(d, ff_of(x[i].x), wf, ff_close(ax[i]), nb, ff_of(xp[i].x)));
+      h[i].y = ffr_of(ff_dot3(d, ff_of(x[i].y), wf, ff_close(ay[i]), nb, ff_of(xp[i].y)));
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) h[i] = vscale<V>(dj[i], x[i]);
+#pragma unroll 2
+    for (int q = 0; q < p.na2; ++q) {
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        const unsigned w = (tid + NT * i <= D) ? ta[q * p.rows + NT * i] : tab[q * p.rows + D];
+        h[i] = vaxpy<V>(wa, S[w & 0xffffu], h[i]);
+        h[i] = vaxpy<V>(wa, S[w >> 16], h[i]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) h[i] = vaxpy<V>(-bk, xp[i], h[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) {  // list B: the same number of words for all lanes of a warp
+    const int g = (tid >> 5) + (NT / 32) * i;
+    if (g < p.groups) {
+      const unsigned mt = meta[g];
+      const R wb = (R)p.wb;
+      for (unsigned q = 0; q < (mt & 0xffu); ++q) {
+        const unsigned w = tb[(mt >> 8) + 32 * q];
+        h[i] = vaxpy<V>(wb, S[w & 0xffffu], h[i]);
+        h[i] = vaxpy<V>(wb, S[w >> 16], h[i]);
+      }
+    }
+  }
+}
+
+// The diagonals of H0 and of Hc on the row of state st: a weight (float-float, so that FP32 and
+// float-float need no FP64 instruction) times a small whole number.
+__device__ __forceinline__ float sec_times(const SecSmem& sm, int which, int n, float) {
+  const float2 q = sm.diag_ff[which];
+  return fmaf(q.x, (float)n, q.y * (float)n);
+}
+__device__ __forceinline__ FFR sec_times(const SecSmem& sm, int which, int n, FFR) {
+  const float2 q = sm.diag_ff[which];
+  return ffr_of(ff_mul(FF{q.x, q.y}, FF{(float)n, 0.f}));
+}
+__device__ __forceinline__ double sec_times(const SecSmem& sm, int which, int n, double) {
+  return sm.diag_d[which] * (double)n;
+}
+template <class R>
+__device__ __forceinline__ R sec_d0(const SectorParams& p, const SecSmem& sm, unsigned st) {
+  return sec_times(sm, 0, p.L1 - 2 * __popc((st ^ (st >> 1)) & p.maskL1), R());
+}
+template <class R>
+__device__ __forceinline__ R sec_hc(const SectorParams& p, const SecSmem& sm, unsigned st) {
+  return sec_times(sm, 1, __popc(p.hc_mask) - 2 * __popc(st & p.hc_mask), R());
 }
 
 // Taylor-hierarchy terms of backward slice j (App. B, Eq. gradp), this thread's partial sum:
@@ -275,26 +406,23 @@ __device__ __forceinline__ SecStep sec_scalars(const FF (&o)[3], bool last, FF& 
 // line: it runs once per backward slice and its arrays would crowd the Lanczos loop's registers.
 template <class V, int NT, int RPT>
 __device__ __noinline__ typename VecTraits<V>::R sec_taylor(const SectorParams& p, SecSmem& sm, V* Sa, V* Sb,
-                                                          const unsigned short* ell, const V* basis, double uj,
+                                                          const unsigned* tab, const V* basis, double uj,
                                                           int meff, typename VecTraits<V>::R nin, int taylor,
                                                           const V* psi_end) {
   using R = typename VecTraits<V>::R;
   constexpr bool F32 = sizeof(R) == 4;
-  const int tid = threadIdx.x, D = p.D, ne = p.ell;
-  const R* wcls = F32 ? (const R*)sm.wcls_f : (const R*)sm.wcls_d;
-  // the diagonals of H0 and Hc, formed again here from the rows' states (as in sec_eval)
+  const int tid = threadIdx.x, D = p.D;
+  // the diagonals of H0 and Hc, formed again here from the rows' states
   R dj[RPT], hh[RPT];
-  const int npc = __popc(p.hc_mask);
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
     const int r = tid + NT * i;
     dj[i] = 0;
     hh[i] = 0;
     if (r < D) {
-      const unsigned st = p.states[r];
-      const R d0 = (R)(p.qz * (double)(p.L1 - 2 * __popc((st ^ (st >> 1)) & p.maskL1)));
-      hh[i] = (R)(0.5 * p.hc_amp * (double)(npc - 2 * __popc(st & p.hc_mask)));
-      dj[i] = fma((R)uj, hh[i], d0);
+      const unsigned st = __ldg(p.states + r);
+      hh[i] = sec_hc<R>(p, sm, st);
+      dj[i] = fma((R)uj, hh[i], sec_d0<R>(p, sm, st));
     }
   }
   R pt = 0;
@@ -303,40 +431,19 @@ __device__ __noinline__ typename VecTraits<V>::R sec_taylor(const SectorParams& 
   for (int i = 0; i < RPT; ++i) {
     const int r = tid + NT * i;
     b0[i] = (r < D) ? psi_end[r] : vmake<V>(0, 0);
-    b2[i] = vmake<V>(0, 0);
+    b1[i] = b2[i] = vmake<V>(0, 0);
     if (r < D) Sa[r] = b0[i];
   }
   sec_sync();
-#pragma unroll
-  for (int i = 0; i < RPT; ++i) {
-    const int r = tid + NT * i;
-    V h = vmake<V>(0, 0);
-    if (r < D) {
-      h = vscale<V>(dj[i], b0[i]);
-#pragma unroll 4
-      for (int e = 0; e < ne; ++e) {
-        const unsigned en = ell[e * D + r];
-        h = vaxpy<V>(wcls[en >> kSecColBits], Sa[en & (kSecMaxD - 1)], h);
-      }
-      if (taylor >= 2) Sb[r] = h;
-    }
-    b1[i] = h;
-  }
+  sec_apply<V, NT, RPT>(p, Sa, tab, dj, b0, (R)0, b2, b1);
   if (taylor >= 2) {
-    sec_sync();
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
       const int r = tid + NT * i;
-      if (r < D) {
-        V h = vscale<V>(dj[i], b1[i]);
-#pragma unroll 4
-        for (int e = 0; e < ne; ++e) {
-          const unsigned en = ell[e * D + r];
-          h = vaxpy<V>(wcls[en >> kSecColBits], Sb[en & (kSecMaxD - 1)], h);
-        }
-        b2[i] = h;
-      }
+      if (r < D) Sb[r] = b1[i];
     }
+    sec_sync();
+    sec_apply<V, NT, RPT>(p, Sb, tab, dj, b1, (R)0, b0, b2);
   }
   const R al0 = (meff > 0) ? (F32 ? (R)sm.alpha_f[0] : (R)sm.alpha[0]) : (R)0;
   const R al1 = (meff > 1) ? (F32 ? (R)sm.alpha_f[1] : (R)sm.alpha[1]) : (R)0;
@@ -379,13 +486,12 @@ __device__ __noinline__ typename VecTraits<V>::R sec_interior(const SectorParams
   using R = typename VecTraits<V>::R;
   constexpr bool F32 = sizeof(R) == 4;
   const int tid = threadIdx.x, D = p.D;
-  const int npc = __popc(p.hc_mask);
   R pg = 0;
   for (int w = 1; w <= 2; ++w) {
     V y[RPT];
 #pragma unroll
     for (int i = 0; i < RPT; ++i) y[i] = vmake<V>(0, 0);
-    for (int k = 0; k < meff; ++k) {
+    for (int k = meff - 1; k >= 0; --k) {
       const R a = F32 ? (R)sm.coef_f[w][0][k] : (R)sm.coef_d[w][0][k];
       const R b = F32 ? (R)sm.coef_f[w][1][k] : (R)sm.coef_d[w][1][k];
 #pragma unroll
@@ -406,228 +512,233 @@ __device__ __noinline__ typename VecTraits<V>::R sec_interior(const SectorParams
       if (lob == 1) {
         slot[r] = y[i];
       } else {
-        const unsigned st = p.states[r];
-        const R hc = (R)(0.5 * p.hc_amp * (double)(npc - 2 * __popc(st & p.hc_mask)));
         const V o = slot[r];
-        pg = fma(hc, y[i].x * o.y - y[i].y * o.x, pg);  // Im(conj(chi_s) Hc psi_s), Hc diagonal
+        pg = fma(sec_hc<R>(p, sm, __ldg(p.states + r)), y[i].x * o.y - y[i].y * o.x, pg);  // Im(conj(chi_s) Hc psi_s), Hc diagonal
       }
     }
   }
   return pg;
 }
 
-// One slice: x (own rows, norm nrm) -> x = ||x|| V exp(-i tau T) e_1 (App. A), written to dst
-// (if not null), then ||x||^2 and, for extra = 1, G = Im <x| Hc |other> over the own rows are
-// reduced.  Returns false after a non-finite coefficient (status set).
-template <class V, int NT, int RPT>
-__device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, int& par, V* Sa, V* Sb,
-                                          const unsigned short* ell, V* basis,
-                                          const typename VecTraits<V>::R (&dd)[RPT],
-                                          const typename VecTraits<V>::R (&hh)[RPT], double uj, double tau,
-                                          V (&x)[RPT], double& nrm, typename VecTraits<V>::R& inv, int extra,
-                                          const V* other, V* dst, double& ex, int taylor = 0,
-                                          const V* psi_end = nullptr, double* tay = nullptr, int lob = 0,
-                                          V* tint_io = nullptr) {
+// The small exponentials of a slice and the recombination coefficients, one warp each: the slice end
+// (w = 0) and, with lob, the interior nodes s_a, s_b = (1 -+ 1/sqrt 5) dt/2 (forward exp(-i s H) psi_{j-1},
+// backward exp(+i (dt - s) H) chi_j, dt - s_a = s_b).  Warp 0 also keeps the error indicator and checks
+// the pulse's time limit.
+template <class V>
+__device__ __forceinline__ void sec_coefficients(const SectorParams& p, SecSmem& sm, int w, bool back, int meff,
+                                                 bool broke, float beta_m, typename SecPrec<V>::N nrm, float2 fact) {
   using R = typename VecTraits<V>::R;
   constexpr bool F32 = sizeof(R) == 4;
+  const int k = threadIdx.x & 31;
+  // The exponential takes ceil(||tau T|| / 4) sub-steps: refuse a T whose Gershgorin bound is not a
+  // finite, sane number (it would come from corrupted coefficients) instead of looping on it.
+  float row = 0.f;
+  if (k < meff) row = (float)p.dt * (fabsf(sm.alpha_f[k]) + (k >= 1 ? sm.beta_f[k] : 0.f) + (k + 1 < meff ? sm.beta_f[k + 1] : 0.f));
+  row = (row == row) ? row : 3.0e38f;  // NaN -> refused
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) row = fmaxf(row, __shfl_xor_sync(0xffffffffu, row, o));
+  const bool sane = row <= 1.0e5f;
+  if (w == 0 && k == 0 && !sane) {
+    sec_flag(p, KG_ERR_NONFINITE);
+    sec_record(sm, -1, 3);
+    sm.abort = 1;
+  }
+  float tnorm = 0.f, cre = 0.f, cim = 0.f, n0;
+  if constexpr (F32) {
+    const float2 a2 = (k < meff) ? sm.ff_a[k] : make_float2(0.f, 0.f);
+    const float2 b2 = (k >= 1 && k < meff) ? sm.ff_e[k - 1] : make_float2(0.f, 0.f);
+    const float2 t2 = sm.tau_ff[back && w > 0 ? 3 - w : w];
+    const FF t = back ? FF{-t2.x, -t2.y} : FF{t2.x, t2.y};
+    FF fr{0.f, 0.f}, fi{0.f, 0.f};
+    if (meff > 0 && sane) tridiag_expv_e1_fff(FF{a2.x, a2.y}, ff_sqrt(FF{b2.x, b2.y}), meff, t, 1e-13f, fact, fr, fi, tnorm);
+    const FF cr = ff_mul(fr, nrm), ci = ff_mul(fi, nrm);
+    cre = __fadd_rn(cr.hi, cr.lo);
+    cim = __fadd_rn(ci.hi, ci.lo);
+    n0 = nrm.hi;
+    if (k < meff) {
+      sm.coef_f[w][0][k] = cre;
+      sm.coef_f[w][1][k] = cim;
+    }
+  } else {
+    double tw = p.dt;
+    if (w > 0) tw = 0.5 * p.dt * (1.0 + ((w == 1) != back ? -1.0 : 1.0) / ::sqrt(5.0));
+    if (back) tw = -tw;
+    double cr = 0.0, ci = 0.0;
+    if (meff > 0 && sane) tridiag_expv_e1(sm.alpha, sm.beta, sm.alpha_f, sm.beta_f, meff, tw, (float)tw, 1e-18, cr, ci, tnorm);
+    cr *= nrm;
+    ci *= nrm;
+    if (k < meff) {
+      sm.coef_d[w][0][k] = cr;
+      sm.coef_d[w][1][k] = ci;
+    }
+    cre = (float)cr;
+    cim = (float)ci;
+    n0 = (float)nrm;
+  }
+  if (w == 0 && k == meff - 1) {  // a-posteriori indicator ||x|| b_m |c_{m-1}| (0 after a breakdown)
+    float cm = sqrtf(cre * cre + cim * cim);
+    if (cm == 0.f && !broke) {
+      cm = n0;
+      for (int i = 1; i < meff; ++i) cm *= tnorm * kInvFF[i].x;
+    }
+    if (broke) sm.breakdowns += 1;
+    else sm.err_max = fmaxf(sm.err_max, beta_m * cm);
+  }
+  __syncwarp();
+  if (w == 0 && k == 0) {
+    sm.ff_e_set = 0u;
+    // time limit of one pulse: a pulse that runs past it ends with KG_ERR_TIMEOUT
+    if (sm.abort == 0 && (long long)(globaltimer_ns() - sm.t_start) > p.time_limit_ns) {
+      sec_flag(p, KG_ERR_TIMEOUT);
+      sec_record(sm, -1, 4);
+      sm.abort = 1;
+    }
+  }
+}
+
+// One slice: x (own rows, norm nrm, inv = 1/nrm) -> x = ||x|| V exp(-+i dt T) e_1 (App. A; back: the
+// co-state sweep), written to dst (if not null), then ||x||^2 and, back, ex = Im <x| Hc |other> over the
+// own rows are reduced.  Returns false after a non-finite coefficient (status set).
+template <class V, int NT, int RPT>
+__device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, int& par, V* Sa, V* Sb,
+                                          const unsigned* tab, V* basis, double uj, bool back, V (&x)[RPT],
+                                          typename SecPrec<V>::N& nrm, typename VecTraits<V>::R& inv, const V* other,
+                                          V* dst, typename SecPrec<V>::N& ex, int taylor, const V* psi_end,
+                                          typename SecPrec<V>::N& tay, int lob, V* tint_io, float2 fact) {
+  using R = typename VecTraits<V>::R;
+  using S = typename SecPrec<V>::S;
+  using A = typename SecAcc<R>::T;
+  constexpr bool F32 = sizeof(R) == 4;
   constexpr bool FFM = std::is_same<R, FFR>::value;  // float-float vectors (KG_PREC_FF)
-  const int tid = threadIdx.x, D = p.D, m = p.m, ne = p.ell;
-  const R* wcls = F32 ? (const R*)sm.wcls_f : FFM ? (const R*)sm.wcls_ff : (const R*)sm.wcls_d;
+  const int tid = threadIdx.x, D = p.D, m = p.m;
   R dj[RPT];
 #pragma unroll
-  for (int i = 0; i < RPT; ++i) dj[i] = fma((R)uj, hh[i], dd[i]);
+  for (int i = 0; i < RPT; ++i) {
+    const int r = tid + NT * i;
+    dj[i] = 0;
+    if (r < D) {
+      const unsigned st = __ldg(p.states + r);
+      dj[i] = fma((R)uj, sec_hc<R>(p, sm, st), sec_d0<R>(p, sm, st));
+    }
+  }
   // ---- v_0 = x / ||x||
-  const R inv0 = inv;
-  const R nin = (R)nrm;  // ||x||: the Taylor terms rebuild H x, H^2 x from the basis
+  V v[RPT], vp[RPT], w[RPT];
   V* Sc = Sa;
   V* Sn = Sb;
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
     const int r = tid + NT * i;
+    v[i] = vscale<V>(inv, x[i]);
+    vp[i] = vmake<V>(0, 0);
     if (r < D) {
-      const V v = vscale<V>(inv0, x[i]);
-      Sc[r] = v;
-      basis[r] = v;
+      Sc[r] = v[i];
+      basis[r] = v[i];
     }
   }
-  sec_sync();
-  int meff = (nrm > 0.0) ? m : 0;
+  int meff = (sec_top(nrm) > 0) ? m : 0;
   bool broke = false;
-  R bk = 0, amax = 0, bmax = 0;
-  const R tol = (R)p.bd_tol;
-  V w[RPT], vv[RPT];
+  R alpha = 0, bk = 0, ib = 0;
+  float amax = 0.f, bmax = 0.f, beta_m = 0.f;
+  const float tol = (float)p.bd_tol;
   for (int k = 0; k < meff; ++k) {
     const bool last = (k == m - 1);
-    R pa = 0, pn = 0, pq = 0;
+    sec_sync();  // v_k is in shared memory
+    sec_apply<V, NT, RPT>(p, Sc, tab, dj, v, bk, vp, w);
+    A pa = A(), pn = A(), pq = A();
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
-      const int r = tid + NT * i;
-      V h = vmake<V>(0, 0), v = vmake<V>(0, 0);
-      if (r < D) {
-        v = Sc[r];
-        h = vscale<V>(dj[i], v);
-#pragma unroll 4
-        for (int e = 0; e < ne; ++e) {
-          const unsigned en = ell[e * D + r];
-          h = vaxpy<V>(wcls[en >> kSecColBits], Sc[en & (kSecMaxD - 1)], h);
-        }
-        if (k > 0) h = vaxpy<V>(-bk, Sn[r], h);
-        pa = fma(v.x, h.x, fma(v.y, h.y, pa));
-        pn = fma(h.x, h.x, fma(h.y, h.y, pn));
-        pq = fma(v.x, v.x, fma(v.y, v.y, pq));
-      }
-      w[i] = h;
-      vv[i] = v;
+      sacc(pa, v[i].x, w[i].x);
+      sacc(pa, v[i].y, w[i].y);
+      sacc(pn, w[i].x, w[i].x);
+      sacc(pn, w[i].y, w[i].y);
+      sacc(pq, v[i].x, v[i].x);
+      sacc(pq, v[i].y, v[i].y);
     }
-    R alpha, beta;
-    R b2;
-    if constexpr (F32) {
-      const float vals[3] = {pa, pn, pq};
-      FF o[3], b2ff;
-      sec_mark(p, sm, 0);
-      sec_reduce<NT, 3>(sm, par, vals, o);
-      sec_mark(p, sm, 1);
-      SecStep st = sec_scalars(o, last, b2ff);
-      if (st.code == 2) {
+    sec_mark(p, sm, 0);
+    S o[3];
+    sec_reduce<NT>(sm, par, sclose(pa), sclose(pn), sclose(pq), o);
+    sec_mark(p, sm, 1);
+    alpha = sec_real(o[0], R());
+    S b2 = sec_b2(o);
+    sec_roots(b2, bk, ib);
+    const float af = fabsf(sec_f32(alpha));
+    const bool usual = isfinite(sec_top(o[0])) && isfinite(sec_top(o[1])) &&
+                       !sec_cancels(b2, o[1]) &&
+                       sec_f32(bk) > tol * fmaxf(1.f, fmaxf(amax, af) + bmax);
+    if (!usual) {
+      if (!isfinite(sec_top(o[0])) || !isfinite(sec_top(o[1]))) {
         if (tid == 0) {
           sec_flag(p, KG_ERR_NONFINITE);
           sec_record(sm, k, 1);
         }
         return false;
       }
-      if (tid == 0) {
-        sm.ff_a[k] = make_float2(o[0].hi, o[0].lo);
-        sm.ff_n[k] = make_float2(o[1].hi, o[1].lo);
-        sm.ff_q[k] = make_float2(o[2].hi, o[2].lo);
-      }
-      if (st.code == 1) {  // near an invariant subspace: ||w - alpha v||^2 explicitly
-        float e1[1] = {0.f};
+      if (!last && sec_cancels(b2, o[1])) {
+        // near an invariant subspace: ||w - alpha v||^2 explicitly
+        A e = A();
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
-          const V d = vaxpy<V>(-st.alpha, vv[i], w[i]);
-          e1[0] = fmaf(d.x, d.x, fmaf(d.y, d.y, e1[0]));
+          const V d = vaxpy<V>(-alpha, v[i], w[i]);
+          sacc(e, d.x, d.x);
+          sacc(e, d.y, d.y);
         }
-        FF o1[1];
-        sec_reduce<NT, 1>(sm, par, e1, o1);
-        if (tid == 0) {
-          sm.ff_e[k] = make_float2(o1[0].hi, o1[0].lo);
-          sm.ff_e_set |= 1u << k;
+        S oe[3];
+        sec_reduce<NT>(sm, par, sclose(e), A(), A(), oe);
+        b2 = oe[0];
+        sec_roots(b2, bk, ib);
+        if constexpr (FFM) {
+          if (tid == 0) {
+            sm.ff_e[k] = make_float2(b2.hi, b2.lo);
+            sm.ff_e_set |= 1u << k;
+          }
         }
-        st.b2 = __fadd_rn(o1[0].hi, o1[0].lo);
       }
-      alpha = st.alpha;
-      b2 = st.b2;
-    } else if constexpr (FFM) {
-      // float-float sums and scalars: alpha_k and b_{k+1}^2 = ||w||^2 + alpha^2 (||v||^2 - 2) in
-      // float-float, as the complex64 path forms them, but kept at float-float for the vectors
-      const FF vals[3] = {FF{pa.hi, pa.lo}, FF{pn.hi, pn.lo}, FF{pq.hi, pq.lo}};
-      FF o[3];
-      sec_mark(p, sm, 0);
-      sec_reduce<NT, 3>(sm, par, vals, o);
-      sec_mark(p, sm, 1);
-      if (!isfinite(o[0].hi) || !isfinite(o[1].hi)) {
-        if (tid == 0) {
-          sec_flag(p, KG_ERR_NONFINITE);
-          sec_record(sm, k, 1);
-        }
-        return false;
-      }
-      FF b2ff = ff_add(o[1], ff_mul(ff_mul(o[0], o[0]), ff_add(o[2], FF{-2.f, 0.f})));
-      if (tid == 0) {
-        sm.ff_a[k] = make_float2(o[0].hi, o[0].lo);
-        sm.ff_n[k] = make_float2(o[1].hi, o[1].lo);
-        sm.ff_q[k] = make_float2(o[2].hi, o[2].lo);
-      }
-      if (!last && b2ff.hi < 1e-3f * o[1].hi) {  // near an invariant subspace: ||w - alpha v||^2 explicitly
-        const R ra = R(o[0].hi, o[0].lo);
-        R e = 0;
-#pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-          const V d = vaxpy<V>(-ra, vv[i], w[i]);
-          e = fma(d.x, d.x, fma(d.y, d.y, e));
-        }
-        const FF e1[1] = {FF{e.hi, e.lo}};
-        FF o1[1];
-        sec_reduce<NT, 1>(sm, par, e1, o1);
-        if (tid == 0) {
-          sm.ff_e[k] = make_float2(o1[0].hi, o1[0].lo);
-          sm.ff_e_set |= 1u << k;
-        }
-        b2ff = o1[0];
-      }
-      alpha = R(o[0].hi, o[0].lo);
-      b2 = R(b2ff.hi, b2ff.lo);
-    } else {
-      const double vals[3] = {(double)pa, (double)pn, (double)pq};
-      double o[3];
-      sec_mark(p, sm, 0);
-      sec_reduce<NT, 3>(sm, par, vals, o);
-      sec_mark(p, sm, 1);
-      double bd = o[1] - 2.0 * o[0] * o[0] + o[0] * o[0] * o[2];
-      if (!isfinite(o[0]) || !isfinite(o[1])) {
-        if (tid == 0) {
-          sec_flag(p, KG_ERR_NONFINITE);
-          sec_record(sm, k, 1);
-        }
-        return false;
-      }
-      if (!last && bd < 1e-3 * o[1]) {
-        double e1[1] = {0.0};
-        const R ra = (R)o[0];
-#pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-          const V d = vaxpy<V>(-ra, vv[i], w[i]);
-          const double dx = (double)d.x, dy = (double)d.y;
-          e1[0] = fma(dx, dx, fma(dy, dy, e1[0]));
-        }
-        double o1[1];
-        sec_reduce<NT, 1>(sm, par, e1, o1);
-        bd = o1[0];
-      }
-      alpha = (R)o[0];
-      b2 = (R)bd;
-      if (tid == 0) sm.alpha[k] = o[0];
+      // Alg. "Lanczos": b_j > 0, with a tolerance
+      if (!last) broke = sec_f32(bk) <= tol * fmaxf(1.f, fmaxf(amax, af) + bmax);
     }
-    beta = sqrt(fmax(b2, (R)0));
+    amax = fmaxf(amax, af);
+    bmax = fmaxf(bmax, sec_f32(bk));
     if (tid == 0) {
-      sm.alpha_f[k] = (float)alpha;
-      if (last) sm.beta_m_f = (float)beta;  // b_m of the error indicator
+      sm.alpha_f[k] = sec_f32(alpha);
+      sm.beta_f[k + 1] = sec_f32(bk);
+      if constexpr (F32) {
+        sm.ff_a[k] = make_float2(o[0].hi, o[0].lo);
+        sm.ff_e[k] = make_float2(b2.hi, b2.lo);
+      } else if constexpr (FFM) {
+        sm.ff_a[k] = make_float2(o[0].hi, o[0].lo);
+        sm.ff_n[k] = make_float2(o[1].hi, o[1].lo);
+        sm.ff_q[k] = make_float2(o[2].hi, o[2].lo);
+      } else {
+        sm.alpha[k] = o[0];
+        sm.beta[k + 1] = bk;
+      }
     }
-    if (last) break;
-    amax = fmax(amax, fabs(alpha));
-    if (beta <= tol * fmax((R)1, amax + bmax)) {  // Alg. "Lanczos": b_j > 0, with a tolerance
+    if (last || broke) {
+      beta_m = sec_f32(bk);
       meff = k + 1;
-      broke = true;
       break;
     }
-    bmax = fmax(bmax, beta);
-    if (tid == 0) {
-      sm.beta_f[k + 1] = (float)beta;
-      if (!F32) sm.beta[k + 1] = (double)beta;
-    }
-    const R ib = (R)1 / beta;
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
       const int r = tid + NT * i;
+      vp[i] = v[i];
+      v[i] = vscale<V>(ib, vaxpy<V>(-alpha, v[i], w[i]));
       if (r < D) {
-        const V vn = vscale<V>(ib, vaxpy<V>(-alpha, vv[i], w[i]));
-        Sn[r] = vn;
-        basis[(size_t)(k + 1) * D + r] = vn;
+        Sn[r] = v[i];
+        basis[(size_t)(k + 1) * D + r] = v[i];
       }
     }
-    bk = beta;
     V* t = Sc;
     Sc = Sn;
     Sn = t;
-    sec_sync();
   }
   sec_mark(p, sm, 0);
-  // ---- T (FP64), exp(-i tau T) e_1 and the recombination coefficients (warp 0; with lob, warps 1
-  // and 2 form the coefficients of the two interior Gauss-Lobatto nodes at the same time)
+  // ---- T, exp(-+i dt T) e_1 and the recombination coefficients (warp 0; with lob, warps 1 and 2 form the
+  // coefficients of the two interior Gauss-Lobatto nodes at the same time)
   if (tid < 32) {
     __syncwarp();  // thread 0's stores of the step sums are visible to the warp
-    const int k = tid;
-    if constexpr (F32 || FFM) {
+    if constexpr (FFM) {  // T in FP64 from the float-float sums, lane k for step k
+      const int k = tid;
       if (k < meff) {
         const double al = ff_to_double(FF{sm.ff_a[k].x, sm.ff_a[k].y});
         double b2;
@@ -639,99 +750,48 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
           b2 = nn - 2.0 * al * al + al * al * q;
         }
         sm.alpha[k] = al;
-        if (k + 1 < meff) sm.beta[k + 1] = sqrt(fmax(b2, 0.0));
+        if (k + 1 < meff) sm.beta[k + 1] = ::sqrt(::fmax(b2, 0.0));
       }
       __syncwarp();
     }
   }
   if (lob) sec_sync();  // T is read by warps 1 and 2 as well
-  if (tid < (lob ? 96 : 32)) {
-    const int w = tid >> 5, k = tid & 31;
-    // slice end, or the interior nodes s_a, s_b = (1 -+ 1/sqrt 5) dt/2: forward exp(-i s H) psi_{j-1},
-    // backward exp(+i (dt - s) H) chi_j
-    double tw = tau;
-    if (w > 0) {
-      const double sn = 0.5 * p.dt * (1.0 + (w == 1 ? -1.0 : 1.0) / sqrt(5.0));
-      tw = (lob == 1) ? sn : -(p.dt - sn);
-    }
-    double cr = 0.0, ci = 0.0;
-    float tnorm = 0.f;
-    const double etol = F32 ? 1e-13 : 1e-18;
-    // The exponential takes ceil(||tau T|| / 4) sub-steps: refuse a T whose Gershgorin bound is not a
-    // finite, sane number (it would come from corrupted coefficients) instead of looping on it.
-    float row = 0.f;
-    if (k < meff)
-      row = fabsf((float)tw) * (fabsf(sm.alpha_f[k]) + (k >= 1 ? sm.beta_f[k] : 0.f) +
-                                (k + 1 < meff ? sm.beta_f[k + 1] : 0.f));
-    row = (row == row) ? row : 3.0e38f;  // NaN -> refused
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) row = fmaxf(row, __shfl_xor_sync(0xffffffffu, row, o));
-    const bool sane = row <= 1.0e5f;
-    if (tid == 0 && !sane) {
-      sec_flag(p, KG_ERR_NONFINITE);
-      sec_record(sm, -1, 3);
-      sm.abort = 1;
-    }
-    if (meff > 0 && sane) {
-      if constexpr (F32)  // float-float: FP64 instructions are slow on this GPU (see tridiag_expv_e1_ff)
-        tridiag_expv_e1_ff(sm.alpha, sm.beta, sm.alpha_f, sm.beta_f, meff, tw, (float)tw, etol, cr, ci, tnorm);
-      else
-        tridiag_expv_e1(sm.alpha, sm.beta, sm.alpha_f, sm.beta_f, meff, tw, (float)tw, etol, cr, ci, tnorm);
-    }
-    if (k < meff) {
-      sm.coef_d[w][0][k] = cr * nrm;
-      sm.coef_d[w][1][k] = ci * nrm;
-      sm.coef_f[w][0][k] = (float)(cr * nrm);
-      sm.coef_f[w][1][k] = (float)(ci * nrm);
-    }
-    if (w == 0 && k == meff - 1) {  // a-posteriori indicator ||x|| b_m |c_{m-1}| (0 after a breakdown)
-      double cm = nrm * sqrt(cr * cr + ci * ci);
-      if (cm == 0.0 && !broke) {
-        cm = nrm;
-        for (int i = 1; i < meff; ++i) cm *= (double)tnorm / (double)i;
-      }
-      const double err = broke ? 0.0 : (double)sm.beta_m_f * cm;
-      sm.err_max = fmax(sm.err_max, err);
-      if (broke) sm.breakdowns += 1;
-    }
-    __syncwarp();
-    if (tid == 0) {
-      sm.ff_e_set = 0u;
-      // time limit of one pulse: a pulse that runs past it ends with KG_ERR_TIMEOUT
-      if (sm.abort == 0 && (long long)(globaltimer_ns() - sm.t_start) > p.time_limit_ns) {
-        sec_flag(p, KG_ERR_TIMEOUT);
-        sec_record(sm, -1, 4);
-        sm.abort = 1;
-      }
-    }
-  }
+  if (tid < (lob ? 96 : 32)) sec_coefficients<V>(p, sm, tid >> 5, back, meff, broke, beta_m, nrm, fact);
   sec_sync();
   if (sm.abort) return false;
   sec_mark(p, sm, 4);
-  // ---- recombination x = sum_k coef_k v_k (own rows), fused ||x||^2 and the overlap
-  // the own rows' basis values come from L2: KB basis vectors' loads are issued together
-  constexpr int KB = F32 ? 4 : 2;
+  // ---- recombination x = sum_k coef_k v_k (own rows), the small terms first; fused ||x||^2 and overlap.
+  // The own rows' basis values come from L2: KB basis vectors' loads are issued together.
+  constexpr int KB = (F32 ? 16 : 8) / RPT < 2 ? 2 : (F32 ? 16 : 8) / RPT;
   V y[RPT];
 #pragma unroll
   for (int i = 0; i < RPT; ++i) y[i] = vmake<V>(0, 0);
-  for (int k0 = 0; k0 < meff; k0 += KB) {
+  for (int k0 = meff - 1; k0 >= 0; k0 -= KB) {
     V q[KB][RPT];
 #pragma unroll
     for (int u = 0; u < KB; ++u)
 #pragma unroll
       for (int i = 0; i < RPT; ++i) {
         const int r = tid + NT * i;
-        q[u][i] = (k0 + u < meff && r < D) ? basis[(size_t)(k0 + u) * D + r] : vmake<V>(0, 0);
+        q[u][i] = (k0 >= u && r < D) ? basis[(size_t)(k0 - u) * D + r] : vmake<V>(0, 0);
       }
 #pragma unroll
     for (int u = 0; u < KB; ++u) {
-      const int k = k0 + u;
-      const R a = (k < meff) ? (F32 ? (R)sm.coef_f[0][0][k] : (R)sm.coef_d[0][0][k]) : (R)0;
-      const R b = (k < meff) ? (F32 ? (R)sm.coef_f[0][1][k] : (R)sm.coef_d[0][1][k]) : (R)0;
+      if (k0 >= u) {
+        const int k = k0 - u;
+        const R a = F32 ? (R)sm.coef_f[0][0][k] : (R)sm.coef_d[0][0][k];
+        const R b = F32 ? (R)sm.coef_f[0][1][k] : (R)sm.coef_d[0][1][k];
 #pragma unroll
-      for (int i = 0; i < RPT; ++i) {
-        y[i].x = fma(a, q[u][i].x, fma(-b, q[u][i].y, y[i].x));
-        y[i].y = fma(a, q[u][i].y, fma(b, q[u][i].x, y[i].y));
+        for (int i = 0; i < RPT; ++i) {
+          if constexpr (FFM) {
+            const FF nb = ff_of(-b), fa = ff_of(a), fb = ff_of(b), one{1.f, 0.f};
+            y[i] = V{ffr_of(ff_dot3(fa, ff_of(q[u][i].x), nb, ff_of(q[u][i].y), one, ff_of(y[i].x))),
+                     ffr_of(ff_dot3(fa, ff_of(q[u][i].y), fb, ff_of(q[u][i].x), one, ff_of(y[i].y)))};
+          } else {
+            y[i].x = fma(a, q[u][i].x, fma(-b, q[u][i].y, y[i].x));
+            y[i].y = fma(a, q[u][i].y, fma(b, q[u][i].x, y[i].y));
+          }
+        }
       }
     }
   }
@@ -742,9 +802,9 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
     if (r < D) {
       if (dst) dst[r] = y[i];
       pn = fma(y[i].x, y[i].x, fma(y[i].y, y[i].y, pn));
-      if (extra == 1) {
+      if (back) {
         const V o = other[r];
-        pg = fma(hh[i], y[i].x * o.y - y[i].y * o.x, pg);  // Im(conj(y) Hc o), Hc diagonal
+        pg = fma(sec_hc<R>(p, sm, __ldg(p.states + r)), y[i].x * o.y - y[i].y * o.x, pg);  // Im(conj(y) Hc o), Hc diagonal
       }
     }
     x[i] = y[i];
@@ -752,14 +812,23 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
   // ---- Taylor hierarchy (App. B, Eq. gradp), backward slice j (sec_taylor)
   R pt = 0;
   if constexpr (!FFM) {  // the float-float path offers the centred and zeroth-order gradients
-    if (taylor > 0) pt = sec_taylor<V, NT, RPT>(p, sm, Sa, Sb, ell, basis, uj, meff, nin, taylor, psi_end);
+    if (taylor > 0) {
+      R nx;
+      if constexpr (F32) nx = __fadd_rn(nrm.hi, nrm.lo);
+      else nx = nrm;
+      pt = sec_taylor<V, NT, RPT>(p, sm, Sa, Sb, tab, basis, uj, meff, nx, taylor, psi_end);
+    }
     if (lob > 0) pt = sec_interior<V, NT, RPT>(p, sm, basis, meff, lob, tint_io);
   }
+  sec_mark(p, sm, 5);
   if constexpr (F32) {
-    const float vals[3] = {pn, pg, pt};
     FF o[3];
-    sec_mark(p, sm, 5);
-    sec_reduce<NT, 3>(sm, par, vals, o);
+    sec_reduce<NT>(sm, par, pn, pg, pt, o);
+    nrm = ff_sqrt(o[0]);
+    const float n = __fadd_rn(nrm.hi, nrm.lo);
+    inv = (n > 0.f) ? __frcp_rn(n) : 0.f;
+    ex = o[1];
+    tay = o[2];
     if (!isfinite(o[0].hi)) {
       if (tid == 0) {
         sec_flag(p, KG_ERR_NONFINITE);
@@ -767,25 +836,9 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
       }
       return false;
     }
-    // FP64 is slow on this GPU: thread 0 forms ||x|| and 1/||x|| for everyone (the next write of
-    // these fields comes a whole slice later, after many barriers)
-    if (tid == 0) {
-      const double n = sqrt(fmax(ff_to_double(o[0]), 0.0));
-      sm.nrm_d = n;
-      sm.inv_f = (n > 0.0) ? (float)(1.0 / n) : 0.f;
-      sm.ex_d = (extra == 1) ? ff_to_double(o[1]) : 0.0;
-      sm.tay_d = (taylor > 0 || lob == 2) ? ff_to_double(o[2]) : 0.0;  // Taylor or interior overlaps
-    }
-    sec_sync();
-    nrm = sm.nrm_d;
-    inv = (R)sm.inv_f;
-    ex = sm.ex_d;
-    if (tay) *tay = sm.tay_d;
   } else {
-    const double vals[3] = {(double)pn, (double)pg, (double)pt};
     double o[3];
-    sec_mark(p, sm, 5);
-    sec_reduce<NT, 3>(sm, par, vals, o);
+    sec_reduce<NT>(sm, par, (double)pn, (double)pg, (double)pt, o);
     if (!isfinite(o[0])) {
       if (tid == 0) {
         sec_flag(p, KG_ERR_NONFINITE);
@@ -793,19 +846,14 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
       }
       return false;
     }
-    nrm = sqrt(fmax(o[0], 0.0));
-    inv = (nrm > 0.0) ? (R)(1.0 / nrm) : (R)0;
+    double id;
+    sec_roots(o[0], nrm, id);
+    inv = (R)id;
     ex = o[1];
-    if (tay) *tay = o[2];
+    tay = o[2];
   }
   sec_mark(p, sm, 1);
   return true;
-}
-
-// FP64 sums of the own rows of the pulse's first and last states (once per evaluation).
-template <int NT, int NV>
-__device__ __forceinline__ void sec_reduce_fp64(SecSmem& sm, int& par, const double (&vals)[NV], double (&out)[NV]) {
-  sec_reduce<NT, NV>(sm, par, vals, out);
 }
 
 // Thread 0: F = NaN and the failure record of pulse b, abandoned in slice j (negative: backward).
@@ -817,33 +865,36 @@ __device__ __forceinline__ void sec_abandon(const SectorParams& p, const SecSmem
   sc[7] = (double)sm.fail_check;
 }
 
+__device__ __forceinline__ void sec_norm(double n2, FF& n, float& inv) {
+  const double d = ::sqrt(n2);
+  n = ff_from_double(d);
+  inv = (d > 0.0) ? (float)(1.0 / d) : 0.f;
+}
+template <class R>
+__device__ __forceinline__ void sec_norm(double n2, double& n, R& inv) {
+  n = ::sqrt(n2);
+  inv = (n > 0.0) ? (R)(1.0 / n) : (R)0;
+}
+__device__ __forceinline__ double sec_double(FF a) { return ff_to_double(a); }
+__device__ __forceinline__ double sec_double(double a) { return a; }
+
 template <class V, int NT, int RPT>
-__device__ __forceinline__ void sec_eval(const SectorParams& p, int b, SecSmem& sm, V* S0, V* S1,
-                                      const unsigned short* ell) {
+__device__ __forceinline__ void sec_eval(const SectorParams& p, int b, SecSmem& sm, V* S0, V* S1, const unsigned* tab,
+                                         float2 fact) {
   using R = typename VecTraits<V>::R;
-  const int tid = threadIdx.x, D = p.D, N = p.N;
-  V* traj = (V*)p.traj + (size_t)blockIdx.x * (size_t)(N + 1) * D;
+  using N = typename SecPrec<V>::N;
+  constexpr bool F32 = sizeof(R) == 4;
+  const int tid = threadIdx.x, D = p.D, NS = p.N;
+  V* traj = (V*)p.traj + (size_t)blockIdx.x * (size_t)(NS + 1) * D;
   V* basis = (V*)p.basis + (size_t)blockIdx.x * (size_t)p.m * D;
-  double* G = p.G + (size_t)blockIdx.x * (N + 1);
-  const double* u = p.u + (size_t)b * N;
+  double* G = p.G + (size_t)blockIdx.x * (NS + 1);
+  double* gb = p.grad ? p.grad + (size_t)b * NS : nullptr;
+  const double* u = p.u + (size_t)b * NS;
   const double2* psi0 = reinterpret_cast<const double2*>(p.psi0);
   const double2* tgt = reinterpret_cast<const double2*>(p.target);
-  R dd[RPT], hh[RPT];
-  const int npc = __popc(p.hc_mask);
-#pragma unroll
-  for (int i = 0; i < RPT; ++i) {
-    const int r = tid + NT * i;
-    dd[i] = 0;
-    hh[i] = 0;
-    if (r < D) {
-      const unsigned s = p.states[r];
-      dd[i] = (R)(p.qz * (double)(p.L1 - 2 * __popc((s ^ (s >> 1)) & p.maskL1)));
-      hh[i] = (R)(0.5 * p.hc_amp * (double)(npc - 2 * __popc(s & p.hc_mask)));
-    }
-  }
   sec_sync();  // the previous pulse (possibly abandoned after a non-finite value) is done with shared memory
   if (tid == 0) {
-    sm.err_max = 0.0;
+    sm.err_max = 0.f;
     sm.breakdowns = 0;
     sm.ff_e_set = 0u;
     sm.abort = 0;
@@ -854,9 +905,10 @@ __device__ __forceinline__ void sec_eval(const SectorParams& p, int b, SecSmem& 
   }
   int par = 0;
   V x[RPT];
-  double nrm;
+  N nrm;
+  R inv;
   {  // psi_0 into the trajectory and its norm (FP64)
-    double acc[1] = {0.0};
+    double acc = 0.0, o[3];
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
       const int r = tid + NT * i;
@@ -865,95 +917,102 @@ __device__ __forceinline__ void sec_eval(const SectorParams& p, int b, SecSmem& 
         const double2 q = psi0[r];
         x[i] = vmake<V>((R)q.x, (R)q.y);
         traj[r] = x[i];
-        acc[0] = fma((double)x[i].x, (double)x[i].x, fma((double)x[i].y, (double)x[i].y, acc[0]));
+        acc = ::fma((double)x[i].x, (double)x[i].x, ::fma((double)x[i].y, (double)x[i].y, acc));
       }
     }
-    double o[1];
-    sec_reduce_fp64<NT, 1>(sm, par, acc, o);
-    nrm = sqrt(o[0]);
+    sec_reduce<NT>(sm, par, acc, 0.0, 0.0, o);
+    sec_norm(o[0], nrm, inv);
   }
-  R inv = (nrm > 0.0) ? (R)(1.0 / nrm) : (R)0;
-  double ex = 0.0;
   sec_mark(p, sm, 6);
   const bool exact = (p.grad_mode == KG_GRAD_EXACT);
-  V* tint = exact ? (V*)p.tint + (size_t)blockIdx.x * 2 * (size_t)N * D : nullptr;
-  for (int j = 1; j <= N; ++j) {
-    if (!sec_slice<V, NT, RPT>(p, sm, par, S0, S1, ell, basis, dd, hh, u[j - 1], p.dt, x, nrm, inv, 0, nullptr,
-                               traj + (size_t)j * D, ex, 0, nullptr, nullptr, exact ? 1 : 0,
-                               exact ? tint + (size_t)2 * (j - 1) * D : nullptr)) {
-      if (tid == 0) sec_abandon(p, sm, b, j);
+  const int taylor = (p.grad_mode == KG_GRAD_TAYLOR1) ? 1 : (p.grad_mode == KG_GRAD_TAYLOR2) ? 2 : 0;
+  V* tint = exact ? (V*)p.tint + (size_t)blockIdx.x * 2 * (size_t)NS * D : nullptr;
+  // Forward slices j = 1..N, then the co-state's j = N..1: one loop, one copy of the slice's code.
+  double br = 0.0, bi = 0.0, nfin = 0.0;
+  bool back = false;
+  for (int j = 1;;) {
+    N ex, tay;
+    if (!sec_slice<V, NT, RPT>(p, sm, par, S0, S1, tab, basis, u[j - 1], back, x, nrm, inv, traj + (size_t)(j - 1) * D,
+                               back ? nullptr : traj + (size_t)j * D, ex, back ? taylor : 0, traj + (size_t)j * D, tay,
+                               !exact ? 0 : back ? 2 : 1, exact ? tint + (size_t)2 * (j - 1) * D : nullptr, fact)) {
+      if (tid == 0) sec_abandon(p, sm, b, back ? -j : j);
       return;
     }
-  }
-  // beta = <f|psi_N> (FP64), F = |beta|^2
-  double br, bi, nfin = nrm;
-  {
-    double acc[2] = {0.0, 0.0};
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      const int r = tid + NT * i;
-      if (r < D) {
-        const double2 f = tgt[r];
-        const double xr = (double)x[i].x, xi = (double)x[i].y;
-        acc[0] = fma(f.x, xr, fma(f.y, xi, acc[0]));   // Re(conj(f) x)
-        acc[1] = fma(f.x, xi, fma(-f.y, xr, acc[1]));  // Im(conj(f) x)
-      }
-    }
-    double o[2];
-    sec_reduce_fp64<NT, 2>(sm, par, acc, o);
-    br = o[0];
-    bi = o[1];
-  }
-  if (p.grad_mode != KG_GRAD_NONE) {
-    const int taylor = (p.grad_mode == KG_GRAD_TAYLOR1) ? 1 : (p.grad_mode == KG_GRAD_TAYLOR2) ? 2 : 0;
-    // chi_N = beta f; G_N = 2 dt Im <chi_N|Hc|psi_N>
-    double acc[2] = {0.0, 0.0};
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      const int r = tid + NT * i;
-      V c = vmake<V>(0, 0);
-      if (r < D) {
-        const double2 f = tgt[r];
-        c = vmake<V>((R)(br * f.x - bi * f.y), (R)(br * f.y + bi * f.x));
-        const double cr = (double)c.x, ci = (double)c.y;
-        acc[0] = fma(cr, cr, fma(ci, ci, acc[0]));
-        acc[1] = fma((double)hh[i], cr * (double)x[i].y - ci * (double)x[i].x, acc[1]);
-      }
-      x[i] = c;
-    }
-    double o[2];
-    sec_reduce_fp64<NT, 2>(sm, par, acc, o);
-    nrm = sqrt(o[0]);
-    inv = (nrm > 0.0) ? (R)(1.0 / nrm) : (R)0;
-    if (tid == 0) G[N] = 2.0 * p.dt * o[1];
-    sec_mark(p, sm, 6);
-    for (int j = N; j >= 1; --j) {
-      // chi_{j-1} = exp(+i dt H_j) chi_j, fused G_{j-1} = 2 dt Im <chi_{j-1}|Hc|psi_{j-1}>
-      double tay = 0.0;
-      if (!sec_slice<V, NT, RPT>(p, sm, par, S0, S1, ell, basis, dd, hh, u[j - 1], -p.dt, x, nrm, inv, 1,
-                                 traj + (size_t)(j - 1) * D, nullptr, ex, taylor, traj + (size_t)j * D, &tay,
-                                 exact ? 2 : 0, exact ? tint + (size_t)2 * (j - 1) * D : nullptr)) {
-        if (tid == 0) sec_abandon(p, sm, b, -j);
-        return;
-      }
+    if (back) {
       if (tid == 0) {
-        G[j - 1] = 2.0 * p.dt * ex;
-        if (taylor) G[j] = 2.0 * p.dt * tay;  // slice j's Taylor-hierarchy value replaces G_j
-        if (exact)  // 4-point Gauss-Lobatto over slice j: weights 1/12, 5/12, 5/12, 1/12
-          p.grad[(size_t)b * N + (j - 1)] = (G[j - 1] + G[j]) / 12.0 + (5.0 / 12.0) * 2.0 * p.dt * tay;
+        G[j - 1] = sec_pack(ex);
+        if (taylor) G[j] = sec_pack(tay);     // slice j's Taylor-hierarchy value replaces G_j
+        if (exact) gb[j - 1] = sec_pack(tay);  // the interior nodes' share, weighted below
+      }
+      if (--j == 0) break;
+      continue;
+    }
+    if (j < NS) {
+      ++j;
+      continue;
+    }
+    // ---- beta = <f|psi_N> (FP64), F = |beta|^2
+    nfin = sec_double(nrm);
+    {
+      double a0 = 0.0, a1 = 0.0, o[3];
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        const int r = tid + NT * i;
+        if (r < D) {
+          const double2 f = tgt[r];
+          const double xr = (double)x[i].x, xi = (double)x[i].y;
+          a0 = ::fma(f.x, xr, ::fma(f.y, xi, a0));   // Re(conj(f) x)
+          a1 = ::fma(f.x, xi, ::fma(-f.y, xr, a1));  // Im(conj(f) x)
+        }
+      }
+      sec_reduce<NT>(sm, par, a0, a1, 0.0, o);
+      br = o[0];
+      bi = o[1];
+    }
+    if (p.grad_mode == KG_GRAD_NONE) break;
+    {  // chi_N = beta f; G_N = 2 dt Im <chi_N|Hc|psi_N>
+      double a0 = 0.0, a1 = 0.0, o[3];
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        const int r = tid + NT * i;
+        V c = vmake<V>(0, 0);
+        if (r < D) {
+          const double2 f = tgt[r];
+          c = vmake<V>((R)(br * f.x - bi * f.y), (R)(br * f.y + bi * f.x));
+          const double cr = (double)c.x, ci = (double)c.y;
+          a0 = ::fma(cr, cr, ::fma(ci, ci, a0));
+          a1 = ::fma((double)sec_hc<R>(p, sm, __ldg(p.states + r)), cr * (double)x[i].y - ci * (double)x[i].x, a1);
+        }
+        x[i] = c;
+      }
+      sec_reduce<NT>(sm, par, a0, a1, 0.0, o);
+      sec_norm(o[0], nrm, inv);
+      if constexpr (F32) {
+        if (tid == 0) G[NS] = sec_pack(ff_from_double(o[1]));
+      } else {
+        if (tid == 0) G[NS] = o[1];
       }
     }
+    sec_mark(p, sm, 6);
+    back = true;
+  }
+  if (back) {
     sec_sync();  // G complete (written by thread 0)
-    double* gb = p.grad + (size_t)b * N;
-    for (int j = tid; j < N && !exact; j += NT)
-      gb[j] = (p.grad_mode == KG_GRAD_CENTERED) ? 0.5 * (G[j] + G[j + 1]) : G[j + 1];  // zeroth, Taylor
+    const double f = 2.0 * p.dt;
+    for (int j = tid; j < NS; j += NT) {
+      const double gl = f * sec_unpack<F32>(G[j]), gr = f * sec_unpack<F32>(G[j + 1]);
+      if (exact)  // 4-point Gauss-Lobatto over slice j: weights 1/12, 5/12, 5/12, 1/12
+        gb[j] = (gl + gr) / 12.0 + (5.0 / 12.0) * f * sec_unpack<F32>(gb[j]);
+      else
+        gb[j] = (p.grad_mode == KG_GRAD_CENTERED) ? 0.5 * (gl + gr) : gr;  // zeroth, Taylor
+    }
   }
   if (tid == 0) {
     p.fid[b] = br * br + bi * bi;
     double* sc = p.scal + (size_t)b * kScCount;
     sc[kScBetaRe] = br;
     sc[kScBetaIm] = bi;
-    sc[kScErrMax] = sm.err_max;
+    sc[kScErrMax] = (double)sm.err_max;
     sc[kScNormFinal] = nfin;
     sc[kScBreakdowns] = (double)sm.breakdowns;
     sc[5] = sc[6] = sc[7] = 0.0;
@@ -973,25 +1032,37 @@ constexpr int sec_min_blocks() {
                                                     : (NT <= 256) ? 2 : 1;
 }
 
+// Elements of a vector in shared memory: D, the zero element behind it, 16-element steps.
+__host__ __device__ constexpr int sec_padded(int D) { return (D + 16) & ~15; }
+
 template <class V, int NT, int RPT>
 __global__ void __launch_bounds__(NT, (sec_min_blocks<V, NT>())) kg_sector_kernel(const __grid_constant__ SectorParams p) {
   extern __shared__ __align__(16) unsigned char sec_dyn[];
   __shared__ SecSmem sm;
-  const int Dp = (p.D + 15) & ~15;
+  const int Dp = sec_padded(p.D);
   V* S0 = reinterpret_cast<V*>(sec_dyn);
   V* S1 = S0 + Dp;
-  unsigned short* ell = reinterpret_cast<unsigned short*>(S1 + Dp);
-  for (int i = threadIdx.x; i < p.ell * p.D; i += NT) ell[i] = p.ell_g[i];
-  if (threadIdx.x < kSecClasses) {
-    sm.wcls_f[threadIdx.x] = (float)p.wcls[threadIdx.x];
-    sm.wcls_d[threadIdx.x] = p.wcls[threadIdx.x];
-    const float wh = (float)p.wcls[threadIdx.x];
-    sm.wcls_ff[threadIdx.x] = make_float2(wh, (float)(p.wcls[threadIdx.x] - (double)wh));
+  unsigned* tab = reinterpret_cast<unsigned*>(S1 + Dp);
+  for (int i = threadIdx.x; i < p.words; i += NT) tab[i] = p.tab_g[i];
+  if (threadIdx.x == 0) {
+    S0[p.D] = S1[p.D] = vmake<V>(0, 0);  // what the tables' padding points at
+    const double sa = 0.5 * p.dt * (1.0 - 1.0 / ::sqrt(5.0));
+    const double w[5] = {p.qz, 0.5 * p.hc_amp, p.dt, sa, p.dt - sa};
+    for (int i = 0; i < 5; ++i) {
+      const FF f = ff_from_double(w[i]);
+      if (i < 2) {
+        sm.diag_d[i] = w[i];
+        sm.diag_ff[i] = make_float2(f.hi, f.lo);
+      } else {
+        sm.tau_ff[i - 2] = make_float2(f.hi, f.lo);
+      }
+    }
   }
   if (threadIdx.x < 8) sm.prof_acc[threadIdx.x] = 0;
   const long long t0 = clock64();
+  const float2 fact = kInvFactFF[min((int)threadIdx.x & 31, 29)];
   sec_sync();
-  for (int b = blockIdx.x; b < p.B; b += gridDim.x) sec_eval<V, NT, RPT>(p, b, sm, S0, S1, ell);
+  for (int b = blockIdx.x; b < p.B; b += gridDim.x) sec_eval<V, NT, RPT>(p, b, sm, S0, S1, tab, fact);
   if (p.prof && blockIdx.x == 0 && threadIdx.x == 0) {
     for (int i = 0; i < 7; ++i) p.prof[i] = sm.prof_acc[i];
     p.prof[7] = clock64() - t0;
@@ -1009,43 +1080,51 @@ static SecKernel sec_choice() {
   return {reinterpret_cast<const void*>(&kg_sector_kernel<V, NT, RPT>), NT};
 }
 
+// 128 threads: as many rows a thread as D needs (a row beyond D costs its FP64 or float-float work).
+template <class V>
+static SecKernel sec_small(int D) {
+  if (D <= 128) return sec_choice<V, 128, 1>();
+  if (D <= 256) return sec_choice<V, 128, 2>();
+  return (D <= 512) ? sec_choice<V, 128, 4>() : SecKernel{nullptr, 0};
+}
+
 // Threads and rows per thread by dimension: the smallest block that covers D with <= 8 rows per
 // thread (10 for complex64 up to 2560, which keeps two CTAs on an SM); or, with nt = 128, 256 or
 // 512 threads, that block with the fewest rows per thread that covers D (nt.threads == 0: none).
 static SecKernel sec_pick(int prec, int D, int nt = 0) {
   if (prec == KG_PREC_FF) {  // the complex128 path's shapes (16-byte amplitudes); 512 x 5 up to
                              // D = 2560 holds its arrays in registers (512 x 8 spills)
-    if (nt == 128) return (D <= 512) ? sec_choice<FFC, 128, 4>() : SecKernel{nullptr, 0};
+    if (nt == 128) return sec_small<FFC>(D);
     if (nt == 256) return (D <= 1024) ? sec_choice<FFC, 256, 4>()
                                       : (D <= 2048) ? sec_choice<FFC, 256, 8>() : SecKernel{nullptr, 0};
     if (nt == 512)
       return (D <= 2560) ? sec_choice<FFC, 512, 5>() : (D <= 4096) ? sec_choice<FFC, 512, 8>() : SecKernel{nullptr, 0};
-    if (D <= 512) return sec_choice<FFC, 128, 4>();
+    if (D <= 512) return sec_small<FFC>(D);
     if (D <= 1024) return sec_choice<FFC, 256, 4>();
     if (D <= 2048) return sec_choice<FFC, 256, 8>();
     if (D <= 2560) return sec_choice<FFC, 512, 5>();
     return sec_choice<FFC, 512, 8>();
   }
   if (prec == KG_PREC_C128) {  // 512 x 5 up to D = 2560 spills less than 512 x 8
-    if (nt == 128) return (D <= 512) ? sec_choice<double2, 128, 4>() : SecKernel{nullptr, 0};
+    if (nt == 128) return sec_small<double2>(D);
     if (nt == 256) return (D <= 1024) ? sec_choice<double2, 256, 4>()
                                       : (D <= 2048) ? sec_choice<double2, 256, 8>() : SecKernel{nullptr, 0};
     if (nt == 512)
       return (D <= 2560) ? sec_choice<double2, 512, 5>()
                          : (D <= 4096) ? sec_choice<double2, 512, 8>() : SecKernel{nullptr, 0};
-    if (D <= 512) return sec_choice<double2, 128, 4>();
+    if (D <= 512) return sec_small<double2>(D);
     if (D <= 1024) return sec_choice<double2, 256, 4>();
     if (D <= 2048) return sec_choice<double2, 256, 8>();
     if (D <= 2560) return sec_choice<double2, 512, 5>();
     return sec_choice<double2, 512, 8>();
   }
-  if (nt == 128) return (D <= 512) ? sec_choice<float2, 128, 4>() : SecKernel{nullptr, 0};
+  if (nt == 128) return sec_small<float2>(D);
   if (nt == 256)
     return (D <= 1024) ? sec_choice<float2, 256, 4>()
                        : (D <= 2048) ? sec_choice<float2, 256, 8>()
                                      : (D <= 2560) ? sec_choice<float2, 256, 10>() : SecKernel{nullptr, 0};
   if (nt == 512) return (D <= 4096) ? sec_choice<float2, 512, 8>() : SecKernel{nullptr, 0};
-  if (D <= 512) return sec_choice<float2, 128, 4>();
+  if (D <= 512) return sec_small<float2>(D);
   if (D <= 1024) return sec_choice<float2, 256, 4>();
   if (D <= 2048) return sec_choice<float2, 256, 8>();
   if (D <= 2560) return sec_choice<float2, 256, 10>();  // two CTAs per SM (registers)
@@ -1054,16 +1133,15 @@ static SecKernel sec_pick(int prec, int D, int nt = 0) {
 
 constexpr int kSecMaxRows = 4096;  // 512 threads x 8 rows
 
-size_t sector_smem_bytes(int prec, int D, int ell) {
+size_t sector_smem_bytes(int prec, int D, int words) {
   const size_t vb = (prec == KG_PREC_C64_F64REC) ? 8 : 16;
-  const size_t Dp = ((size_t)D + 15) & ~(size_t)15;
-  return 2 * Dp * vb + (size_t)ell * D * 2;
+  return 2 * (size_t)sec_padded(D) * vb + (size_t)words * 4;
 }
 
-cudaError_t sector_kernel_max_ctas(int prec, int D, int ell, int nt, int* out) {
+cudaError_t sector_kernel_max_ctas(int prec, int D, int words, int nt, int* out) {
   const SecKernel k = sec_pick(prec, D, nt);
   if (!k.fn) return cudaErrorInvalidValue;
-  const size_t smem = sector_smem_bytes(prec, D, ell);
+  const size_t smem = sector_smem_bytes(prec, D, words);
   cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per = 0;
@@ -1080,7 +1158,7 @@ bool sector_shape_ok(int prec, int D, int nt) { return sec_pick(prec, D, nt).fn 
 cudaError_t launch_sector_kernel(int prec, const SectorParams& p, int ctas, int nt, cudaStream_t stream) {
   const SecKernel k = sec_pick(prec, p.D, nt);
   if (!k.fn) return cudaErrorInvalidValue;
-  const size_t smem = sector_smem_bytes(prec, p.D, p.ell);
+  const size_t smem = sector_smem_bytes(prec, p.D, p.words);
   cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<SectorParams*>(&p)};
@@ -1096,8 +1174,10 @@ using kg::host_fail;
 
 struct SectorBasis {
   std::vector<uint64_t> states;       // s_r, ascending
-  std::vector<unsigned short> ell;    // [ell][D]
-  int D = 0, ell_width = 0;
+  std::vector<unsigned> tab;          // list A, the 32-row groups' meta words, list B (see sec_apply)
+  int D = 0, bonds = 0;               // bonds: most antiparallel bonds of a row
+  int na2 = 0, rows = 0, groups = 0;
+  int words() const { return (int)tab.size(); }
 };
 
 uint64_t mirror_bits(uint64_t s, int L) {
@@ -1187,41 +1267,68 @@ bool build_basis(const kg_sector* s, size_t limit, bool want_ell, SectorBasis& o
     return false;
   }
   if (!want_ell) return true;
-  // per row: one entry per antiparallel bond of s_r whose image has a basis vector
-  std::vector<std::vector<unsigned short>> rows(out.D);
-  int width = 0;
+  // per row: one column per antiparallel bond of s_r whose image has a basis vector, on the list of its weight
+  std::vector<std::vector<int>> la(out.D), lb(out.D);
+  size_t wide = 0;
   for (int r = 0; r < out.D; ++r) {
     const uint64_t st = out.states[r];
     const int nr = orb[st].n;
+    int bonds = 0;
     for (int b = 0; b + 1 < L; ++b) {
       if (((st >> b) & 1ull) == ((st >> (b + 1)) & 1ull)) continue;
       const OrbitInfo& o = orb.at(st ^ (3ull << b));
       if (o.row < 0) continue;
-      int cls;
-      if (P == 1) cls = (nr == o.n) ? kg::kSecW1 : (nr == 2 ? kg::kSecWSqrt2 : kg::kSecWInvSqrt2);
-      else if (P == -1) cls = (o.phi > 0) ? kg::kSecW1 : kg::kSecWMinus1;
-      else cls = kg::kSecW1;
-      rows[r].push_back((unsigned short)((cls << kg::kSecColBits) | o.row));
+      ++bonds;
+      if (P == 1 && nr != o.n) {  // factor sqrt(n_r'/n_r): sqrt 2 = 2 / sqrt 2, or 1 / sqrt 2
+        lb[r].push_back(o.row);
+        if (nr == 2) lb[r].push_back(o.row);
+      } else if (P == -1 && o.phi < 0) {
+        lb[r].push_back(o.row);
+      } else {
+        la[r].push_back(o.row);
+      }
     }
-    width = std::max(width, (int)rows[r].size());
+    out.bonds = std::max(out.bonds, bonds);
+    wide = std::max(wide, la[r].size());
   }
-  out.ell_width = width;
-  out.ell.assign((size_t)width * out.D, 0);
-  for (int r = 0; r < out.D; ++r)
-    for (int e = 0; e < width; ++e)
-      out.ell[(size_t)e * out.D + r] = (e < (int)rows[r].size())
-                                           ? rows[r][e]
-                                           : (unsigned short)((kg::kSecWZero << kg::kSecColBits) | r);
+  const int D = out.D;
+  auto word = [&](const std::vector<int>& l, size_t q) {  // entries 2q, 2q + 1; padding: the zero element D
+    const unsigned c0 = (2 * q < l.size()) ? (unsigned)l[2 * q] : (unsigned)D;
+    const unsigned c1 = (2 * q + 1 < l.size()) ? (unsigned)l[2 * q + 1] : (unsigned)D;
+    return c0 | (c1 << 16);
+  };
+  out.na2 = (int)((wide + 1) / 2);
+  out.rows = D + 1;  // row D: all padding, for the threads without a row of their own
+  out.groups = (D + 31) / 32;
+  out.tab.clear();
+  const std::vector<int> none;
+  for (int q = 0; q < out.na2; ++q)
+    for (int r = 0; r <= D; ++r) out.tab.push_back(word(r < D ? la[r] : none, (size_t)q));
+  const size_t meta = out.tab.size();
+  out.tab.resize(meta + out.groups);
+  for (int g = 0; g < out.groups; ++g) {
+    size_t nb = 0;
+    for (int r = 32 * g; r < std::min(D, 32 * g + 32); ++r) nb = std::max(nb, (lb[r].size() + 1) / 2);
+    out.tab[meta + g] = (unsigned)((out.tab.size() - meta - out.groups) << 8) | (unsigned)nb;
+    for (size_t q = 0; q < nb; ++q)
+      for (int i = 0; i < 32; ++i) out.tab.push_back(word(32 * g + i < D ? lb[32 * g + i] : none, q));
+  }
   return true;
 }
 
+// Weights of the two lists.
+void list_weights(const kg_sector* s, double& wa, double& wb) {
+  wa = 0.5 * s->Jxy;
+  wb = (s->parity > 0) ? wa / std::sqrt(2.0) : (s->parity < 0) ? -wa : 0.0;
+}
+
 struct SectorLayout {
-  size_t ctrl = 0, scal = 0, prof = 0, G = 0, basis = 0, traj = 0, tint = 0, ell = 0, states = 0, total = 0;
+  size_t ctrl = 0, scal = 0, prof = 0, G = 0, basis = 0, traj = 0, tint = 0, tab = 0, states = 0, total = 0;
 };
 
 size_t align_up(size_t x) { return (x + kg::kAlign - 1) / kg::kAlign * kg::kAlign; }
 
-SectorLayout sector_layout(int D, int ell, const kg_options* o, int B, int grid) {
+SectorLayout sector_layout(int D, int words, const kg_options* o, int B, int grid) {
   SectorLayout l;
   const size_t vb = (size_t)D * (o->prec == KG_PREC_C64_F64REC ? 8 : 16);
   size_t off = 0;
@@ -1237,7 +1344,7 @@ SectorLayout sector_layout(int D, int ell, const kg_options* o, int B, int grid)
   l.basis = take(vb * (size_t)o->m * grid);
   l.traj = take(vb * (size_t)(o->N + 1) * grid);
   l.tint = take(o->grad == KG_GRAD_EXACT ? vb * 2 * (size_t)o->N * grid : 0);
-  l.ell = take((size_t)ell * D * 2);
+  l.tab = take((size_t)words * 4);
   l.states = take(sizeof(unsigned) * (size_t)D);
   l.total = off;
   return l;
@@ -1266,13 +1373,21 @@ kg_status check_sector_opts(const kg_options* o, int B) {
   return KG_OK;
 }
 
+// Whether a subspace is taken: two vectors and one 16-bit column per row and antiparallel bond within
+// 200 KB (the split lists, which pad and double some entries, then stay below 224 KB).
+bool sector_fits(const kg_options* o, const SectorBasis& b) {
+  const size_t vb = (o->prec == KG_PREC_C64_F64REC) ? 8 : 16;
+  const size_t Dp = ((size_t)b.D + 15) & ~(size_t)15;
+  return 2 * Dp * vb + (size_t)b.bonds * b.D * 2 <= 200 * 1024 &&
+         kg::sector_smem_bytes(o->prec, b.D, b.words()) <= 224 * 1024;
+}
+
 // Grid for B pulses: every CTA that fits co-resident, at most B, at most opts->ctas.
-kg_status sector_grid(const kg_options* o, int D, int ell, int nt, int B, int* grid) {
-  const size_t smem = kg::sector_smem_bytes(o->prec, D, ell);
-  if (smem > 200 * 1024)
+kg_status sector_grid(const kg_options* o, const SectorBasis& b, int nt, int B, int* grid) {
+  if (!sector_fits(o, b))
     return host_fail(KG_ERR_UNSUPPORTED, "the subspace's state and tables exceed one CTA's shared memory");
   int maxc = 0;
-  cudaError_t e = kg::sector_kernel_max_ctas(o->prec, D, ell, nt, &maxc);
+  cudaError_t e = kg::sector_kernel_max_ctas(o->prec, b.D, b.words(), nt, &maxc);
   if (e != cudaSuccess) {
     return host_fail(KG_ERR_CUDA, std::string("occupancy query: ") + cudaGetErrorName(e));
   }
@@ -1328,23 +1443,24 @@ kg_status kg_sector_apply_h0(const kg_sector* s, const double* v, double* w, int
   std::string why;
   if (!build_basis(s, (size_t)kg::kSecMaxRows, true, b, why)) return host_fail(KG_ERR_UNSUPPORTED, why);
   if (D != b.D) return host_fail(KG_ERR_INVALID_ARG, "D must equal the subspace dimension " + std::to_string(b.D));
-  double wc[kg::kSecClasses] = {0, 0, 0, 0, 0, 0, 0, 0};
-  const double hxy = 0.5 * s->Jxy;
-  wc[kg::kSecW1] = hxy;
-  wc[kg::kSecWSqrt2] = hxy * std::sqrt(2.0);
-  wc[kg::kSecWInvSqrt2] = hxy / std::sqrt(2.0);
-  wc[kg::kSecWMinus1] = -hxy;
+  double wa, wb;
+  list_weights(s, wa, wb);
   const uint64_t maskL1 = (1ull << (s->L - 1)) - 1ull;
-  for (int r = 0; r < b.D; ++r) {  // the kernel's row: diagonal from s_r, then the table's entries
+  const unsigned* meta = b.tab.data() + (size_t)b.na2 * b.rows;
+  for (int r = 0; r < b.D; ++r) {  // the kernel's row: diagonal from s_r, then the two lists
     const uint64_t x = b.states[r];
     const double d = 0.25 * s->Jz * (double)(s->L - 1 - 2 * __builtin_popcountll((x ^ (x >> 1)) & maskL1));
     double re = d * v[2 * r], im = d * v[2 * r + 1];
-    for (int e = 0; e < b.ell_width; ++e) {
-      const unsigned en = b.ell[(size_t)e * b.D + r];
-      const int c = (int)(en & (kg::kSecMaxD - 1));
-      re += wc[en >> kg::kSecColBits] * v[2 * c];
-      im += wc[en >> kg::kSecColBits] * v[2 * c + 1];
-    }
+    auto add = [&](unsigned word, double wt) {
+      for (const int c : {(int)(word & 0xffffu), (int)(word >> 16)}) {
+        if (c >= b.D) continue;  // padding
+        re += wt * v[2 * c];
+        im += wt * v[2 * c + 1];
+      }
+    };
+    for (int q = 0; q < b.na2; ++q) add(b.tab[(size_t)q * b.rows + r], wa);
+    const unsigned mt = meta[r >> 5];
+    for (unsigned q = 0; q < (mt & 0xffu); ++q) add(meta[b.groups + (mt >> 8) + 32 * q + (r & 31)], wb);
     w[2 * r] = re;
     w[2 * r + 1] = im;
   }
@@ -1366,14 +1482,14 @@ kg_status kg_sector_workspace_bytes(const kg_sector* s, const kg_options* o, int
   int grid = B;
   int dev = 0, maxc = 0;
   if (cudaGetDevice(&dev) == cudaSuccess &&
-      kg::sector_smem_bytes(o->prec, b.D, b.ell_width) <= 200 * 1024 &&
-      kg::sector_kernel_max_ctas(o->prec, b.D, b.ell_width, s->block_threads, &maxc) == cudaSuccess && maxc > 0) {
+      sector_fits(o, b) &&
+      kg::sector_kernel_max_ctas(o->prec, b.D, b.words(), s->block_threads, &maxc) == cudaSuccess && maxc > 0) {
     grid = std::min(B, maxc);
     if (o->ctas > 0) grid = std::min(grid, o->ctas);
   } else {
     cudaGetLastError();  // no device here: clear the error the query left
   }
-  *bytes = sector_layout(b.D, b.ell_width, o, B, grid).total;
+  *bytes = sector_layout(b.D, b.words(), o, B, grid).total;
   return KG_OK;
 }
 
@@ -1398,7 +1514,7 @@ kg_status kg_sector_create(kg_sector_handle** handle, const kg_sector* s, const 
     delete h;
     return host_fail(KG_ERR_INVALID_ARG, "block_threads too few for the subspace's dimension");
   }
-  const size_t need1 = sector_layout(h->basis.D, h->basis.ell_width, o, B, 1).total;  // one CTA
+  const size_t need1 = sector_layout(h->basis.D, h->basis.words(), o, B, 1).total;  // one CTA
   if (!workspace || ((uintptr_t)workspace % kg::kAlign) != 0 || bytes < need1) {
     delete h;
     return host_fail(KG_ERR_WORKSPACE, "workspace must be 256-byte aligned and hold at least " +
@@ -1411,11 +1527,11 @@ kg_status kg_sector_create(kg_sector_handle** handle, const kg_sector* s, const 
     return host_fail(KG_ERR_CUDA, std::string("cudaGetDevice: ") + cudaGetErrorName(e));
   }
   int grid = 1;
-  if ((st = sector_grid(o, h->basis.D, h->basis.ell_width, s->block_threads, B, &grid)) != KG_OK) {
+  if ((st = sector_grid(o, h->basis, s->block_threads, B, &grid)) != KG_OK) {
     delete h;
     return st;
   }
-  const size_t need = sector_layout(h->basis.D, h->basis.ell_width, o, B, grid).total;
+  const size_t need = sector_layout(h->basis.D, h->basis.words(), o, B, grid).total;
   if (bytes < need) {
     delete h;
     return host_fail(KG_ERR_WORKSPACE, "workspace too small: need " + std::to_string(need) + " bytes, got " +
@@ -1425,7 +1541,7 @@ kg_status kg_sector_create(kg_sector_handle** handle, const kg_sector* s, const 
   h->opts = *o;
   if (!(h->opts.breakdown_tol > 0.0))
     h->opts.breakdown_tol = (o->prec == KG_PREC_C128) ? 1e-12 : (o->prec == KG_PREC_FF) ? 1e-10 : 1e-5;
-  h->lay = sector_layout(h->basis.D, h->basis.ell_width, o, B, grid);
+  h->lay = sector_layout(h->basis.D, h->basis.words(), o, B, grid);
   h->ws = (char*)workspace;
   h->stream = (cudaStream_t)cuda_stream;
   h->device = dev;
@@ -1435,8 +1551,8 @@ kg_status kg_sector_create(kg_sector_handle** handle, const kg_sector* s, const 
   std::vector<unsigned> st32(h->basis.states.begin(), h->basis.states.end());
   e = cudaMemcpyAsync(h->ws + h->lay.states, st32.data(), st32.size() * sizeof(unsigned), cudaMemcpyHostToDevice,
                       h->stream);
-  if (e == cudaSuccess && !h->basis.ell.empty())
-    e = cudaMemcpyAsync(h->ws + h->lay.ell, h->basis.ell.data(), h->basis.ell.size() * 2, cudaMemcpyHostToDevice,
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h->ws + h->lay.tab, h->basis.tab.data(), h->basis.tab.size() * 4, cudaMemcpyHostToDevice,
                         h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
@@ -1464,7 +1580,10 @@ kg_status kg_sector_evaluate(kg_sector_handle* h, const double* u, const void* p
   p.D = h->basis.D;
   p.N = o.N;
   p.m = o.m;
-  p.ell = h->basis.ell_width;
+  p.na2 = h->basis.na2;
+  p.rows = h->basis.rows;
+  p.groups = h->basis.groups;
+  p.words = h->basis.words();
   p.B = h->B;
   p.L1 = s.L - 1;
   p.grad_mode = o.grad;
@@ -1474,14 +1593,9 @@ kg_status kg_sector_evaluate(kg_sector_handle* h, const double* u, const void* p
   p.hc_amp = s.hc_amp;
   p.dt = o.dt;
   p.bd_tol = o.breakdown_tol;
-  for (int c = 0; c < kg::kSecClasses; ++c) p.wcls[c] = 0.0;
-  const double hxy = 0.5 * s.Jxy;
-  p.wcls[kg::kSecW1] = hxy;
-  p.wcls[kg::kSecWSqrt2] = hxy * std::sqrt(2.0);
-  p.wcls[kg::kSecWInvSqrt2] = hxy / std::sqrt(2.0);
-  p.wcls[kg::kSecWMinus1] = -hxy;
+  list_weights(&s, p.wa, p.wb);
   char* ws = h->ws;
-  p.ell_g = (const unsigned short*)(ws + h->lay.ell);
+  p.tab_g = (const unsigned*)(ws + h->lay.tab);
   p.states = (const unsigned*)(ws + h->lay.states);
   p.u = u;
   p.psi0 = (const double*)psi0;

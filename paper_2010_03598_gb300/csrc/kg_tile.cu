@@ -195,7 +195,7 @@ struct Tile {
   unsigned bonds_hi;   // MULTI: active bonds with both bits above the tile, bit b
   V wo[APT];           // own W_k
   float2 fact;         // complex64: this lane's entry of kInvFactFF
-  float w1[kTileSums];  // one warp, complex64: its sums
+  float w1;            // one warp, complex64: its sums (lane i: sum i)
   S nrm;               // ||W_0||
   R inv;               // 1 / ||W_0||
 
@@ -218,26 +218,14 @@ struct Tile {
   // warp); collect (after the barrier that follows): the totals, the same bits in every thread.
   __device__ __forceinline__ void post(const R (&v)[kTileSums]) {
     const int lane = tid & 31, warp = tid >> 5;
-    if constexpr (F32) {
-      float s[kTileSums];
-#pragma unroll
-      for (int i = 0; i < kTileSums; ++i) s[i] = warp_sum(v[i]);
-      if constexpr (NW == 1) {
-        w1[0] = s[0], w1[1] = s[1], w1[2] = s[2];
-        return;
-      }
-      if (lane < kTileSums) sm.red_f[par][warp][lane] = (lane == 0) ? s[0] : (lane == 1) ? s[1] : s[2];
-    } else {
-      // transposed butterfly: a lane ends up with one of four values, six additions instead of fifteen
-      const bool o1 = lane & 1, o2 = lane & 2;
-      const double a0 = o1 ? v[1] : v[0], g0 = o1 ? v[0] : v[1];
-      const double a1 = o1 ? 0.0 : v[2], g1 = o1 ? v[2] : 0.0;
-      const double s0 = a0 + __shfl_xor_sync(0xffffffffu, g0, 1);
-      const double s1 = a1 + __shfl_xor_sync(0xffffffffu, g1, 1);
-      double s = (o2 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, o2 ? s0 : s1, 2);
-#pragma unroll
-      for (int o = 4; o <= 16; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane < kTileSums) sm.red_d[par][warp][lane] = s;  // lane 0: v0, 1: v1, 2: v2
+    const R s = warp_sum3<R>(v[0], v[1], v[2]);
+    if constexpr (F32 && NW == 1) {
+      w1 = s;
+      return;
+    }
+    if (lane < 4) {
+      if constexpr (F32) sm.red_f[par][warp][lane] = s;
+      else sm.red_d[par][warp][lane] = s;
     }
     if constexpr (MULTI) {
       if (tid == 0) sm.cmd = kTileCmdSums | (par << 2);
@@ -245,7 +233,6 @@ struct Tile {
     }
   }
   __device__ __forceinline__ bool collect(S (&out)[kTileSums]) {
-    const int lane = tid & 31;
     if constexpr (MULTI) {
       nbar_sync(kTileBarGroup, NT + 32);
 #pragma unroll
@@ -254,24 +241,12 @@ struct Tile {
       return sm.ok != 0;
     } else if constexpr (F32 && NW == 1) {
 #pragma unroll
-      for (int i = 0; i < kTileSums; ++i) out[i] = FF{w1[i], 0.f};
+      for (int i = 0; i < kTileSums; ++i) out[i] = FF{__shfl_sync(0xffffffffu, w1, i), 0.f};
     } else if constexpr (F32) {
-#pragma unroll
-      for (int i = 0; i < kTileSums; ++i) {
-        FF s{sm.red_f[par][lane & (NW - 1)][i], 0.f};
-#pragma unroll
-        for (int o = 1; o < NW; o <<= 1)
-          s = ff_add(s, FF{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)});
-        out[i] = s;
-      }
+      warps_sum3<NW, FF>([&](int w, int i) { return FF{sm.red_f[par][w][i], 0.f}; }, out);
       par ^= 1;
     } else {
-      // lane = 4 w + i adds value i over the warps w
-      double s = sm.red_d[par][(lane >> 2) & (NW - 1)][lane & 3];
-#pragma unroll
-      for (int o = 1; o < NW; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, 4 * o);
-#pragma unroll
-      for (int i = 0; i < kTileSums; ++i) out[i] = __shfl_sync(0xffffffffu, s, i);
+      warps_sum3<NW, double>([&](int w, int i) { return sm.red_d[par][w][i]; }, out);
       par ^= 1;
     }
     return true;
@@ -1078,13 +1053,7 @@ __device__ __forceinline__ void tile_control(const EvalParams& p, TileSmem& sm, 
     }
     ok = __all_sync(0xffffffffu, ok);
     __threadfence();  // what the workers read after the barrier was stored before the messages
-    // transposed butterfly over the lanes, as in Tile::post
-    const bool o1 = lane & 1, o2 = lane & 2;
-    const double s0 = (o1 ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, o1 ? t[0] : t[1], 1);
-    const double s1 = (o1 ? 0.0 : t[2]) + __shfl_xor_sync(0xffffffffu, o1 ? t[2] : 0.0, 1);
-    double x = (o2 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, o2 ? s0 : s1, 2);
-#pragma unroll
-    for (int o = 4; o <= 16; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    const double x = warp_sum3(t[0], t[1], t[2]);
     if (lane < kTileSums) sm.tot[par][lane] = x;
     if (lane == 0) sm.ok = ok ? 1 : 0;
     __syncwarp();
