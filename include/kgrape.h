@@ -124,8 +124,8 @@ typedef struct kg_options {
                               kg_report.ckpt_every */
   int32_t tile_bits;       /* 0 = automatic; else amplitudes per tile = 2^tile_bits (6..13) */
   int32_t ctas;            /* 0 = automatic; else CTAs cooperating on the problem.  With both 0, chains
-                              that fit the registers of one CTA, or (complex128, L <= 18) of one
-                              tile per CTA, run there */
+                              of up to 18 spins run with one tile in the registers of each CTA
+                              (complex64 one CTA up to 12 spins, complex128 up to 8) */
   int32_t flags;           /* KG_FLAG_* */
   double dt;               /* slice length, dt > 0 */
   double breakdown_tol;    /* <= 0: 1e-12 (C128) or 1e-5 (C64); Lanczos stops when

@@ -211,8 +211,11 @@ kg_status configure_handle(const kg_chain* chain, const kg_options* opts, const 
     int maxr = 0;
     e = kg::eval_kernel_max_ctas(opts->prec, kg::kVariantResident, t, &maxr);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
-    // default: two tiles per CTA (paired so that every CTA has the same cross-tile work)
+    // default: two tiles per CTA (paired so that every CTA has the same cross-tile work); with the
+    // schedule left to the library one, where there are CTAs for it (19 spins, m = 20: 166 against 211 us a
+    // slice)
     int c = (opts->ctas > 0) ? opts->ctas : (ntiles >= 2 ? ntiles / 2 : 1);
+    if (autosched && ntiles <= maxr) c = ntiles;
     if (c > ntiles) c = ntiles;
     if (c > maxr) c = maxr;
     if (c > kg::kMaxCtas) c = kg::kMaxCtas;
@@ -687,7 +690,7 @@ kg_status kg_batch_create(kg_batch** batch, int32_t B, const kg_chain* chains, c
     for (int i = 0; i < B; ++i) {
       const int L = chains[order_of[i]].L;
       if (classes.empty() || classes.back().L != L)
-        classes.push_back(BatchClass{L, i, 0, kg::tile_kernel_covers(opts->prec, L) ? 0 : 1 << (L - 13)});
+        classes.push_back(BatchClass{L, i, 0, kg::tile_kernel_ctas(opts->prec, L) == 1 ? 0 : 1 << (L - 13)});
       classes.back().n++;
     }
   }

@@ -1,8 +1,8 @@
 // K-GRAPE evaluation with one tile of amplitudes per CTA, held in registers: the forward Krylov
 // sweep, target overlap, co-state sweep and gradient of one pulse, in one launch.
 //
-// For chains whose amplitudes fit the registers of one CTA (or, complex128, of the co-resident CTAs
-// with one tile each) an evaluation is a chain of short Krylov steps, whose cost is latency: block
+// For chains whose amplitudes fit the registers of one CTA (or of the co-resident CTAs with one tile
+// each) an evaluation is a chain of short Krylov steps, whose cost is latency: block
 // barriers, warp sums, the recurrence's scalars and the small exponential.  This kernel is laid out
 // for that chain.  A CTA has as many threads as its tile needs (a thread owns APT amplitudes
 // li = tid + NT j), one barrier per Lanczos step, and no FP64 instruction on the complex64 path
@@ -18,7 +18,7 @@
 // scalars for itself.  v_{k-1}, v_k and W stay in registers; the basis holds the v_k (shared memory if
 // it fits, else global).
 //
-// Several CTAs (complex128): the stencil acts on the raw vector W_k, which needs none of the step's
+// Several CTAs: the stencil acts on the raw vector W_k, which needs none of the step's
 // scalars, so that it runs while the group's sums are under way:
 //   v_k = (W_k - alpha_{k-1} v_{k-1}) / b_k,   H v_k = (H W_k - alpha_{k-1} H v_{k-1}) / b_k.
 // (On one CTA the waits it would hide are short, and H v_k by its recurrence carries more rounding.)  The tiles' W_k are exchanged through global memory.  A control warp posts
@@ -137,7 +137,7 @@ constexpr int kTileSums = 3;  // values of one reduction
 struct TileSmem {
   float red_f[2][16][4];     // warp partials (complex64: FP32 sums), by reduction parity
   double red_d[2][16][4];    // warp partials (complex128, and the FP64 overlaps of complex64)
-  double tot[2][4];          // group totals (several CTAs), by parity
+  double tot[2][4];          // group totals (several CTAs), by parity (complex64: packed float-float)
   float2 al_ff[kMaxM], b2_ff[kMaxM];  // complex64: alpha_k, b_{k+1}^2 of the slice (float-float)
   double al[kMaxM], be[kMaxM + 1];    // complex128: alpha_k, b_{k+1}
   double coef_re[3][kMaxM], coef_im[3][kMaxM];
@@ -164,8 +164,11 @@ __device__ __forceinline__ ulonglong2 ld_msg(const ulonglong2* p) {
   return r;
 }
 
+// Lighter than __threadfence(), which is sequentially consistent.
+__device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
 constexpr int kTileBarPost = 2, kTileBarGroup = 3;
-constexpr int kTileCmdSums = 1, kTileCmdExit = 2;
+constexpr int kTileCmdSums = 1, kTileCmdExit = 2, kTileCmdFp64 = 8;  // bit 2: the reduction's parity
 
 template <class V, int NT, int APT, bool SB, bool MULTI>
 struct Tile {
@@ -236,7 +239,7 @@ struct Tile {
     if constexpr (MULTI) {
       nbar_sync(kTileBarGroup, NT + 32);
 #pragma unroll
-      for (int i = 0; i < kTileSums; ++i) out[i] = sfrom(sm.tot[par][i], S());
+      for (int i = 0; i < kTileSums; ++i) out[i] = sunpack(sm.tot[par][i], S());
       par ^= 1;
       return sm.ok != 0;
     } else if constexpr (F32 && NW == 1) {
@@ -263,6 +266,15 @@ struct Tile {
       for (int i = 0; i < kTileSums; ++i) {
         const double s = warp_sum(v[i]);
         if (lane == 0) sm.red_d[par][warp][i] = s;
+      }
+      if constexpr (MULTI) {  // the other CTAs' share arrives in float-float
+        if (tid == 0) sm.cmd = kTileCmdSums | kTileCmdFp64 | (par << 2);
+        nbar_arrive(kTileBarPost, NT + 32);
+        S o[kTileSums];
+        if (!collect(o)) return false;
+#pragma unroll
+        for (int i = 0; i < kTileSums; ++i) out[i] = sdouble(o[i]);
+        return true;
       }
       sync();
 #pragma unroll
@@ -365,14 +377,32 @@ struct Tile {
     constexpr int b = LT + LA - 1;
     return ((unsigned)(li(j) >> b) ^ (unsigned)(base >> (b + 1))) & 1u;
   }
-  static constexpr int RD = (T <= 1024) ? 6 : 4;  // slots of the ring
+  // Blocks in flight: complex128 through a ring in shared memory, complex64 (8-byte amplitudes, which
+  // cp.async moves through L1 only) in registers.
+  static constexpr int RD = F32 ? (APT <= 4 ? 6 : 3) : (T <= 1024) ? 6 : 4;
+  V xr[MULTI && F32 ? RD : 1][MULTI && F32 ? APT : 1];
   __device__ __forceinline__ int cross_count() const {
     return 1 + __popc(bonds_hi) + ((p.hc_kind == KG_HC_SX_SITE && p.hc_site >= LT + LA) ? 1 : 0);
+  }
+  // Block n, loaded into q; `act` as below.
+  __device__ __forceinline__ void cross_load(const V* w, int n, unsigned& act, V (&q)[MULTI && F32 ? APT : 1]) {
+    if constexpr (MULTI && F32) {
+      if (n == 0) {
+#pragma unroll
+        for (int j = 0; j < APT; ++j)
+          q[j] = top_active(j) ? ldv(w + ((base + li(j)) ^ ((size_t)3 << (LT + LA - 1)))) : vmake<V>(0, 0);
+      } else {
+        const V* s = w + (base ^ (act ? (size_t)3 << (__ffs(act) - 1) : (size_t)1 << p.hc_site));
+        act &= act - 1;
+#pragma unroll
+        for (int j = 0; j < APT; ++j) q[j] = ldv(s + li(j));
+      }
+    }
   }
   // Copies of block n into slot n % RD; `act`: the active bonds from block n on.  One commit group per
   // block, empty past the last.
   __device__ __forceinline__ void cross_copy(const V* w, int n, int count, unsigned& act) {
-    if constexpr (MULTI) {
+    if constexpr (MULTI && !F32) {
       V* r = ring + (n % RD) * T;
       if (n == 0) {
 #pragma unroll
@@ -391,14 +421,40 @@ struct Tile {
     act = bonds_hi;
     const int count = cross_count();
 #pragma unroll
-    for (int n = 0; n < RD; ++n) cross_copy(w, n, count, act);
+    for (int n = 0; n < RD; ++n) {
+      if constexpr (F32) {
+        if (n < count) cross_load(w, n, act, xr[n]);
+      } else {
+        cross_copy(w, n, count, act);
+      }
+    }
   }
   __device__ __forceinline__ void cross_add(const V* w, unsigned act, V (&h)[APT]) {
     const int count = cross_count(), nb1 = 1 + __popc(bonds_hi);
     V x[APT];
 #pragma unroll
     for (int j = 0; j < APT; ++j) x[j] = vmake<V>(0, 0);
-    for (int n = 0; n < count; ++n) {
+    if constexpr (F32) {
+      auto take = [&](int n, const V (&q)[MULTI && F32 ? APT : 1]) {
+        if constexpr (MULTI && F32) {
+          if (n < nb1) {
+#pragma unroll
+            for (int j = 0; j < APT; ++j) x[j] = vadd(x[j], q[j]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < APT; ++j) h[j] = vfma(cx, q[j], h[j]);
+          }
+        }
+      };
+#pragma unroll
+      for (int n = 0; n < RD; ++n)
+        if (n < count) take(n, xr[n]);
+      for (int n = RD; n < count; ++n) {
+        cross_load(w, n, act, xr[0]);
+        take(n, xr[0]);
+      }
+    }
+    for (int n = 0; n < count && !F32; ++n) {
       cp_async_wait<RD - 1>();
       const V* r = ring + (n % RD) * T;
       if (n == 0) {
@@ -441,8 +497,9 @@ struct Tile {
       v[j] = vmul(inv, wo[j]);
       s[li(j)] = v[j];
     }
-    R alpha = 0, bk = 0, ib = 0, amax = 0, bmax = 0;
-    const R tol = (R)p.bd_tol;
+    R alpha = 0, bk = 0, ib = 0;
+    float amax = 0.f, bmax = 0.f;
+    const float tol = (float)p.bd_tol;
     meff = (sround(nrm) > 0) ? m : 0;
     broke = false;
     beta_m = 0;
@@ -487,8 +544,9 @@ struct Tile {
     V vp[APT], hp[APT];
 #pragma unroll
     for (int j = 0; j < APT; ++j) vp[j] = hp[j] = vmake<V>(0, 0);
-    R ap = 0, ib = inv, bk = 0, amax = 0, bmax = 0;
-    const R tol = (R)p.bd_tol;
+    R ap = 0, ib = inv, bk = 0;
+    float amax = 0.f, bmax = 0.f;
+    const float tol = (float)p.bd_tol;
     meff = (sround(nrm) > 0) ? m : 0;
     broke = false;
     beta_m = 0;
@@ -629,12 +687,13 @@ struct Tile {
   // near an invariant subspace b_{k+1}^2 = ||W_{k+1} - alpha_k v_k||^2 formed explicitly.  broke:
   // b_{k+1} vanishes (Alg. "Lanczos", b_j > 0 with a tolerance).  false: not finite, or aborted.
   __device__ __forceinline__ bool step_scalars(int k, bool last, const S (&o)[kTileSums], const V (&v)[APT],
-                                               const V (&w)[APT], R tol,
-                                               R& amax, R& bmax, R& alpha, R& beta, R& inv_b, bool& broke) {
+                                               const V (&w)[APT], float tol,
+                                               float& amax, float& bmax, R& alpha, R& beta, R& inv_b, bool& broke) {
     alpha = sround(o[0]);
     S b2 = sb2(o[0], o[1], o[2]);
     sroot(b2, beta, inv_b);
-    const bool usual = !scancels(b2, o[1]) && sfinite(o[0]) && sfinite(o[1]) && beta > tol * fmax((R)1, fmax(amax, fabs(alpha)) + bmax);
+    const float af = fabsf((float)alpha);  // the breakdown test needs no more than FP32
+    const bool usual = !scancels(b2, o[1]) && sfinite(o[0]) && sfinite(o[1]) && (float)beta > tol * fmaxf(1.f, fmaxf(amax, af) + bmax);
     if (!usual) {
       if (!sfinite(o[0]) || !sfinite(o[1])) {
         fail_nonfinite();
@@ -654,10 +713,10 @@ struct Tile {
         b2 = oe[0];
         sroot(b2, beta, inv_b);
       }
-      if (!last) broke = beta <= tol * fmax((R)1, fmax(amax, fabs(alpha)) + bmax);
+      if (!last) broke = (float)beta <= tol * fmaxf(1.f, fmaxf(amax, af) + bmax);
     }
-    amax = fmax(amax, fabs(alpha));
-    bmax = fmax(bmax, beta);
+    amax = fmaxf(amax, af);
+    bmax = fmaxf(bmax, (float)beta);
     if (tid == 0) {
       if constexpr (F32) {
         sm.al_ff[k] = make_float2(o[0].hi, o[0].lo);
@@ -1002,8 +1061,10 @@ struct Tile {
 // reduction's number, then reads every CTA's message (lane l those of CTAs l, l + 32, ...) until it
 // carries that number, adds them up and answers the workers.  Two sets of slots, by the number's
 // parity: a CTA posts reduction n + 2 only after every CTA has posted n + 1, so has read n.
-template <int NT>
+template <class V, int NT>
 __device__ __forceinline__ void tile_control(const EvalParams& p, TileSmem& sm, int rank, int size) {
+  using S = typename Prec<V>::S;
+  constexpr bool F32 = Prec<V>::F32;
   constexpr int NW = NT / 32;
   const int lane = threadIdx.x & 31;
   unsigned long long seq = 0;
@@ -1014,26 +1075,44 @@ __device__ __forceinline__ void tile_control(const EvalParams& p, TileSmem& sm, 
     const int par = (cmd >> 2) & 1;
     ++seq;
     ulonglong2* slots = reinterpret_cast<ulonglong2*>(p.red) + (size_t)(seq & 1) * size * kNRed;
-    double s = sm.red_d[par][(lane >> 2) & (NW - 1)][lane & 3];
+    // lane i < 3: the CTA's sum i (FP64 sums of the complex64 path come through the FP64 partials too)
+    S c[kTileSums];
+    if constexpr (F32) {
+      if (cmd & kTileCmdFp64) {
+        double d[kTileSums];
+        warps_sum3<NW, double>([&](int w, int i) { return sm.red_d[par][w][i]; }, d);
 #pragma unroll
-    for (int o = 1; o < NW; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, 4 * o);
-    __threadfence();  // the workers' stores, ordered before this warp by the named barrier
+        for (int i = 0; i < kTileSums; ++i) c[i] = ff_from_double(d[i]);
+      } else {
+        warps_sum3<NW, FF>([&](int w, int i) { return FF{sm.red_f[par][w][i], 0.f}; }, c);
+      }
+    } else {
+      warps_sum3<NW, double>([&](int w, int i) { return sm.red_d[par][w][i]; }, c);
+    }
+    const S mine = (lane == 0) ? c[0] : (lane == 1) ? c[1] : c[2];
+    fence_acq_rel();  // the workers' stores, ordered before this warp by the named barrier
     const bool skip = rank == 0 && ((p.debug_fault == 1 && seq == 1) || (p.debug_fault == 2 && seq == 2));
-    if (lane < kTileSums && !skip) st_msg(slots + rank * kNRed + lane, (unsigned long long)__double_as_longlong(s), seq);
-    double t[kTileSums] = {0.0, 0.0, 0.0};
+    if (lane < kTileSums && !skip) st_msg(slots + rank * kNRed + lane, (unsigned long long)__double_as_longlong(spack(mine)), seq);
+    S t[kTileSums] = {S(), S(), S()};
     bool ok = true;
     unsigned long long t0 = 0;
     unsigned polls = 0;
-    for (int r = lane; r < size && ok; r += 32) {
-      ulonglong2 q[kTileSums];
+    for (int r = lane; r < size && ok; r += 64) {  // two slots in a round
+      ulonglong2 q[2][kTileSums];
+      unsigned open = (r + 32 < size) ? 3u : 1u;
+      const bool two = open == 3u;
       for (;;) {
-        bool all = true;
 #pragma unroll
-        for (int i = 0; i < kTileSums; ++i) {
-          q[i] = ld_msg(slots + r * kNRed + i);
-          all = all && q[i].y == seq;
+        for (int i = 0; i < 2; ++i) {
+          if ((open >> i) & 1u) {
+#pragma unroll
+            for (int j = 0; j < kTileSums; ++j) q[i][j] = ld_msg(slots + (r + 32 * i) * kNRed + j);
+          }
         }
-        if (all) break;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          if (((open >> i) & 1u) && q[i][0].y == seq && q[i][1].y == seq && q[i][2].y == seq) open &= ~(1u << i);
+        if (!open) break;
         if ((++polls & 31u) == 0u) {
           if (ld_volatile_i32(p.ctrl + kCtrlAbort)) { ok = false; break; }
           const unsigned long long now = globaltimer_ns();
@@ -1047,14 +1126,18 @@ __device__ __forceinline__ void tile_control(const EvalParams& p, TileSmem& sm, 
           }
         }
       }
-      if (ok)
+      if (ok) {
 #pragma unroll
-        for (int i = 0; i < kTileSums; ++i) t[i] += __longlong_as_double((long long)q[i].x);
+        for (int j = 0; j < kTileSums; ++j) t[j] = vx_add(t[j], sunpack(__longlong_as_double((long long)q[0][j].x), S()));
+        if (two)
+#pragma unroll
+          for (int j = 0; j < kTileSums; ++j) t[j] = vx_add(t[j], sunpack(__longlong_as_double((long long)q[1][j].x), S()));
+      }
     }
     ok = __all_sync(0xffffffffu, ok);
-    __threadfence();  // what the workers read after the barrier was stored before the messages
-    const double x = warp_sum3(t[0], t[1], t[2]);
-    if (lane < kTileSums) sm.tot[par][lane] = x;
+    fence_acq_rel();  // what the workers read after the barrier was stored before the messages
+    const S x = warp_sum3(t[0], t[1], t[2]);
+    if (lane < kTileSums) sm.tot[par][lane] = spack(x);
     if (lane == 0) sm.ok = ok ? 1 : 0;
     __syncwarp();
     nbar_arrive(kTileBarGroup, NT + 32);
@@ -1074,7 +1157,7 @@ __device__ __forceinline__ void tile_cta(const EvalParams& p, TileSmem& sm, V* s
   }
   __syncthreads();
   if (MULTI && threadIdx.x >= NT) {
-    tile_control<NT>(p, sm, rank, (int)gridDim.x);
+    tile_control<V, NT>(p, sm, rank, (int)gridDim.x);
     return;
   }
   TileT t{p, sm, sw, sw + 2 * TileT::T};
@@ -1141,21 +1224,28 @@ TileKernel tile_single(int m) {
   return tile_choice<V, NT, APT, false>(2 * vec);
 }
 
-// One of several CTAs: two W_k buffers and the ring of partner blocks.
+// One of several CTAs: two W_k buffers and (complex128) the ring of partner blocks.
 template <class V, int NT, int APT>
 TileKernel tile_multi(int L) {
   using TileT = Tile<V, NT, APT, false, true>;
   const int t = __builtin_ctz(NT * APT);
   return {reinterpret_cast<const void*>(&kg_tile_kernel<V, NT, APT, false, true>), nullptr, NT + 32, t,
-          (size_t)(2 + TileT::RD) * TileT::T * sizeof(V), 1 << (L - t)};
+          (size_t)(2 + (sizeof(V) == 16 ? TileT::RD : 0)) * TileT::T * sizeof(V), 1 << (L - t)};
 }
 
 // Threads x amplitudes by chain length.  More threads shorten every thread's chain of shared-memory
 // loads, fewer make the block's sums cheaper; measured (us per slice, m = 16, complex64):
 //   L = 7: 64 x 2 12.7, 32 x 4 12.3;  8: 128 x 2 14.1, 32 x 8 15.3, 64 x 4 15.7;  9: 256 x 2 17.3, 128 x 4
 //   17.7, 64 x 8 18.5;  10: 128 x 8 22.2, 256 x 4 22.6;  11: 256 x 8 29.7, 512 x 4 34.8;
-//   12: 256 x 16 (raw vectors) 47.7, 512 x 8 61.0 (128 registers).
-// The kernels that ran these chains before took 100 (L = 5) to 148 us (L = 11) and 77 us (L = 12).
+//   12: 256 x 16 (raw vectors) 47.7, 512 x 8 61.0 (128 registers), 4 CTAs of 128 x 8 44.7.
+// (With three sums by one butterfly since: 8 11.3, 10 20.2, 11 27.3, 12 45.0.)  On several CTAs a step
+// costs 3.0 (16 CTAs) to 4.7 us (128), nearly all of it the exchange, so the tiles are as large as the
+// registers let them be cheap:
+//   13: 128 x 4 52.2, 128 x 8 54.2;  14: 128 x 4 58.8, 128 x 8 59.3;  15: 128 x 8 64.4, 128 x 4 64.8, 128 x 2 75.7;
+//   16: 128 x 8 72.8, 256 x 4 72.9, 128 x 4 77.7;  17: 128 x 8 85.0, 256 x 8 89.1;  18: 256 x 8 101.1.
+// At L = 19 the resident loop is the faster one (139 against 171).
+// The kernels that ran these chains before took 100 (L = 5) to 148 us (L = 11), 77 us (L = 12) and, two
+// 4096-amplitude tiles per CTA, 128 (L = 13) to 164 us (L = 18).
 // complex128 is bound by the FP64 units, one quarter in each quarter of the SM: one warp per quarter
 // as soon as there are amplitudes for it, and as many CTAs as there are SMs (us per slice, m = 16):
 //   L = 8: 128 x 2 76, 64 x 4 113, 256 x 1 91;  9: 4 CTAs of 128 x 1 76, 2 of 128 x 2 88, one CTA 125;
@@ -1173,6 +1263,9 @@ TileKernel pick_tile(int prec, int L, int m) {
     if (L == 10) return tile_single<float2, 128, 8>(m);
     if (L == 11) return tile_single<float2, 256, 8>(m);
     if (L == 12) return tile_single<float2, 256, 16>(m);
+    if (L <= 14) return tile_multi<float2, 128, 4>(L);
+    if (L <= 17) return tile_multi<float2, 128, 8>(L);
+    if (L == 18) return tile_multi<float2, 256, 8>(L);
   }
   if (prec == KG_PREC_C128) {
     if (L <= 5) return tile_single<double2, 32, 1>(m);

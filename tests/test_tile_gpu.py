@@ -69,28 +69,31 @@ def test_every_block_shape_and_mode_vs_oracle(L, hc, m, mode, prec):
     assert rep["status"] == 0 and abs(rep["norm_final"] - 1.0) < (1e-12 if prec == "c128" else 1e-5)
 
 
-@pytest.mark.parametrize("L,hc,m,mode", [(13, 12, 9, "exact"), (14, 13, 6, "centered"), (15, "sz", 8, "zeroth"), (15, 7, 7, "none"),
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("L,hc,m,mode", [(13, 12, 9, "exact"), (14, 13, 6, "centered"), (14, 8, 7, "zeroth"), (15, "sz", 8, "zeroth"), (15, 7, 7, "none"),
+                                         (14, 9, 8, "exact"), (15, 10, 8, "centered"),
                                          (16, 8, 8, "centered"), (16, 9, 6, "exact"), (17, 16, 6, "centered"), (18, 0, 6, "zeroth")])
-def test_complex128_over_several_ctas_vs_oracle(L, hc, m, mode):
-    # 64 to 128 CTAs with one tile each: tiles of 128 to 2048 amplitudes, the control inside the tile, on
-    # its top bit (L = 16: bit 8) and above it
+def test_several_ctas_vs_oracle(L, hc, m, mode, prec):
+    # 16 to 128 CTAs with one tile each: tiles of 128 to 2048 amplitudes, the control inside the tile, on
+    # its top bit (complex128, L = 16: bit 8; complex64, L = 14: bit 8, L = 15: bit 9) and above it
     N, dt = 2, 0.05
     u, psi0, f, spec, ch = problem(L, N, 750 + L, hc)
     F_ref, g_ref, _ = oracle.evaluate(ch, u, dt, m, psi0, f, "centered" if mode == "none" else mode)
-    F, g, rep = evaluate(spec, dict(N=N, dt=dt, m=m, prec="c128", grad=mode), u, psi0, f)
-    check("c128", F, g, F_ref, g_ref)
+    F, g, rep = evaluate(spec, dict(N=N, dt=dt, m=m, prec=prec, grad=mode), u, psi0, f)
+    check(prec, F, g, F_ref, g_ref)
     assert rep["status"] == 0 and rep["ctas"] > 1
 
 
-def test_group_that_a_member_never_joins_times_out_cleanly():
+@pytest.mark.parametrize("prec,L", [("c128", 12), ("c64", 14)])
+def test_group_that_a_member_never_joins_times_out_cleanly(prec, L):
     # CTA 0 does not post its first sums (host-side fault injection): every wait runs out, the launch ends
     # with KG_ERR_TIMEOUT, and the next launch on the same engine is clean and deterministic.
     from paper_2010_03598_gb300 import _abi
     from paper_2010_03598_gb300 import api as A
-    L, N = 12, 3
+    N = 3
     u, psi0, f, spec, ch = problem(L, N, 77, 0)
     dev = torch.device("cuda", 0)
-    eng = A.KGrape(A.ChainSpec(**spec), A.Options(N, 0.05, 8, prec="c128"))
+    eng = A.KGrape(A.ChainSpec(**spec), A.Options(N, 0.05, 8, prec=prec))
     t = [torch.tensor(x, device=dev) for x in (u, psi0, f)]
     for kind in (1, 2):
         try:
@@ -111,11 +114,11 @@ def test_group_that_a_member_never_joins_times_out_cleanly():
     eng.close()
     assert got[0][0] == got[1][0] and np.array_equal(got[0][1], got[1][1])
     F_ref, g_ref, _ = oracle.evaluate(ch, u, 0.05, 8, psi0, f, "centered")
-    check("c128", *got[0], F_ref, g_ref)
+    check(prec, *got[0], F_ref, g_ref)
 
 
 @pytest.mark.parametrize("prec", ["c64", "c128"])
-@pytest.mark.parametrize("L,N,C", [(4, 9, 2), (8, 11, 4), (9, 6, 1), (11, 10, 9), (7, 5, 7)])
+@pytest.mark.parametrize("L,N,C", [(4, 9, 2), (8, 11, 4), (9, 6, 1), (11, 10, 9), (7, 5, 7), (14, 7, 3)])
 def test_checkpoints_are_bitwise_equal_to_the_full_trajectory(L, N, C, prec):
     u, psi0, f, spec, ch = problem(L, N, 800 + L, 0)
     full = evaluate(spec, dict(N=N, dt=0.05, m=10, prec=prec, grad="centered"), u, psi0, f)
@@ -126,7 +129,7 @@ def test_checkpoints_are_bitwise_equal_to_the_full_trajectory(L, N, C, prec):
 
 
 @pytest.mark.parametrize("prec", ["c64", "c128"])
-@pytest.mark.parametrize("L", [6, 8, 11])
+@pytest.mark.parametrize("L", [6, 8, 11, 13])
 def test_invariant_and_nearly_invariant_subspaces(L, prec):
     # |0...0> is an eigenstate of H0 and of the Sz control: the basis ends after one vector.  With 1 %
     # of a random state the identity for b_1 cancels, and b_1 is formed explicitly, in every slice.
