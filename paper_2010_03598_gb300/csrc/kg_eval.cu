@@ -2040,38 +2040,14 @@ struct StrBlk {
   int gx;
 };
 
-// Partner blocks of the tile at `base` (for W = vector w): bond 11 (own half h = 1 - bt against
-// half bt of tile base ^ 2^12: granules g with bit 1 = h, source granule g ^ 2), the antiparallel
-// bonds b >= 12 (tile base ^ (3 << b)), an Sx control on a site >= 12 (tile base ^ (1 << s),
-// weight of the control).  str_partners returns their number; str_partner the n-th of them.
+// Partner blocks of the tile at `base` (for W = vector w), in order: bond 11 (own half h = 1 - bt
+// against half bt of tile base ^ 2^12: granules g with bit 1 = h, source granule g ^ 2), the
+// antiparallel bonds b >= 12 (tile base ^ (3 << b)), an Sx control on a site >= 12 (tile base ^ (1 << s),
+// weight of the control).  str_outer: the antiparallel bonds as a mask (bit b - 12).  Whoever walks the
+// blocks keeps the mask of those left and takes its lowest bit: looking each block's bond up from the
+// start, bond by bond, cost more than moving the block (1.6 us a block of 32 KB; L = 24).
 __device__ __forceinline__ unsigned str_outer(size_t base, int L1) {
-  unsigned act = 0;
-  for (int b = 12; b < L1; ++b)
-    if (((base >> b) ^ (base >> (b + 1))) & 1u) act |= 1u << (b - 12);
-  return act;
-}
-__device__ __forceinline__ int str_partners(size_t base, int L1, bool sx12) {
-  return ((L1 > 11) ? 1 : 0) + __popc(str_outer(base, L1)) + (sx12 ? 1 : 0);
-}
-__device__ __forceinline__ StrBlk str_partner(size_t base, const float2* w, int L1, int hs, bool sx12, int n,
-                                              bool& is_ctrl) {
-  is_ctrl = false;
-  if (L1 > 11) {
-    if (n == 0) {
-      const unsigned h = 1u - (unsigned)((base >> 12) & 1u);
-      return {w + (base ^ ((size_t)1 << 12)), h ? 0xcu : 0x3u, 2};
-    }
-    --n;
-  }
-  unsigned act = str_outer(base, L1);
-  const int na = __popc(act);
-  if (n < na) {
-    for (int i = 0; i < n; ++i) act &= act - 1;
-    const int b = 12 + __ffs(act) - 1;
-    return {w + (base ^ ((size_t)3 << b)), 0xfu, 0};
-  }
-  is_ctrl = sx12;
-  return {w + (base ^ ((size_t)1 << hs)), 0xfu, 0};
+  return (L1 > 12) ? (unsigned)(((base ^ (base >> 1)) & (((size_t)1 << L1) - 1)) >> 12) : 0u;
 }
 
 // This thread's copies of block `bk` into ring stage st: stage layout [kStrDepth][4][512] float4.
@@ -2084,8 +2060,8 @@ __device__ __forceinline__ void str_issue(float4* ring, int st, const StrBlk& bk
 }
 
 // The stream of one step: for every own tile c (in order) its partner blocks, then X_{k-1}
-// and v_{k-1} (k > 0), then W_k.  StrCursor walks it; both the issuer (kStrDepth blocks ahead)
-// and the consumer use one, all threads identically.
+// and v_{k-1} (k > 0), then W_k.  The issuer's cursor walks it kStrDepth blocks ahead of the consumer
+// (lanczos_str64), all threads identically.
 struct StrStep {
   const float2* w;      // W_k (all tiles)
   const float2* x;      // X_{k-1}
@@ -2093,31 +2069,18 @@ struct StrStep {
   int k, L1, hs, n_own;
   bool sx12;
 };
+enum { kStrHalf, kStrOuter, kStrCtrl, kStrX, kStrV, kStrW };
 struct StrCursor {
-  int c, b, nb;  // tile, block within the tile, blocks of the tile
+  int c, stage;   // tile, kind of the next block
+  unsigned act;   // outer bonds left
   size_t base;
 };
-__device__ __forceinline__ int str_nblk(const StrStep& S, size_t base) {
-  return str_partners(base, S.L1, S.sx12) + (S.k > 0 ? 3 : 1);
-}
 __device__ __forceinline__ void str_cursor_tile(const Ctx<float2>& c, const StrStep& S, StrCursor& u) {
   if (u.c < S.n_own) {
     u.base = c.tile_base(u.c);
-    u.nb = str_nblk(S, u.base);
+    u.act = str_outer(u.base, S.L1);
+    u.stage = (S.L1 > 11) ? kStrHalf : kStrOuter;
   }
-}
-// Block b of the tile at `base`: partners first, then (k > 0) X and V, then W.
-__device__ __forceinline__ StrBlk str_block(const StrStep& S, size_t base, int b) {
-  const int np = str_partners(base, S.L1, S.sx12);
-  if (b < np) {
-    bool ctrl;
-    return str_partner(base, S.w, S.L1, S.hs, S.sx12, b, ctrl);
-  }
-  b -= np;
-  if (S.k == 0) return {S.w + base, 0xfu, 0};
-  if (b == 0) return {S.x + base, 0xfu, 0};
-  if (b == 1) return {S.vprev + base, 0xfu, 0};
-  return {S.w + base, 0xfu, 0};
 }
 // Issuer: copy the block under the cursor (if the step has one left) and advance; one commit
 // group per call, empty past the end, so that every consumed block is exactly kStrDepth - 1
@@ -2125,10 +2088,38 @@ __device__ __forceinline__ StrBlk str_block(const StrStep& S, size_t base, int b
 __device__ __forceinline__ void str_issue_next(const Ctx<float2>& c, const StrStep& S, StrCursor& u, float4* ring,
                                                int& slot) {
   if (u.c < S.n_own) {
-    str_issue(ring, slot, str_block(S, u.base, u.b));
-    if (++u.b == u.nb) {
+    if (u.stage == kStrOuter && !u.act) u.stage = S.sx12 ? kStrCtrl : S.k > 0 ? kStrX : kStrW;
+    StrBlk bk{nullptr, 0xfu, 0};
+    bool end = false;
+    switch (u.stage) {
+      case kStrHalf:
+        bk = {S.w + (u.base ^ ((size_t)1 << 12)), ((u.base >> 12) & 1u) ? 0x3u : 0xcu, 2};
+        u.stage = kStrOuter;
+        break;
+      case kStrOuter:
+        bk.src = S.w + (u.base ^ ((size_t)3 << (12 + __ffs(u.act) - 1)));
+        u.act &= u.act - 1;
+        break;
+      case kStrCtrl:
+        bk.src = S.w + (u.base ^ ((size_t)1 << S.hs));
+        u.stage = S.k > 0 ? kStrX : kStrW;
+        break;
+      case kStrX:
+        bk.src = S.x + u.base;
+        u.stage = kStrV;
+        break;
+      case kStrV:
+        bk.src = S.vprev + u.base;
+        u.stage = kStrW;
+        break;
+      default:
+        bk.src = S.w + u.base;
+        end = true;
+        break;
+    }
+    str_issue(ring, slot, bk);
+    if (end) {
       ++u.c;
-      u.b = 0;
       str_cursor_tile(c, S, u);
     }
   }
@@ -2190,26 +2181,26 @@ __device__ __noinline__ bool lanczos_str64(Ctx<float2>& c, const float2* src, do
     float2* wdst = last ? nullptr : wb + (size_t)((k + 1) & 1) * D;    // W_{k+1}
     const float ap = ss.f_ap, ib = ss.f_ib, bk = ss.f_bk;
     const float vsc = (k == 1) ? ss.f_ib0 : 1.f;  // slot 0 is psi itself: v_0 = psi / b_0
-    StrCursor iu{0, 0, 0, 0};
+    StrCursor iu{0, 0, 0u, 0};
     str_cursor_tile(c, S, iu);
     int islot = 0, cslot = 0;
     for (int d = 0; d < kStrDepth; ++d) str_issue_next(c, S, iu, ring, islot);
     float acc_a = 0.f, acc_n = 0.f, acc_q = 0.f;
     for (int ct = 0; ct < S.n_own; ++ct) {
       const size_t base = c.tile_base(ct);
-      const int np = str_partners(base, L1, S.sx12);
-      // ---- partner sums of W_k, block by block
+      // ---- partner sums of W_k, block by block (the order of StrCursor)
       float4 xs[4];
 #pragma unroll
       for (int g = 0; g < 4; ++g) xs[g] = f4zero();
+      const int np = ((L1 > 11) ? 1 : 0) + __popc(str_outer(base, L1)) + (S.sx12 ? 1 : 0);
+      const unsigned half = ((base >> 12) & 1u) ? 0x3u : 0xcu;
       for (int b = 0; b < np; ++b) {
-        bool ctrl;
-        const StrBlk blk = str_partner(base, S.w, L1, hs, S.sx12, b, ctrl);
-        const float wg = ctrl ? cu_sx : hxy;
+        const float wg = (S.sx12 && b == np - 1) ? cu_sx : hxy;
+        const unsigned gmask = (L1 > 11 && b == 0) ? half : 0xfu;
         const float4* q = str_wait(ring, cslot);
 #pragma unroll
         for (int g = 0; g < 4; ++g)
-          if ((blk.gmask >> g) & 1u) xs[g] = f4fma(wg, q[g * NT], xs[g]);
+          if ((gmask >> g) & 1u) xs[g] = f4fma(wg, q[g * NT], xs[g]);
         str_issue_next(c, S, iu, ring, islot);
         cslot = (cslot + 1 == kStrDepth) ? 0 : cslot + 1;
       }
