@@ -111,6 +111,7 @@ struct SmemSlice {
   Group grp;  // the group's barrier state while the resident loop runs (written by thread 0)
   float2 ff_a[kMaxM], ff_n[kMaxM], ff_q[kMaxM], ff_e[kMaxM];
   float4 slotbuf[2 * kSlotRanks];  // the group's reduction slots, prefetched by warp 0
+  int tables;      // headline loop: the partner tables of this evaluation are built
   int recomb_pre;  // the Lanczos loop has issued the recombination's first copies (complex64)
   int ctl_cmd;  // control warp: the step whose sums were handed over (| kCtlLast), or kCtlExit
   int ctl_ok;   // control warp: the group barrier passed (0: aborted or timed out)
@@ -1832,8 +1833,11 @@ __device__ __noinline__ bool lanczos_res64b(Ctx<float2>& c, const float2* src, d
     ss.grp = c.g;
     lz_init(ss, nrm_src, p.m);
     ss.ff_e_set = 0u;
-    build_chunk_table(c, p, ss);
-    build_unit_table(ss, c.n_own);
+    if (!ss.tables) {  // the partner tables depend on the tiles alone: once per evaluation
+      ss.tables = 1;
+      build_chunk_table(c, p, ss);
+      build_unit_table(ss, c.n_own);
+    }
   }
   // W_0 = psi: the own pairs into shared memory; the diagonal of H_j (pair order) beside it
   {
@@ -2509,7 +2513,7 @@ __device__ __noinline__ bool run_eval(const EvalParams& p, int rank, int size, S
   for (int i = 0; i < 8; ++i)
     if (c.prof_on && threadIdx.x == 0) ss.prof_acc[i] = 0;
   const bool lead = (rank == 0 && threadIdx.x == 0);
-  if (threadIdx.x == 0) ss.recomb_pre = 0;
+  if (threadIdx.x == 0) ss.recomb_pre = ss.tables = 0;
 
   // ---- forward sweep (Alg. "Basic GRAPE", step 4)
   double nrm_prev;
