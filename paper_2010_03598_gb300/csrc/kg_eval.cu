@@ -684,7 +684,9 @@ constexpr int kRecombDepth = 3;  // 3 x 64 KB: all of the resident path's shared
 // This thread's asynchronous copies of basis vector vk for the own tiles at rb[0..n_own):
 // amplitude pairs 2 (tid + 512 g) + {0, 1}, g < 4, into stage st[(ct * 4 + g) * kThreads + tid].
 // The basis is read once here: the copies carry an evict_first L2 policy (see l2_policy_first).
-__device__ __forceinline__ void recomb_issue(const float2* vk, const size_t (&rb)[2], int n_own, float4* st) {
+// flip (even): the pairs at index ^ flip instead.
+__device__ __forceinline__ void recomb_issue(const float2* vk, const size_t (&rb)[2], int n_own, float4* st,
+                                             size_t flip = 0) {
   const int tid = threadIdx.x;
   const unsigned long long pol = l2_policy_first();
 #pragma unroll
@@ -692,7 +694,7 @@ __device__ __forceinline__ void recomb_issue(const float2* vk, const size_t (&rb
     if (ct < n_own) {
 #pragma unroll
       for (int g = 0; g < 4; ++g)
-        cp_async16_hint(st + (ct * 4 + g) * kThreads + tid, vk + rb[ct] + 2 * (size_t)(tid + g * kThreads), pol);
+        cp_async16_hint(st + (ct * 4 + g) * kThreads + tid, vk + ((rb[ct] + 2 * (size_t)(tid + g * kThreads)) ^ flip), pol);
     }
   }
 }
@@ -705,32 +707,32 @@ struct RecombConsts {
   float h_amp;
 };
 
-// One recombined amplitude y at global index gi: store it and add its contributions to
-// ||dst||^2 and to the fused overlap (see recomb_finalize).
+// One recombined pair (amplitudes gi, gi + 1, gi even): store it and add its contributions to ||dst||^2
+// and to the fused overlap (see recomb_finalize).  qp: the pair of psi_other that Hc couples it to.
 template <class A>
-__device__ __forceinline__ void recomb_amp(const RecombConsts& rc, size_t gi, float2 y, float2* dst, int extra,
-                                           const float2* psi_other, A& nacc, A& gacc, double& ex0, double& ex1) {
-  stv_hint(dst + gi, y, l2_policy_first());
-  nacc += (A)(y.x * y.x + y.y * y.y);
-  if (extra == kExtraOverlapTarget) {
-    const double2 f = rc.target[gi];
-    ex0 += f.x * (double)y.x + f.y * (double)y.y;
-    ex1 += f.x * (double)y.y - f.y * (double)y.x;
-  } else if (extra == kExtraGradOverlap) {
-    float2 q;
-    if (rc.sx_site >= 0) {
-      q = ldv(psi_other + (gi ^ ((size_t)1 << rc.sx_site)));
-      const float h = 0.5f * rc.h_amp;
-      q.x *= h;
-      q.y *= h;
-    } else {
-      const int nz = __popc(rc.mk) - 2 * __popc((unsigned)gi & rc.mk);
-      const float dz = rc.h_amp * 0.5f * (float)nz;
-      q = ldv(psi_other + gi);
+__device__ __forceinline__ void recomb_pair(const RecombConsts& rc, size_t gi, float4 y4, float2* dst, int extra,
+                                            float4 qp, A& nacc, A& gacc, double& ex0, double& ex1) {
+  const unsigned long long pol = l2_policy_first();
+  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(dst + gi), "f"(y4.x), "f"(y4.y),
+               "f"(y4.z), "f"(y4.w), "l"(pol)
+               : "memory");
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const float2 y = x ? make_float2(y4.z, y4.w) : make_float2(y4.x, y4.y);
+    nacc += (A)(y.x * y.x + y.y * y.y);
+    if (extra == kExtraOverlapTarget) {
+      const double2 f = rc.target[gi + x];
+      ex0 += f.x * (double)y.x + f.y * (double)y.y;
+      ex1 += f.x * (double)y.y - f.y * (double)y.x;
+    } else if (extra == kExtraGradOverlap) {
+      // an Sx control on site 1 couples the two amplitudes of the pair
+      float2 q = ((rc.sx_site == 0) != (x == 1)) ? make_float2(qp.z, qp.w) : make_float2(qp.x, qp.y);
+      const int nz = __popc(rc.mk) - 2 * __popc((unsigned)(gi + x) & rc.mk);
+      const float dz = (rc.sx_site >= 0) ? 0.5f * rc.h_amp : rc.h_amp * 0.5f * (float)nz;
       q.x *= dz;
       q.y *= dz;
+      gacc += (A)(y.x * q.y - y.y * q.x);  // Im(conj(y) q)
     }
-    gacc += (A)(y.x * q.y - y.y * q.x);  // Im(conj(y) q)
   }
 }
 
@@ -858,6 +860,10 @@ __device__ __forceinline__ bool finish_slice(Ctx<V>& c, const V* src, double nrm
     // The basis vectors are read newest first: the slice has just written all m of them (8 MB
     // each at L=20) and L2 still holds the latest ones, while in order of age every read would
     // evict the next vector needed before it is reached.
+    // The own pairs of psi_other follow the basis through the same copies (fetched after the
+    // recombination instead, their latency was all exposed).
+    const size_t flip = (p.hc_kind == KG_HC_SX_SITE && p.hc_site >= 1) ? (size_t)1 << p.hc_site : 0;
+    const bool grad = extra == kExtraGradOverlap, staged = grad && meff >= kRecombDepth;
     for (int i = 0; i < meff; ++i) {
       cp_async_wait<kRecombDepth - 1>();  // this thread's copies of basis vector k have landed
       const int k = meff - 1 - i;
@@ -876,11 +882,10 @@ __device__ __forceinline__ bool finish_slice(Ctx<V>& c, const V* src, double nrm
           }
         }
       }
-      if (i + kRecombDepth < meff) {
-        const int kn = meff - 1 - (i + kRecombDepth);
-        recomb_issue(kn == 0 ? (const float2*)src : slot1 + (size_t)(kn - 1) * D, rb, n_own,
-                     stg + (size_t)(i % kRecombDepth) * 8 * kThreads);
-      }
+      const int kn = meff - 1 - (i + kRecombDepth);
+      float4* st = stg + (size_t)(i % kRecombDepth) * 8 * kThreads;
+      if (kn >= 0) recomb_issue(kn == 0 ? (const float2*)src : slot1 + (size_t)(kn - 1) * D, rb, n_own, st);
+      else if (kn == -1 && staged) recomb_issue((const float2*)psi_other, rb, n_own, st, flip);
       cp_async_commit();
     }
     cp_async_wait<0>();
@@ -889,12 +894,15 @@ __device__ __forceinline__ bool finish_slice(Ctx<V>& c, const V* src, double nrm
     rc.mk = (unsigned)p.hc_mask;
     rc.sx_site = (p.hc_kind == KG_HC_SX_SITE) ? p.hc_site : -1;
     rc.h_amp = (float)p.hc_amp;
+    const float4* qs = stg + (size_t)(meff % kRecombDepth) * 8 * kThreads + tid;
     for (int ct = 0; ct < n_own; ++ct) {
 #pragma unroll
       for (int g = 0; g < 4; ++g) {
         const size_t gi = rb[ct] + 2 * (size_t)(tid + g * kThreads);
-        recomb_amp<A>(rc, gi, make_float2(y[ct][g].x, y[ct][g].y), dst, extra, psi_other, nacc, gacc, ex0, ex1);
-        recomb_amp<A>(rc, gi + 1, make_float2(y[ct][g].z, y[ct][g].w), dst, extra, psi_other, nacc, gacc, ex0, ex1);
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (staged) q = qs[(ct * 4 + g) * kThreads];
+        else if (grad) q = __ldcg(reinterpret_cast<const float4*>((const float2*)psi_other + (gi ^ flip)));
+        recomb_pair<A>(rc, gi, y[ct][g], dst, extra, q, nacc, gacc, ex0, ex1);
       }
     }
   } else {
