@@ -736,7 +736,11 @@ __device__ __forceinline__ void recomb_pair(const RecombConsts& rc, size_t gi, f
   }
 }
 
-template <class V, class A, int APT, bool WBASIS>
+constexpr int kStrRecombVecs = 4;  // streaming: basis vectors in flight (24 spins: 4 8.35 ms a slice, 3 8.79, 2 8.77)
+
+// WBASIS: the resident complex64 loops (basis of raw vectors W_k, tiles on chip).  STREAM: the complex64
+// streaming loop.
+template <class V, class A, int APT, bool WBASIS, bool STREAM>
 __device__ __forceinline__ bool finish_slice(Ctx<V>& c, const V* src, double nrm_src, double tau, V* dst, int extra,
                                              const V* psi_other, double& nrm_dst, double2& e, bool interior = false) {
   using R = typename VecTraits<V>::R;
@@ -904,6 +908,51 @@ __device__ __forceinline__ bool finish_slice(Ctx<V>& c, const V* src, double nrm
         else if (grad) q = __ldcg(reinterpret_cast<const float4*>((const float2*)psi_other + (gi ^ flip)));
         recomb_pair<A>(rc, gi, y[ct][g], dst, extra, q, nacc, gacc, ex0, ex1);
       }
+    }
+  } else if constexpr (STREAM) {
+    // Amplitude pairs 2 (tid + 512 g) + {0, 1} by 16-byte loads, kStrRecombVecs basis vectors in flight
+    // (newest first); the own pairs of psi_other are asked for first and used last.
+    const float2* slot1 = (const float2*)p.basis;
+    const size_t flip = (p.hc_kind == KG_HC_SX_SITE && p.hc_site >= 1) ? (size_t)1 << p.hc_site : 0;
+    RecombConsts rc;
+    rc.target = reinterpret_cast<const double2*>(p.target);
+    rc.mk = (unsigned)p.hc_mask;
+    rc.sx_site = (p.hc_kind == KG_HC_SX_SITE) ? p.hc_site : -1;
+    rc.h_amp = (float)p.hc_amp;
+    for (int ct = 0; ct < c.n_own; ++ct) {
+      const size_t base = c.tile_base(ct);
+      float4 y[4], qp[4];
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const size_t gi = base + 2 * (size_t)(tid + g * kThreads);
+        y[g] = qp[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (extra == kExtraGradOverlap) qp[g] = __ldcg(reinterpret_cast<const float4*>((const float2*)psi_other + (gi ^ flip)));
+      }
+      for (int k0 = meff - 1; k0 >= 0; k0 -= kStrRecombVecs) {
+        float4 q[kStrRecombVecs][4];
+#pragma unroll
+        for (int u = 0; u < kStrRecombVecs; ++u) {
+          const int k = k0 - u;
+          const float4* v = reinterpret_cast<const float4*>(((k <= 0) ? (const float2*)src : slot1 + (size_t)(k - 1) * c.D) + base) + tid;
+#pragma unroll
+          for (int g = 0; g < 4; ++g) q[u][g] = (k >= 0) ? __ldcg(v + g * kThreads) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < kStrRecombVecs; ++u) {
+          const int k = k0 - u;
+          const float a = (k >= 0) ? ss.coef_re_f[k] : 0.f, b = (k >= 0) ? ss.coef_im_f[k] : 0.f;
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            y[g].x += a * q[u][g].x - b * q[u][g].y;
+            y[g].y += a * q[u][g].y + b * q[u][g].x;
+            y[g].z += a * q[u][g].z - b * q[u][g].w;
+            y[g].w += a * q[u][g].w + b * q[u][g].z;
+          }
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+        recomb_pair<A>(rc, base + 2 * (size_t)(tid + g * kThreads), y[g], (float2*)dst, extra, qp[g], nacc, gacc, ex0, ex1);
     }
   } else {
     for (int ct = 0; ct < c.n_own; ++ct) {
@@ -2376,7 +2425,7 @@ __device__ __noinline__ bool krylov_slice(Ctx<V>& c, const V* src, double nrm_sr
   else if constexpr (MODE == kModeStream64) ok = lanczos_str64(c, src, nrm_src, uj);
   else ok = lanczos_generic<V, A, APT, TPC, RES>(c, src, nrm_src, uj);
   if (!ok) return false;
-  return finish_slice<V, A, APT, MODE == kModeResident64 || MODE == kModeResident64b>(c, src, nrm_src, tau, dst, extra,
+  return finish_slice<V, A, APT, MODE == kModeResident64 || MODE == kModeResident64b, MODE == kModeStream64>(c, src, nrm_src, tau, dst, extra,
                                                                                      psi_other, nrm_dst, e);
 }
 
@@ -2387,7 +2436,7 @@ template <class V, class A, int APT, int TPC, bool RES, int MODE>
 __device__ __noinline__ bool interior_step(Ctx<V>& c, const V* src, double nrm_src, double tau, V* dst, int extra,
                                            const V* psi_other, double2& e) {
   double nrm_dst;
-  return finish_slice<V, A, APT, MODE == kModeResident64 || MODE == kModeResident64b>(c, src, nrm_src, tau, dst, extra,
+  return finish_slice<V, A, APT, MODE == kModeResident64 || MODE == kModeResident64b, MODE == kModeStream64>(c, src, nrm_src, tau, dst, extra,
                                                                                      psi_other, nrm_dst, e, true);
 }
 
