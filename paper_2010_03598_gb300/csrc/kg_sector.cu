@@ -156,8 +156,8 @@ struct SecSmem {
   float2 ff_a[kMaxM], ff_n[kMaxM], ff_q[kMaxM], ff_e[kMaxM];  // the steps' sums; ff_e: b_{k+1}^2 (complex64),
                                                               // or the explicit one (float-float)
   float2 tau_ff[3];            // complex64: dt and the interior quadrature nodes
-  float2 diag_ff[2];           // Jz / 4 and hc_amp / 2
-  double diag_d[2];
+  float2 diag_ff[4];           // Jz / 4, hc_amp / 2, weights of lists A and B: float-float
+  double diag_d[4];
   float coef_f[3][2][kMaxM];   // [slice end, interior node a, b][re, im][k]
   double coef_d[3][2][kMaxM];
   float err_max;
@@ -307,12 +307,46 @@ __device__ __forceinline__ double sec_unpack(double d) {
   else return d;
 }
 
+// The diagonals of H0 and of Hc on the row of state st: a weight (float-float, so that FP32 and
+// float-float need no FP64 instruction) times a small whole number.
+__device__ __forceinline__ float sec_times(const SecSmem& sm, int which, int n, float) {
+  const float2 q = sm.diag_ff[which];
+  return fmaf(q.x, (float)n, q.y * (float)n);
+}
+// The weights of lists A (2) and B (3) in the vectors' real type.  Complex64: converted from the
+// parameters, which the compiler does once; float-float and complex128: from shared memory, as their
+// conversion or constant operand in the loop costs FP64 issue (2 and 7 % at D = 2445).
+__device__ __forceinline__ float sec_weight(const SectorParams& p, const SecSmem&, int which, float) {
+  return (float)(which == 2 ? p.wa : p.wb);
+}
+__device__ __forceinline__ FFR sec_weight(const SectorParams&, const SecSmem& sm, int which, FFR) {
+  return FFR(sm.diag_ff[which].x, sm.diag_ff[which].y);
+}
+__device__ __forceinline__ double sec_weight(const SectorParams&, const SecSmem& sm, int which, double) {
+  return sm.diag_d[which];
+}
+__device__ __forceinline__ FFR sec_times(const SecSmem& sm, int which, int n, FFR) {
+  const float2 q = sm.diag_ff[which];
+  return ffr_of(ff_mul(FF{q.x, q.y}, FF{(float)n, 0.f}));
+}
+__device__ __forceinline__ double sec_times(const SecSmem& sm, int which, int n, double) {
+  return sm.diag_d[which] * (double)n;
+}
+template <class R>
+__device__ __forceinline__ R sec_d0(const SectorParams& p, const SecSmem& sm, unsigned st) {
+  return sec_times(sm, 0, p.L1 - 2 * __popc((st ^ (st >> 1)) & p.maskL1), R());
+}
+template <class R>
+__device__ __forceinline__ R sec_hc(const SectorParams& p, const SecSmem& sm, unsigned st) {
+  return sec_times(sm, 1, __popc(p.hc_mask) - 2 * __popc(st & p.hc_mask), R());
+}
+
 // ---------------------------------------------------------------- H in the subspace
 // h = (diagonal + H0's couplings) x - bk xp on the own rows; S holds x for the gather (element D is 0).
 // The words of list A are read row by row in step, so that every thread has its rows' loads in flight
 // together.
 template <class V, int NT, int RPT>
-__device__ __forceinline__ void sec_apply(const SectorParams& p, const V* S, const unsigned* tab,
+__device__ __forceinline__ void sec_apply(const SectorParams& p, const SecSmem& sm, const V* S, const unsigned* tab,
                                           const typename VecTraits<V>::R (&dj)[RPT], const V (&x)[RPT],
                                           typename VecTraits<V>::R bk, const V (&xp)[RPT], V (&h)[RPT]) {
   using R = typename VecTraits<V>::R;
@@ -321,7 +355,7 @@ __device__ __forceinline__ void sec_apply(const SectorParams& p, const V* S, con
   const unsigned* ta = tab + min(tid, D);
   const unsigned* meta = tab + p.na2 * p.rows;
   const unsigned* tb = meta + p.groups + (tid & 31);
-  const R wa = (R)p.wa;
+  const R wa = sec_weight(p, sm, 2, R());
   if constexpr (FFM) {
     FF ax[RPT], ay[RPT];
 #pragma unroll
@@ -364,7 +398,7 @@ __device__ __forceinline__ void sec_apply(const SectorParams& p, const V* S, con
     const int g = (tid >> 5) + (NT / 32) * i;
     if (g < p.groups) {
       const unsigned mt = meta[g];
-      const R wb = (R)p.wb;
+      const R wb = sec_weight(p, sm, 3, R());
       for (unsigned q = 0; q < (mt & 0xffu); ++q) {
         const unsigned w = tb[(mt >> 8) + 32 * q];
         h[i] = vaxpy<V>(wb, S[w & 0xffffu], h[i]);
@@ -372,28 +406,6 @@ __device__ __forceinline__ void sec_apply(const SectorParams& p, const V* S, con
       }
     }
   }
-}
-
-// The diagonals of H0 and of Hc on the row of state st: a weight (float-float, so that FP32 and
-// float-float need no FP64 instruction) times a small whole number.
-__device__ __forceinline__ float sec_times(const SecSmem& sm, int which, int n, float) {
-  const float2 q = sm.diag_ff[which];
-  return fmaf(q.x, (float)n, q.y * (float)n);
-}
-__device__ __forceinline__ FFR sec_times(const SecSmem& sm, int which, int n, FFR) {
-  const float2 q = sm.diag_ff[which];
-  return ffr_of(ff_mul(FF{q.x, q.y}, FF{(float)n, 0.f}));
-}
-__device__ __forceinline__ double sec_times(const SecSmem& sm, int which, int n, double) {
-  return sm.diag_d[which] * (double)n;
-}
-template <class R>
-__device__ __forceinline__ R sec_d0(const SectorParams& p, const SecSmem& sm, unsigned st) {
-  return sec_times(sm, 0, p.L1 - 2 * __popc((st ^ (st >> 1)) & p.maskL1), R());
-}
-template <class R>
-__device__ __forceinline__ R sec_hc(const SectorParams& p, const SecSmem& sm, unsigned st) {
-  return sec_times(sm, 1, __popc(p.hc_mask) - 2 * __popc(st & p.hc_mask), R());
 }
 
 // Taylor-hierarchy terms of backward slice j (App. B, Eq. gradp), this thread's partial sum:
@@ -435,7 +447,7 @@ __device__ __noinline__ typename VecTraits<V>::R sec_taylor(const SectorParams& 
     if (r < D) Sa[r] = b0[i];
   }
   sec_sync();
-  sec_apply<V, NT, RPT>(p, Sa, tab, dj, b0, (R)0, b2, b1);
+  sec_apply<V, NT, RPT>(p, sm, Sa, tab, dj, b0, (R)0, b2, b1);
   if (taylor >= 2) {
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
@@ -443,7 +455,7 @@ __device__ __noinline__ typename VecTraits<V>::R sec_taylor(const SectorParams& 
       if (r < D) Sb[r] = b1[i];
     }
     sec_sync();
-    sec_apply<V, NT, RPT>(p, Sb, tab, dj, b1, (R)0, b0, b2);
+    sec_apply<V, NT, RPT>(p, sm, Sb, tab, dj, b1, (R)0, b0, b2);
   }
   const R al0 = (meff > 0) ? (F32 ? (R)sm.alpha_f[0] : (R)sm.alpha[0]) : (R)0;
   const R al1 = (meff > 1) ? (F32 ? (R)sm.alpha_f[1] : (R)sm.alpha[1]) : (R)0;
@@ -643,7 +655,7 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
   for (int k = 0; k < meff; ++k) {
     const bool last = (k == m - 1);
     sec_sync();  // v_k is in shared memory
-    sec_apply<V, NT, RPT>(p, Sc, tab, dj, v, bk, vp, w);
+    sec_apply<V, NT, RPT>(p, sm, Sc, tab, dj, v, bk, vp, w);
     A pa = A(), pn = A(), pq = A();
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
@@ -1047,14 +1059,14 @@ __global__ void __launch_bounds__(NT, (sec_min_blocks<V, NT>())) kg_sector_kerne
   if (threadIdx.x == 0) {
     S0[p.D] = S1[p.D] = vmake<V>(0, 0);  // what the tables' padding points at
     const double sa = 0.5 * p.dt * (1.0 - 1.0 / ::sqrt(5.0));
-    const double w[5] = {p.qz, 0.5 * p.hc_amp, p.dt, sa, p.dt - sa};
-    for (int i = 0; i < 5; ++i) {
+    const double w[7] = {p.qz, 0.5 * p.hc_amp, p.wa, p.wb, p.dt, sa, p.dt - sa};
+    for (int i = 0; i < 7; ++i) {
       const FF f = ff_from_double(w[i]);
-      if (i < 2) {
+      if (i < 4) {
         sm.diag_d[i] = w[i];
         sm.diag_ff[i] = make_float2(f.hi, f.lo);
       } else {
-        sm.tau_ff[i - 2] = make_float2(f.hi, f.lo);
+        sm.tau_ff[i - 4] = make_float2(f.hi, f.lo);
       }
     }
   }
