@@ -63,8 +63,11 @@ struct FFR {
   __device__ __forceinline__ explicit operator double() const { return (double)hi + (double)lo; }
   __device__ __forceinline__ explicit operator float() const { return __fadd_rn(hi, lo); }
 };
+// A complex amplitude: high parts of (re, im), then low parts, so that the packed FP32x2 instructions work
+// on both components at once: half the instructions of two scalar float-float numbers, which the
+// kernel's issue slots bound.
 struct __align__(16) FFC {
-  FFR x, y;
+  float2 hi, lo;
 };
 __device__ __forceinline__ FFR operator+(FFR a, FFR b) {
   const FF s = ff_add(FF{a.hi, a.lo}, FF{b.hi, b.lo});
@@ -91,29 +94,73 @@ __device__ __forceinline__ void ff_rsqrt(FF a, FF& root, FF& inv) {
   inv = ff_two_sum(y, __fmul_rn(__fmul_rn(y, r), __fmaf_rn(0.375f, r, 0.5f)));
   root = ff_mul(a, inv);
 }
+// The float-float operations on both components (packed FP32x2; see ff_two_sum, ff_mul, ff_dot3).
+__device__ __forceinline__ float2 p2_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 p2_sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 p2_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 p2_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 p2_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ FFC ffc_two_sum(float2 a, float2 b) {
+  const float2 s = p2_add(a, b), bb = p2_sub(s, a);
+  return {s, p2_add(p2_sub(a, p2_sub(s, bb)), p2_sub(b, bb))};
+}
+__device__ __forceinline__ FFC ffc_close(float2 hi, float2 lo) {  // renormalised hi + lo, |lo| << |hi|
+  const float2 h = p2_add(hi, lo);
+  return {h, p2_sub(lo, p2_sub(h, hi))};
+}
+__device__ __forceinline__ FFC ffc_bcast(FFR a) { return {make_float2(a.hi, a.hi), make_float2(a.lo, a.lo)}; }
+// a b = p + t: the products by FMA TwoProduct with the cross terms in t
+__device__ __forceinline__ void ffc_prod(FFC a, FFC b, float2& p, float2& t) {
+  p = p2_mul(a.hi, b.hi);
+  t = p2_fma(a.hi, b.lo, p2_fma(a.lo, b.hi, p2_fma(a.hi, b.hi, p2_neg(p))));
+}
+__device__ __forceinline__ FFC ffc_mul(FFC a, FFC b) {
+  float2 p, t;
+  ffc_prod(a, b, p, t);
+  return ffc_close(p, t);
+}
+__device__ __forceinline__ FFC ffc_fma(FFC a, FFC b, FFC c) {  // a b + c
+  float2 p, t;
+  ffc_prod(a, b, p, t);
+  const FFC s = ffc_two_sum(c.hi, p);
+  return ffc_close(s.hi, p2_add(s.lo, p2_add(t, c.lo)));
+}
+__device__ __forceinline__ FFC ffc_dot3(FFC a, FFC x, FFC b, FFC y, FFC c, FFC z) {
+  float2 p, q, r, tp, tq, tr;
+  ffc_prod(a, x, p, tp);
+  ffc_prod(b, y, q, tq);
+  ffc_prod(c, z, r, tr);
+  const FFC s = ffc_two_sum(p, r), u = ffc_two_sum(s.hi, q);
+  return ffc_close(u.hi, p2_add(p2_add(p2_add(tp, tr), tq), p2_add(s.lo, u.lo)));
+}
 // Unevaluated sum of many float-float terms: the high parts by TwoSum, everything below them in one FP32
-// accumulator; ff_close renormalises once at the end.
-__device__ __forceinline__ void ff_acc(FF& a, FFR v) {
-  const FF s = ff_two_sum(a.hi, v.hi);
+// accumulator; ffc_close renormalises once at the end.
+__device__ __forceinline__ void ffc_acc(FFC& a, FFC v) {
+  const FFC s = ffc_two_sum(a.hi, v.hi);
   a.hi = s.hi;
-  a.lo = __fadd_rn(a.lo, __fadd_rn(s.lo, v.lo));
+  a.lo = p2_add(a.lo, p2_add(s.lo, v.lo));
 }
-__device__ __forceinline__ void ff_acc_mul(FF& a, FFR x, FFR y) {  // a += x y
-  const float p = __fmul_rn(x.hi, y.hi);
-  const float t = __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, __fmaf_rn(x.hi, y.hi, -p)));
-  const FF s = ff_two_sum(a.hi, p);
+__device__ __forceinline__ void ffc_acc_mul(FFC& a, FFC x, FFC y) {  // a += x y, by component
+  float2 p, t;
+  ffc_prod(x, y, p, t);
+  const FFC s = ffc_two_sum(a.hi, p);
   a.hi = s.hi;
-  a.lo = __fadd_rn(a.lo, __fadd_rn(s.lo, t));
-}
-__device__ __forceinline__ FF ff_close(FF a) {
-  const float hi = __fadd_rn(a.hi, a.lo);
-  return {hi, __fsub_rn(a.lo, __fsub_rn(hi, a.hi))};
+  a.lo = p2_add(a.lo, p2_add(s.lo, t));
 }
 __device__ __forceinline__ FF ff_of(FFR a) { return FF{a.hi, a.lo}; }
 __device__ __forceinline__ FFR ffr_of(FF a) { return FFR(a.hi, a.lo); }
 using ::fma;  // the float and double functions stay visible beside the overload inside namespace kg
 template <> struct VecTraits<FFC> { using R = FFR; };
-template <> __device__ __forceinline__ FFC vmake<FFC>(FFR a, FFR b) { return FFC{a, b}; }
+template <> __device__ __forceinline__ FFC vmake<FFC>(FFR a, FFR b) {
+  return FFC{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)};
+}
+// The components of an amplitude.
+__device__ __forceinline__ float vre(float2 a) { return a.x; }
+__device__ __forceinline__ float vim(float2 a) { return a.y; }
+__device__ __forceinline__ double vre(double2 a) { return a.x; }
+__device__ __forceinline__ double vim(double2 a) { return a.y; }
+__device__ __forceinline__ FFR vre(FFC a) { return FFR(a.hi.x, a.lo.x); }
+__device__ __forceinline__ FFR vim(FFC a) { return FFR(a.hi.y, a.lo.y); }
 
 
 struct SectorParams {
@@ -228,10 +275,23 @@ __device__ __forceinline__ void sec_record(SecSmem& sm, int k, int check) {
 }
 
 template <class V> __device__ __forceinline__ V vscale(typename VecTraits<V>::R a, V x) {
-  return vmake<V>(a * x.x, a * x.y);
+  if constexpr (std::is_same<V, FFC>::value) return ffc_mul(ffc_bcast(a), x);
+  else return vmake<V>(a * x.x, a * x.y);
 }
 template <class V> __device__ __forceinline__ V vaxpy(typename VecTraits<V>::R a, V x, V y) {
-  return vmake<V>(fma(a, x.x, y.x), fma(a, x.y, y.y));
+  if constexpr (std::is_same<V, FFC>::value) return ffc_fma(ffc_bcast(a), x, y);
+  else return vmake<V>(fma(a, x.x, y.x), fma(a, x.y, y.y));
+}
+// (a + ib) x + y, the part with b first
+template <class V>
+__device__ __forceinline__ V vcaxpy(typename VecTraits<V>::R a, typename VecTraits<V>::R b, V x, V y) {
+  if constexpr (std::is_same<V, FFC>::value) {
+    const FFC fb{make_float2(-b.hi, b.hi), make_float2(-b.lo, b.lo)};
+    const FFC xs{make_float2(x.hi.y, x.hi.x), make_float2(x.lo.y, x.lo.x)}, one = ffc_bcast(FFR(1));
+    return ffc_dot3(ffc_bcast(a), x, fb, xs, one, y);
+  } else {
+    return vmake<V>(fma(a, x.x, fma(-b, x.y, y.x)), fma(a, x.y, fma(b, x.x, y.y)));
+  }
 }
 
 // ---------------------------------------------------------------- per-precision scalars
@@ -249,15 +309,18 @@ template <> struct SecPrec<double2> {
   using S = double;
   using N = double;
 };
-// Per-row partial sums: acc += x y.
-__device__ __forceinline__ void sacc(float& a, float x, float y) { a = fmaf(x, y, a); }
-__device__ __forceinline__ void sacc(double& a, double x, double y) { a = ::fma(x, y, a); }
-__device__ __forceinline__ void sacc(FF& a, FFR x, FFR y) { ff_acc_mul(a, x, y); }
+// Per-row partial sums: acc += Re(conj(x) y) (float-float: by component, added up in sclose).
+__device__ __forceinline__ void sacc(float& a, float2 x, float2 y) { a = fmaf(x.y, y.y, fmaf(x.x, y.x, a)); }
+__device__ __forceinline__ void sacc(double& a, double2 x, double2 y) { a = ::fma(x.y, y.y, ::fma(x.x, y.x, a)); }
+__device__ __forceinline__ void sacc(FFC& a, FFC x, FFC y) { ffc_acc_mul(a, x, y); }
 __device__ __forceinline__ float sclose(float a) { return a; }
 __device__ __forceinline__ double sclose(double a) { return a; }
-__device__ __forceinline__ FF sclose(FF a) { return ff_close(a); }
-template <class R> struct SecAcc { using T = R; };
-template <> struct SecAcc<FFR> { using T = FF; };
+__device__ __forceinline__ FF sclose(FFC a) {
+  const FFC c = ffc_close(a.hi, a.lo);
+  return ff_add(FF{c.hi.x, c.lo.x}, FF{c.hi.y, c.lo.y});
+}
+template <class V> struct SecAcc { using T = typename VecTraits<V>::R; };
+template <> struct SecAcc<FFC> { using T = FFC; };
 
 // alpha_k, b_{k+1} and 1/b_{k+1} from a step's sums (or from an explicit b_{k+1}^2).
 __device__ __forceinline__ FF sec_b2(const FF (&o)[3]) {
@@ -357,27 +420,21 @@ __device__ __forceinline__ void sec_apply(const SectorParams& p, const SecSmem& 
   const unsigned* tb = meta + p.groups + (tid & 31);
   const R wa = sec_weight(p, sm, 2, R());
   if constexpr (FFM) {
-    FF ax[RPT], ay[RPT];
+    FFC acc[RPT];
 #pragma unroll
-    for (int i = 0; i < RPT; ++i) ax[i] = ay[i] = FF{0.f, 0.f};
+    for (int i = 0; i < RPT; ++i) acc[i] = FFC{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     for (int q = 0; q < p.na2; ++q) {
 #pragma unroll
       for (int i = 0; i < RPT; ++i) {
         const unsigned w = (tid + NT * i <= D) ? ta[q * p.rows + NT * i] : tab[q * p.rows + D];
-        const V a = S[w & 0xffffu], b = S[w >> 16];
-        ff_acc(ax[i], a.x);
-        ff_acc(ay[i], a.y);
-        ff_acc(ax[i], b.x);
-        ff_acc(ay[i], b.y);
+        ffc_acc(acc[i], S[w & 0xffffu]);
+        ffc_acc(acc[i], S[w >> 16]);
       }
     }
-    const FF wf = ff_of(wa), nb = ff_of(-bk);
+    const FFC wf = ffc_bcast(wa), nb = ffc_bcast(-bk);
 #pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      const FF d = ff_of(dj[i]);
-      h[i].x = ffr_of(ff_dot3(d, ff_of(x[i].x), wf, ff_close(ax[i]), nb, ff_of(xp[i].x)));
-      h[i].y = ffr_of(ff_dot3(d, ff_of(x[i].y), wf, ff_close(ay[i]), nb, ff_of(xp[i].y)));
-    }
+    for (int i = 0; i < RPT; ++i)
+      h[i] = ffc_dot3(ffc_bcast(dj[i]), x[i], wf, ffc_close(acc[i].hi, acc[i].lo), nb, xp[i]);
   } else {
 #pragma unroll
     for (int i = 0; i < RPT; ++i) h[i] = vscale<V>(dj[i], x[i]);
@@ -619,7 +676,7 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
                                           typename SecPrec<V>::N& tay, int lob, V* tint_io, float2 fact) {
   using R = typename VecTraits<V>::R;
   using S = typename SecPrec<V>::S;
-  using A = typename SecAcc<R>::T;
+  using A = typename SecAcc<V>::T;
   constexpr bool F32 = sizeof(R) == 4;
   constexpr bool FFM = std::is_same<R, FFR>::value;  // float-float vectors (KG_PREC_FF)
   const int tid = threadIdx.x, D = p.D, m = p.m;
@@ -659,12 +716,9 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
     A pa = A(), pn = A(), pq = A();
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
-      sacc(pa, v[i].x, w[i].x);
-      sacc(pa, v[i].y, w[i].y);
-      sacc(pn, w[i].x, w[i].x);
-      sacc(pn, w[i].y, w[i].y);
-      sacc(pq, v[i].x, v[i].x);
-      sacc(pq, v[i].y, v[i].y);
+      sacc(pa, v[i], w[i]);
+      sacc(pn, w[i], w[i]);
+      sacc(pq, v[i], v[i]);
     }
     sec_mark(p, sm, 0);
     S o[3];
@@ -691,11 +745,10 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
           const V d = vaxpy<V>(-alpha, v[i], w[i]);
-          sacc(e, d.x, d.x);
-          sacc(e, d.y, d.y);
+          sacc(e, d, d);
         }
         S oe[3];
-        sec_reduce<NT>(sm, par, sclose(e), A(), A(), oe);
+        sec_reduce<NT>(sm, par, sclose(e), sclose(A()), sclose(A()), oe);
         b2 = oe[0];
         sec_roots(b2, bk, ib);
         if constexpr (FFM) {
@@ -795,14 +848,7 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
         const R b = F32 ? (R)sm.coef_f[0][1][k] : (R)sm.coef_d[0][1][k];
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
-          if constexpr (FFM) {
-            const FF nb = ff_of(-b), fa = ff_of(a), fb = ff_of(b), one{1.f, 0.f};
-            y[i] = V{ffr_of(ff_dot3(fa, ff_of(q[u][i].x), nb, ff_of(q[u][i].y), one, ff_of(y[i].x))),
-                     ffr_of(ff_dot3(fa, ff_of(q[u][i].y), fb, ff_of(q[u][i].x), one, ff_of(y[i].y)))};
-          } else {
-            y[i].x = fma(a, q[u][i].x, fma(-b, q[u][i].y, y[i].x));
-            y[i].y = fma(a, q[u][i].y, fma(b, q[u][i].x, y[i].y));
-          }
+          y[i] = vcaxpy<V>(a, b, q[u][i], y[i]);
         }
       }
     }
@@ -813,10 +859,10 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
     const int r = tid + NT * i;
     if (r < D) {
       if (dst) dst[r] = y[i];
-      pn = fma(y[i].x, y[i].x, fma(y[i].y, y[i].y, pn));
+      pn = fma(vre(y[i]), vre(y[i]), fma(vim(y[i]), vim(y[i]), pn));
       if (back) {
         const V o = other[r];
-        pg = fma(sec_hc<R>(p, sm, __ldg(p.states + r)), y[i].x * o.y - y[i].y * o.x, pg);  // Im(conj(y) Hc o), Hc diagonal
+        pg = fma(sec_hc<R>(p, sm, __ldg(p.states + r)), vre(y[i]) * vim(o) - vim(y[i]) * vre(o), pg);  // Im(conj(y) Hc o)
       }
     }
     x[i] = y[i];
@@ -929,7 +975,8 @@ __device__ __forceinline__ void sec_eval(const SectorParams& p, int b, SecSmem& 
         const double2 q = psi0[r];
         x[i] = vmake<V>((R)q.x, (R)q.y);
         traj[r] = x[i];
-        acc = ::fma((double)x[i].x, (double)x[i].x, ::fma((double)x[i].y, (double)x[i].y, acc));
+        const double re = (double)vre(x[i]), im = (double)vim(x[i]);
+        acc = ::fma(re, re, ::fma(im, im, acc));
       }
     }
     sec_reduce<NT>(sm, par, acc, 0.0, 0.0, o);
@@ -972,7 +1019,7 @@ __device__ __forceinline__ void sec_eval(const SectorParams& p, int b, SecSmem& 
         const int r = tid + NT * i;
         if (r < D) {
           const double2 f = tgt[r];
-          const double xr = (double)x[i].x, xi = (double)x[i].y;
+          const double xr = (double)vre(x[i]), xi = (double)vim(x[i]);
           a0 = ::fma(f.x, xr, ::fma(f.y, xi, a0));   // Re(conj(f) x)
           a1 = ::fma(f.x, xi, ::fma(-f.y, xr, a1));  // Im(conj(f) x)
         }
@@ -991,9 +1038,9 @@ __device__ __forceinline__ void sec_eval(const SectorParams& p, int b, SecSmem& 
         if (r < D) {
           const double2 f = tgt[r];
           c = vmake<V>((R)(br * f.x - bi * f.y), (R)(br * f.y + bi * f.x));
-          const double cr = (double)c.x, ci = (double)c.y;
+          const double cr = (double)vre(c), ci = (double)vim(c);
           a0 = ::fma(cr, cr, ::fma(ci, ci, a0));
-          a1 = ::fma((double)sec_hc<R>(p, sm, __ldg(p.states + r)), cr * (double)x[i].y - ci * (double)x[i].x, a1);
+          a1 = ::fma((double)sec_hc<R>(p, sm, __ldg(p.states + r)), cr * (double)vim(x[i]) - ci * (double)vre(x[i]), a1);
         }
         x[i] = c;
       }
