@@ -595,7 +595,8 @@ __device__ __noinline__ typename VecTraits<V>::R sec_interior(const SectorParams
 // the pulse's time limit.
 template <class V>
 __device__ __forceinline__ void sec_coefficients(const SectorParams& p, SecSmem& sm, int w, bool back, int meff,
-                                                 bool broke, float beta_m, typename SecPrec<V>::N nrm, float2 fact) {
+                                                 bool broke, float beta_m, typename SecPrec<V>::N nrm, float inv,
+                                                 float2 fact) {
   using R = typename VecTraits<V>::R;
   constexpr bool F32 = sizeof(R) == 4;
   const int k = threadIdx.x & 31;
@@ -620,7 +621,10 @@ __device__ __forceinline__ void sec_coefficients(const SectorParams& p, SecSmem&
     const FF t = back ? FF{-t2.x, -t2.y} : FF{t2.x, t2.y};
     FF fr{0.f, 0.f}, fi{0.f, 0.f};
     if (meff > 0 && sane) tridiag_expv_e1_fff(FF{a2.x, a2.y}, ff_sqrt(FF{b2.x, b2.y}), meff, t, 1e-13f, fact, fr, fi, tnorm);
-    const FF cr = ff_mul(fr, nrm), ci = ff_mul(fi, nrm);
+    // v_0 = inv x with inv rounded to FP32: 1 / inv, not ||x||, takes the rounding out again (with ||x||
+    // every slice would multiply the state's norm by ||x|| inv)
+    const FF sc = (inv > 0.f) ? ff_rcp(FF{inv, 0.f}) : nrm;
+    const FF cr = ff_mul(fr, sc), ci = ff_mul(fi, sc);
     cre = __fadd_rn(cr.hi, cr.lo);
     cim = __fadd_rn(ci.hi, ci.lo);
     n0 = nrm.hi;
@@ -821,7 +825,7 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
     }
   }
   if (lob) sec_sync();  // T is read by warps 1 and 2 as well
-  if (tid < (lob ? 96 : 32)) sec_coefficients<V>(p, sm, tid >> 5, back, meff, broke, beta_m, nrm, fact);
+  if (tid < (lob ? 96 : 32)) sec_coefficients<V>(p, sm, tid >> 5, back, meff, broke, beta_m, nrm, F32 ? (float)sec_f32(inv) : 0.f, fact);
   sec_sync();
   if (sm.abort) return false;
   sec_mark(p, sm, 4);
@@ -882,9 +886,9 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
   if constexpr (F32) {
     FF o[3];
     sec_reduce<NT>(sm, par, pn, pg, pt, o);
-    nrm = ff_sqrt(o[0]);
-    const float n = __fadd_rn(nrm.hi, nrm.lo);
-    inv = (n > 0.f) ? __frcp_rn(n) : 0.f;
+    FF id;
+    ff_rsqrt(o[0], nrm, id);
+    inv = __fadd_rn(id.hi, id.lo);
     ex = o[1];
     tay = o[2];
     if (!isfinite(o[0].hi)) {

@@ -149,3 +149,24 @@ def test_invariant_and_nearly_invariant_subspaces(L, prec):
         # the eigenstate): its rounding is that of the overlap, held to the tolerance on F
         assert np.linalg.norm(gr - g_ref) <= TOL[prec][0] * 2 * dt * np.sqrt(N)
         assert rep["status"] == 0 and rep["breakdowns"] >= (N if share == 0.0 else 0)
+
+
+@pytest.mark.parametrize("dt", [0.2, 0.5])
+def test_subspace_norm_does_not_drift_in_complex64(dt):
+    # 2000 slices on D = 28: FP32 rounding of the states walks by about 6e-8 per slice (sqrt(N) of it, x4 margin)
+    import oracle.sector as OS
+    from paper_2010_03598_gb300 import api as A
+    c = OS.paper_chain(8, 3, 1)
+    N = 2000
+    rng = np.random.default_rng(5)
+    psi0 = rng.standard_normal(c.D) + 1j * rng.standard_normal(c.D)
+    psi0 /= np.linalg.norm(psi0)
+    dev = torch.device("cuda", 0)
+    eng = A.KGrapeSector(A.SectorSpec(8, 3, 1), A.Options(N, dt, 12, prec="c64", grad="none"), B=1)
+    u = torch.tensor(rng.uniform(-1, 1, (1, N)), device=dev)
+    p = torch.tensor(psi0, device=dev)
+    eng.evaluate(u, p, p)
+    rep = eng.sync()
+    assert rep["status"] == 0
+    assert abs(rep["norm_final"] - 1.0) <= 4 * 6e-8 * np.sqrt(N) + 1e-7
+    eng.close()
