@@ -21,11 +21,15 @@
 // Several CTAs: the stencil acts on the raw vector W_k, which needs none of the step's
 // scalars, so that it runs while the group's sums are under way:
 //   v_k = (W_k - alpha_{k-1} v_{k-1}) / b_k,   H v_k = (H W_k - alpha_{k-1} H v_{k-1}) / b_k.
-// (On one CTA the waits it would hide are short, and H v_k by its recurrence carries more rounding.)  The tiles' W_k are exchanged through global memory.  A control warp posts
-// the CTA's sums and the group's barrier in one message, a 16-byte {value, sequence number} per sum:
-// every CTA polls the other CTAs' messages and adds them up in the same order, so that one trip
-// through L2 both closes the step and carries its sums.
+// (On one CTA the waits it would hide are short, and H v_k by its recurrence carries more rounding.)  A
+// control warp posts the CTA's sums in 16-byte {values, sequence number} messages: every CTA polls the
+// other CTAs' messages and adds them up in the same order.  The tiles' W_k are exchanged through global
+// memory: complex64 in such messages as well, which their readers poll, so that a step is one trip
+// through L2; complex128 (16-byte amplitudes) as plain data, which a fence before the sums' message
+// makes visible, and which is copied once the sums have arrived.
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "kg_device.cuh"
 #include "kg_launch.h"
@@ -146,6 +150,7 @@ struct TileSmem {
   float err_max;
   int breakdowns;
   int cmd, ok;               // control warp: hand-over and answer
+  int lost;                  // a worker gave up waiting for partner amplitudes
   long long prof_last, prof_acc[8];
 };
 
@@ -168,7 +173,27 @@ __device__ __forceinline__ ulonglong2 ld_msg(const ulonglong2* p) {
 __device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 constexpr int kTileBarPost = 2, kTileBarGroup = 3;
-constexpr int kTileCmdSums = 1, kTileCmdExit = 2, kTileCmdFp64 = 8;  // bit 2: the reduction's parity
+constexpr int kTileCmdSums = 1, kTileCmdExit = 2, kTileCmdFp64 = 8, kTileCmdFence = 16;  // bit 2: the reduction's parity
+
+// A 16-byte message of three floats and a sequence number.
+struct Atom {
+  float f[3];
+  unsigned seq;
+};
+__device__ __forceinline__ void st_atom(ulonglong2* p, float a, float b, float c, unsigned seq) {
+  asm volatile("{\n .reg .b128 q;\n .reg .b64 x, y;\n mov.b64 x, {%1, %2};\n mov.b64 y, {%3, %4};\n mov.b128 q, {x, y};\n"
+               " st.relaxed.gpu.global.b128 [%0], q;\n}" ::"l"(p), "f"(a), "f"(b), "f"(c), "r"(seq)
+               : "memory");
+}
+__device__ __forceinline__ Atom ld_atom(const ulonglong2* p) {
+  Atom a;
+  asm volatile("{\n .reg .b128 q;\n .reg .b64 x, y;\n ld.relaxed.gpu.global.b128 q, [%4];\n mov.b128 {x, y}, q;\n"
+               " mov.b64 {%0, %1}, x;\n mov.b64 {%2, %3}, y;\n}"
+               : "=f"(a.f[0]), "=f"(a.f[1]), "=f"(a.f[2]), "=r"(a.seq)
+               : "l"(p)
+               : "memory");
+  return a;
+}
 
 template <class V, int NT, int APT, bool SB, bool MULTI>
 struct Tile {
@@ -181,6 +206,7 @@ struct Tile {
   static constexpr int LA = (APT == 1) ? 0 : (APT == 2) ? 1 : (APT == 4) ? 2 : (APT == 8) ? 3 : 4;
   static constexpr int T = NT * APT;
   static constexpr bool RAW = MULTI || APT == 16;  // the stencil acts on the raw vectors
+  static constexpr bool MSG = MULTI && F32;        // W_k travels in messages
   static_assert((1 << LT) == NT && (1 << LA) == APT, "powers of two");
 
   const EvalParams& p;
@@ -196,6 +222,7 @@ struct Tile {
   R cx;                // Sx control weight of the slice
   double hca;          // hc_amp, times 1/2 for an Sx control
   unsigned bonds_hi;   // MULTI: active bonds with both bits above the tile, bit b
+  unsigned seq;        // MSG: number of the newest W_k
   V wo[APT];           // own W_k
   float2 fact;         // complex64: this lane's entry of kInvFactFF
   float w1;            // one warp, complex64: its sums (lane i: sum i)
@@ -219,7 +246,8 @@ struct Tile {
   // -------------------------------------------------------------- sums over the block / the group
   // post: this thread's values into the warp partials (and, MULTI, the hand-over to the control
   // warp); collect (after the barrier that follows): the totals, the same bits in every thread.
-  __device__ __forceinline__ void post(const R (&v)[kTileSums]) {
+  // fence: what the CTA stored before is visible to who reads the sums (several CTAs).
+  __device__ __forceinline__ void post(const R (&v)[kTileSums], bool fence = true) {
     const int lane = tid & 31, warp = tid >> 5;
     const R s = warp_sum3<R>(v[0], v[1], v[2]);
     if constexpr (F32 && NW == 1) {
@@ -231,7 +259,7 @@ struct Tile {
       else sm.red_d[par][warp][lane] = s;
     }
     if constexpr (MULTI) {
-      if (tid == 0) sm.cmd = kTileCmdSums | (par << 2);
+      if (tid == 0) sm.cmd = kTileCmdSums | (fence ? kTileCmdFence : 0) | (par << 2);
       nbar_arrive(kTileBarPost, NT + 32);
     }
   }
@@ -268,7 +296,7 @@ struct Tile {
         if (lane == 0) sm.red_d[par][warp][i] = s;
       }
       if constexpr (MULTI) {  // the other CTAs' share arrives in float-float
-        if (tid == 0) sm.cmd = kTileCmdSums | kTileCmdFp64 | (par << 2);
+        if (tid == 0) sm.cmd = kTileCmdSums | kTileCmdFence | kTileCmdFp64 | (par << 2);
         nbar_arrive(kTileBarPost, NT + 32);
         S o[kTileSums];
         if (!collect(o)) return false;
@@ -377,27 +405,102 @@ struct Tile {
     constexpr int b = LT + LA - 1;
     return ((unsigned)(li(j) >> b) ^ (unsigned)(base >> (b + 1))) & 1u;
   }
-  // Blocks in flight: complex128 through a ring in shared memory, complex64 (8-byte amplitudes, which
-  // cp.async moves through L1 only) in registers.
-  static constexpr int RD = F32 ? (APT <= 4 ? 6 : 3) : (T <= 1024) ? 6 : 4;
-  V xr[MULTI && F32 ? RD : 1][MULTI && F32 ? APT : 1];
+  // Blocks in flight: complex128 through a ring in shared memory, complex64 in registers (more of them find
+  // more messages that have not arrived: 16 spins 59.4 us a slice with 2, 61.4 with 3, 75.5 with 4; 18
+  // spins 89.5 with 1, 98.4 with 2).
+  static constexpr int RD = F32 ? (NT <= 128 ? 2 : 1) : (T <= 1024) ? 6 : 4;
   __device__ __forceinline__ int cross_count() const {
     return 1 + __popc(bonds_hi) + ((p.hc_kind == KG_HC_SX_SITE && p.hc_site >= LT + LA) ? 1 : 0);
   }
-  // Block n, loaded into q; `act` as below.
-  __device__ __forceinline__ void cross_load(const V* w, int n, unsigned& act, V (&q)[MULTI && F32 ? APT : 1]) {
-    if constexpr (MULTI && F32) {
-      if (n == 0) {
+  // complex64: a thread's amplitudes of W_k travel as messages of three floats and the vector's number,
+  // which their readers poll: one trip through L2 for the exchange, where data, a fence and a barrier
+  // take three (m = 16: 16 spins 72.8 -> 59.4 us a slice, 13 spins 52 -> 40).  12 bytes an amplitude: two
+  // vectors' messages take the three vectors wbuf, xbuf of the workspace.  Every partner amplitude belongs to the same thread of another CTA (all bits
+  // of the thread's number lie below those that change), so that a message holds one thread's floats.
+  // Two sets, by the number's parity: number n + 2 is stored only after the sums that every CTA posted
+  // with n already read.  A message is never read in part: the two halves of the amplitudes (by the top bit of the tile) fill
+  // messages of their own, and what is left of the last one of each holds the number too and is checked.
+  // (With a component unused the compiler loads the others apart, and number and floats may then
+  // belong to different vectors.)
+  static constexpr int NH = (APT + 2) / 3, NA = 2 * NH;  // messages of a half, of a thread
+  static_assert(!MSG || NA * 16 <= 12 * APT, "the messages of two vectors fit three vectors");
+  Atom xa[MSG ? RD : 1][MSG ? NA : 1];
+  __device__ __forceinline__ ulonglong2* atoms(unsigned n, int r) const {
+    return reinterpret_cast<ulonglong2*>(p.wbuf) + ((size_t)(n & 1u) << (p.L - LT - LA)) * (NA * NT) + (size_t)r * (NA * NT) + tid;
+  }
+  __device__ __forceinline__ void send() {  // wo as the next number
+    if constexpr (MSG) {
+      ++seq;
+      ulonglong2* q = atoms(seq, rank);
 #pragma unroll
-        for (int j = 0; j < APT; ++j)
-          q[j] = top_active(j) ? ldv(w + ((base + li(j)) ^ ((size_t)3 << (LT + LA - 1)))) : vmake<V>(0, 0);
-      } else {
-        const V* s = w + (base ^ (act ? (size_t)3 << (__ffs(act) - 1) : (size_t)1 << p.hc_site));
-        act &= act - 1;
+      for (int a = 0; a < NA; ++a) {
+        float f[3];
 #pragma unroll
-        for (int j = 0; j < APT; ++j) q[j] = ldv(s + li(j));
+        for (int i = 0; i < 3; ++i) {
+          const int o = 3 * (a % NH) + i, n = a / NH * APT + min(o, APT - 1);  // float n of the thread
+          f[i] = (o >= APT) ? __uint_as_float(seq) : (float)(n & 1 ? wo[n / 2].y : wo[n / 2].x);
+        }
+        st_atom(q + a * NT, f[0], f[1], f[2], seq);
       }
     }
+  }
+  // The CTA of block n > 0; `act` (the active bonds from block n on) moves on.
+  __device__ __forceinline__ int cross_rank(unsigned& act) const {
+    const int r = rank ^ (act ? 3 << (__ffs(act) - 1 - LT - LA) : 1 << (p.hc_site - LT - LA));
+    act &= act - 1;
+    return r;
+  }
+  __device__ __forceinline__ void recv_issue(int r, int half, Atom (&q)[MSG ? NA : 1]) {
+    const ulonglong2* s = atoms(seq, r);
+#pragma unroll
+    for (int a = 0; a < NA; ++a)
+      if (half < 0 || a / NH == half) q[a] = ld_atom(s + a * NT);
+  }
+  static __device__ __forceinline__ bool is_number(const Atom& q, int a, unsigned n) {
+    bool is = q.seq == n;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (3 * (a % NH) + i >= APT) is = is && __float_as_uint(q.f[i]) == n;
+    return is;
+  }
+  // Polls until every atom of the block carries the number; gives up like the control warp, which then
+  // ends the evaluation (sm.lost).
+  __device__ __forceinline__ void recv_wait(int r, int half, Atom (&q)[MSG ? NA : 1]) {
+    const ulonglong2* s = atoms(seq, r);
+    unsigned polls = 0;
+    unsigned long long t0 = 0;
+    for (;;) {
+      bool open = false;
+#pragma unroll
+      for (int a = 0; a < NA; ++a) open |= (half < 0 || a / NH == half) && !is_number(q[a], a, seq);
+      if (!open) break;
+      if ((++polls & 31u) == 0u) {
+        bool give_up = ld_volatile_i32(p.ctrl + kCtrlAbort) != 0;
+        const unsigned long long now = globaltimer_ns();
+        if (t0 == 0) {
+          t0 = now;
+        } else if ((long long)(now - t0) > p.wait_limit_ns) {
+          atomicCAS(p.ctrl + kCtrlStatus, 0, (int)KG_ERR_TIMEOUT);
+          atomicExch(p.ctrl + kCtrlAbort, 1);
+          give_up = true;
+        }
+        if (give_up) {
+          sm.lost = 1;
+          break;
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < NA; ++a)
+        if ((half < 0 || a / NH == half) && !is_number(q[a], a, seq)) q[a] = ld_atom(s + a * NT);
+    }
+    __syncwarp();
+  }
+  static __device__ __forceinline__ float atom_float(const Atom (&q)[MSG ? NA : 1], int n) {
+    return q[n / APT * NH + n % APT / 3].f[n % APT % 3];
+  }
+  static __device__ __forceinline__ V atom_amp(const Atom (&q)[MSG ? NA : 1], int j) {
+    if constexpr (MSG) return vmake<V>(atom_float(q, 2 * j), atom_float(q, 2 * j + 1));
+    else return vmake<V>(0, 0);
   }
   // Copies of block n into slot n % RD; `act`: the active bonds from block n on.  One commit group per
   // block, empty past the last.
@@ -420,58 +523,73 @@ struct Tile {
   __device__ __forceinline__ void cross_issue(const V* w, unsigned& act) {
     act = bonds_hi;
     const int count = cross_count();
+    if constexpr (MSG) {
+      if (rank & 1) recv_issue(rank ^ 1, 1, xa[0]);
+      else recv_issue(rank ^ 1, 0, xa[0]);
 #pragma unroll
-    for (int n = 0; n < RD; ++n) {
-      if constexpr (F32) {
-        if (n < count) cross_load(w, n, act, xr[n]);
-      } else {
-        cross_copy(w, n, count, act);
-      }
+      for (int n = 1; n < RD; ++n)
+        if (n < count) recv_issue(cross_rank(act), -1, xa[n]);
+    } else {
+#pragma unroll
+      for (int n = 0; n < RD; ++n) cross_copy(w, n, count, act);
     }
   }
   __device__ __forceinline__ void cross_add(const V* w, unsigned act, V (&h)[APT]) {
     const int count = cross_count(), nb1 = 1 + __popc(bonds_hi);
-    V x[APT];
+    if constexpr (MSG) {
+      auto top = [&](int half) {  // the own amplitudes with the other top bit
+        recv_wait(rank ^ 1, half, xa[0]);
 #pragma unroll
-    for (int j = 0; j < APT; ++j) x[j] = vmake<V>(0, 0);
-    if constexpr (F32) {
-      auto take = [&](int n, const V (&q)[MULTI && F32 ? APT : 1]) {
-        if constexpr (MULTI && F32) {
-          if (n < nb1) {
-#pragma unroll
-            for (int j = 0; j < APT; ++j) x[j] = vadd(x[j], q[j]);
-          } else {
-#pragma unroll
-            for (int j = 0; j < APT; ++j) h[j] = vfma(cx, q[j], h[j]);
-          }
+        for (int j = 0; j < APT / 2; ++j) {
+          V& y = h[j + (half ? 0 : APT / 2)];
+          y = vfma(hxy, atom_amp(xa[0], j + (half ? APT / 2 : 0)), y);
         }
       };
+      if (rank & 1) top(1);
+      else top(0);
+      auto take = [&](int n, const Atom (&q)[NA]) {
+        const R c = (n < nb1) ? hxy : cx;
 #pragma unroll
-      for (int n = 0; n < RD; ++n)
-        if (n < count) take(n, xr[n]);
+        for (int j = 0; j < APT; ++j) h[j] = vfma(c, atom_amp(q, j), h[j]);
+      };
+      unsigned a2 = bonds_hi;
+#pragma unroll
+      for (int n = 1; n < RD; ++n) {
+        if (n < count) {
+          recv_wait(cross_rank(a2), -1, xa[n]);
+          take(n, xa[n]);
+        }
+      }
       for (int n = RD; n < count; ++n) {
-        cross_load(w, n, act, xr[0]);
-        take(n, xr[0]);
+        const int r = cross_rank(act);
+        recv_issue(r, -1, xa[0]);
+        recv_wait(r, -1, xa[0]);
+        take(n, xa[0]);
       }
     }
-    for (int n = 0; n < count && !F32; ++n) {
-      cp_async_wait<RD - 1>();
-      const V* r = ring + (n % RD) * T;
-      if (n == 0) {
+    if constexpr (!MSG) {
+      V x[APT];
 #pragma unroll
-        for (int j = 0; j < APT; ++j)
-          if (top_active(j)) x[j] = r[li(j)];
-      } else if (n < nb1) {
+      for (int j = 0; j < APT; ++j) x[j] = vmake<V>(0, 0);
+      for (int n = 0; n < count; ++n) {
+        cp_async_wait<RD - 1>();
+        const V* r = ring + (n % RD) * T;
+        if (n == 0) {
 #pragma unroll
-        for (int j = 0; j < APT; ++j) x[j] = vadd(x[j], r[li(j)]);
-      } else {
+          for (int j = 0; j < APT; ++j)
+            if (top_active(j)) x[j] = r[li(j)];
+        } else if (n < nb1) {
 #pragma unroll
-        for (int j = 0; j < APT; ++j) h[j] = vfma(cx, r[li(j)], h[j]);
+          for (int j = 0; j < APT; ++j) x[j] = vadd(x[j], r[li(j)]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < APT; ++j) h[j] = vfma(cx, r[li(j)], h[j]);
+        }
+        cross_copy(w, n + RD, count, act);
       }
-      cross_copy(w, n + RD, count, act);
-    }
 #pragma unroll
-    for (int j = 0; j < APT; ++j) h[j] = vfma(hxy, x[j], h[j]);
+      for (int j = 0; j < APT; ++j) h[j] = vfma(hxy, x[j], h[j]);
+    }
   }
 
   __device__ __forceinline__ V* sbasis(int k) const { return sw + k * T; }  // SB: v_k
@@ -556,20 +674,24 @@ struct Tile {
       const V* wk = (k > 0) ? gw(k) : src;
       unsigned act = 0u;
       stencil(sw + (k & 1) * T, wo, h);
+      if constexpr (MSG) {
+        cross_issue(wk, act);
+        cross_add(wk, act, h);
+      }
       if (k > 0) {  // alpha_{k-1}, b_k from the sums of step k - 1
         S o[kTileSums];
         if (!collect(o)) return false;
-        if constexpr (MULTI) cross_issue(wk, act);
+        if constexpr (MULTI && !MSG) cross_issue(wk, act);
         if (!step_scalars(k - 1, false, o, vp, wo, tol, amax, bmax, ap, bk, ib, broke)) return false;
         if (broke) {
           meff = k;
-          if constexpr (MULTI) cp_async_wait<0>();
+          if constexpr (MULTI && !MSG) cp_async_wait<0>();
           break;
         }
-      } else if constexpr (MULTI) {
+      } else if constexpr (MULTI && !MSG) {
         cross_issue(wk, act);
       }
-      if constexpr (MULTI) cross_add(wk, act, h);
+      if constexpr (MULTI && !MSG) cross_add(wk, act, h);
       R acc[3] = {0, 0, 0};
       V* sn = sw + ((k + 1) & 1) * T;
       V* vslot = (k > 0) ? gbasis(k) : nullptr;
@@ -586,11 +708,17 @@ struct Tile {
         wo[j] = w;
         if (!last) {
           sn[li(j)] = w;
-          if constexpr (MULTI) stv(gw(k + 1) + base + li(j), w);
+          if constexpr (MULTI && !MSG) stv(gw(k + 1) + base + li(j), w);
         }
-        if (k > 0) stv(vslot + li(j), v);
+        if (!MSG && k > 0) stv(vslot + li(j), v);
       }
-      post(acc);
+      if (MSG && !last) send();
+      post(acc, !MSG);
+      if constexpr (MSG) {
+#pragma unroll
+        for (int j = 0; j < APT; ++j)
+          if (k > 0) stv(vslot + li(j), vp[j]);
+      }
       sync();
     }
     if (meff > 0 && !broke) {  // the last step's sums: alpha_{m-1}, b_m of the error indicator
@@ -661,6 +789,7 @@ struct Tile {
       if constexpr (RAW) sw[li(j)] = wo[j];
       if (li(j) < D1) stv(dst + base + li(j), wo[j]);
     }
+    send();
   }
 
   // The amplitudes of vector v that Hc couples to the own ones (Sx: the flipped site; Sz: the same).
@@ -864,10 +993,16 @@ struct Tile {
       wo[j] = (li(j) < D1) ? ldv(v + base + li(j)) : vmake<V>(0, 0);
       if constexpr (RAW) sw[li(j)] = wo[j];
     }
+    send();
   }
 
   __device__ __forceinline__ bool run() {
     init();
+    if constexpr (MSG) {  // before the first reduction: no number of an earlier launch is left
+      seq = 0u;
+#pragma unroll
+      for (int a = 0; a < 2 * NA; ++a) st_atom(atoms(a & 1, rank) + (a >> 1) * NT, 0.f, 0.f, 0.f, 0u);
+    }
     S g, gi;
     // ---- psi_0
     {
@@ -1089,16 +1224,29 @@ __device__ __forceinline__ void tile_control(const EvalParams& p, TileSmem& sm, 
     } else {
       warps_sum3<NW, double>([&](int w, int i) { return sm.red_d[par][w][i]; }, c);
     }
-    const S mine = (lane == 0) ? c[0] : (lane == 1) ? c[1] : c[2];
-    fence_acq_rel();  // the workers' stores, ordered before this warp by the named barrier
+    const bool fence = (cmd & kTileCmdFence) != 0;
+    if (fence) fence_acq_rel();  // the workers' stores, ordered before this warp by the named barrier
     const bool skip = rank == 0 && ((p.debug_fault == 1 && seq == 1) || (p.debug_fault == 2 && seq == 2));
-    if (lane < kTileSums && !skip) st_msg(slots + rank * kNRed + lane, (unsigned long long)__double_as_longlong(spack(mine)), seq);
+    ulonglong2* out = slots + rank * kNRed + lane;
+    if constexpr (F32) {  // three float-float sums in two messages
+      if (lane == 0 && !skip) st_atom(out, c[0].hi, c[0].lo, c[1].hi, (unsigned)seq);
+      if (lane == 1 && !skip) st_atom(out, c[1].lo, c[2].hi, c[2].lo, (unsigned)seq);
+    } else {
+      const double mine = (lane == 0) ? c[0] : (lane == 1) ? c[1] : c[2];
+      if (lane < kTileSums && !skip) st_msg(out, (unsigned long long)__double_as_longlong(mine), seq);
+    }
     S t[kTileSums] = {S(), S(), S()};
-    bool ok = true;
+    bool ok = sm.lost == 0;
     unsigned long long t0 = 0;
     unsigned polls = 0;
+    using Msg = typename std::conditional<F32, Atom, ulonglong2>::type;
+    constexpr int NM = F32 ? 2 : 3;
+    auto numbered = [&](const Msg& q) {
+      if constexpr (F32) return q.seq == (unsigned)seq;
+      else return q.y == seq;
+    };
     for (int r = lane; r < size && ok; r += 64) {  // two slots in a round
-      ulonglong2 q[2][kTileSums];
+      Msg q[2][NM];
       unsigned open = (r + 32 < size) ? 3u : 1u;
       const bool two = open == 3u;
       for (;;) {
@@ -1106,12 +1254,19 @@ __device__ __forceinline__ void tile_control(const EvalParams& p, TileSmem& sm, 
         for (int i = 0; i < 2; ++i) {
           if ((open >> i) & 1u) {
 #pragma unroll
-            for (int j = 0; j < kTileSums; ++j) q[i][j] = ld_msg(slots + (r + 32 * i) * kNRed + j);
+            for (int j = 0; j < NM; ++j) {
+              if constexpr (F32) q[i][j] = ld_atom(slots + (r + 32 * i) * kNRed + j);
+              else q[i][j] = ld_msg(slots + (r + 32 * i) * kNRed + j);
+            }
           }
         }
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
-          if (((open >> i) & 1u) && q[i][0].y == seq && q[i][1].y == seq && q[i][2].y == seq) open &= ~(1u << i);
+        for (int i = 0; i < 2; ++i) {
+          bool all = true;
+#pragma unroll
+          for (int j = 0; j < NM; ++j) all = all && numbered(q[i][j]);
+          if (((open >> i) & 1u) && all) open &= ~(1u << i);
+        }
         if (!open) break;
         if ((++polls & 31u) == 0u) {
           if (ld_volatile_i32(p.ctrl + kCtrlAbort)) { ok = false; break; }
@@ -1128,14 +1283,22 @@ __device__ __forceinline__ void tile_control(const EvalParams& p, TileSmem& sm, 
       }
       if (ok) {
 #pragma unroll
-        for (int j = 0; j < kTileSums; ++j) t[j] = vx_add(t[j], sunpack(__longlong_as_double((long long)q[0][j].x), S()));
-        if (two)
+        for (int i = 0; i < 2; ++i) {
+          if (i == 1 && !two) break;
+          if constexpr (F32) {
+            const Atom &a = q[i][0], &b = q[i][1];
+            t[0] = vx_add(t[0], FF{a.f[0], a.f[1]});
+            t[1] = vx_add(t[1], FF{a.f[2], b.f[0]});
+            t[2] = vx_add(t[2], FF{b.f[1], b.f[2]});
+          } else {
 #pragma unroll
-          for (int j = 0; j < kTileSums; ++j) t[j] = vx_add(t[j], sunpack(__longlong_as_double((long long)q[1][j].x), S()));
+            for (int j = 0; j < kTileSums; ++j) t[j] = vx_add(t[j], __longlong_as_double((long long)q[i][j].x));
+          }
+        }
       }
     }
     ok = __all_sync(0xffffffffu, ok);
-    fence_acq_rel();  // what the workers read after the barrier was stored before the messages
+    if (fence) fence_acq_rel();  // what the workers read after the barrier was stored before the messages
     const S x = warp_sum3(t[0], t[1], t[2]);
     if (lane < kTileSums) sm.tot[par][lane] = spack(x);
     if (lane == 0) sm.ok = ok ? 1 : 0;
@@ -1152,6 +1315,7 @@ __device__ __forceinline__ void tile_cta(const EvalParams& p, TileSmem& sm, V* s
     sm.err_max = 0.f;
     sm.breakdowns = 0;
     sm.ok = 1;
+    sm.lost = 0;
     for (int i = 0; i < 8; ++i) sm.prof_acc[i] = 0;
     sm.prof_last = t0;
   }
@@ -1239,11 +1403,10 @@ TileKernel tile_multi(int L) {
 //   17.7, 64 x 8 18.5;  10: 128 x 8 22.2, 256 x 4 22.6;  11: 256 x 8 29.7, 512 x 4 34.8;
 //   12: 256 x 16 (raw vectors) 47.7, 512 x 8 61.0 (128 registers), 4 CTAs of 128 x 8 44.7.
 // (With three sums by one butterfly since: 8 11.3, 10 20.2, 11 27.3, 12 45.0.)  On several CTAs a step
-// costs 3.0 (16 CTAs) to 4.7 us (128), nearly all of it the exchange, so the tiles are as large as the
+// costs 2.3 (8 CTAs) to 5.3 us (128), nearly all of it the exchange, so the tiles are as large as the
 // registers let them be cheap:
-//   13: 128 x 4 52.2, 128 x 8 54.2;  14: 128 x 4 58.8, 128 x 8 59.3;  15: 128 x 8 64.4, 128 x 4 64.8, 128 x 2 75.7;
-//   16: 128 x 8 72.8, 256 x 4 72.9, 128 x 4 77.7;  17: 128 x 8 85.0, 256 x 8 89.1;  18: 256 x 8 101.1.
-// At L = 19 the resident loop is the faster one (139 against 171).
+//   13: 128 x 8 40.0;  14: 45.7;  15: 56.9;  16: 59.4;  17: 128 x 8 68.4, 256 x 8 81.4;  18: 256 x 8 89.5.
+// At L = 19 the resident loop is the faster one (139 against 171, both before the exchange by messages).
 // The kernels that ran these chains before took 100 (L = 5) to 148 us (L = 11), 77 us (L = 12) and, two
 // 4096-amplitude tiles per CTA, 128 (L = 13) to 164 us (L = 18).
 // complex128 is bound by the FP64 units, one quarter in each quarter of the SM: one warp per quarter
@@ -1263,7 +1426,6 @@ TileKernel pick_tile(int prec, int L, int m) {
     if (L == 10) return tile_single<float2, 128, 8>(m);
     if (L == 11) return tile_single<float2, 256, 8>(m);
     if (L == 12) return tile_single<float2, 256, 16>(m);
-    if (L <= 14) return tile_multi<float2, 128, 4>(L);
     if (L <= 17) return tile_multi<float2, 128, 8>(L);
     if (L == 18) return tile_multi<float2, 256, 8>(L);
   }

@@ -117,6 +117,17 @@ def test_group_that_a_member_never_joins_times_out_cleanly(prec, L):
     check(prec, *got[0], F_ref, g_ref)
 
 
+@pytest.mark.parametrize("L,hc", [(13, 0), (14, 13), (15, "sz"), (16, 15), (17, 0), (18, 17)])
+def test_exchange_by_messages_repeats_bit_for_bit(L, hc):
+    """Every amplitude and every sum is used as it was sent, whenever it arrives: each evaluation gives the same bits."""
+    u, psi0, f, spec, _ = problem(L, 12, 300 + L, hc)
+    opts = dict(N=12, dt=0.1, m=16, prec="c64", grad="centered")
+    F0, g0, _ = evaluate(spec, opts, u, psi0, f)
+    for _ in range(5):
+        F, g, _ = evaluate(spec, opts, u, psi0, f)
+        assert F == F0 and np.array_equal(g, g0)
+
+
 @pytest.mark.parametrize("prec", ["c64", "c128"])
 @pytest.mark.parametrize("L,N,C", [(4, 9, 2), (8, 11, 4), (9, 6, 1), (11, 10, 9), (7, 5, 7), (14, 7, 3)])
 def test_checkpoints_are_bitwise_equal_to_the_full_trajectory(L, N, C, prec):
