@@ -2112,12 +2112,20 @@ __device__ __forceinline__ unsigned str_outer(size_t base, int L1) {
 }
 
 // This thread's copies of block `bk` into ring stage st: stage layout [kStrDepth][4][512] float4.
+// Whole and half blocks apart: with the granules' numbers worked out one by one 21 spins took 930 instead
+// of 907 us a slice, 22 spins 2020 instead of 1980.
 __device__ __forceinline__ void str_issue(float4* ring, int st, const StrBlk& bk) {
   const int tid = threadIdx.x;
+  float4* to = ring + st * 4 * kThreads + tid;
+  const float2* from = bk.src + 2 * tid;
+  if (bk.gx == 0) {  // a whole block: one address, the granules at fixed distances from it
 #pragma unroll
-  for (int g = 0; g < 4; ++g)
-    if ((bk.gmask >> g) & 1u)
-      cp_async16(ring + (st * 4 + g) * kThreads + tid, bk.src + 2 * (size_t)(tid + ((g ^ bk.gx) << 9)));
+    for (int g = 0; g < 4; ++g) cp_async16(to + g * kThreads, from + (g << 10));
+  } else {  // half of one: granules 0, 1 from 2, 3 or the reverse
+    const int g0 = (bk.gmask & 1u) ? 0 : 2;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) cp_async16(to + (g0 + g) * kThreads, from + (((g0 ^ 2) + g) << 10));
+  }
 }
 
 // The stream of one step: for every own tile c (in order) its partner blocks, then X_{k-1}
@@ -2254,14 +2262,21 @@ __device__ __noinline__ bool lanczos_str64(Ctx<float2>& c, const float2* src, do
 #pragma unroll
       for (int g = 0; g < 4; ++g) xs[g] = f4zero();
       const int np = ((L1 > 11) ? 1 : 0) + __popc(str_outer(base, L1)) + (S.sx12 ? 1 : 0);
-      const unsigned half = ((base >> 12) & 1u) ? 0x3u : 0xcu;
       for (int b = 0; b < np; ++b) {
         const float wg = (S.sx12 && b == np - 1) ? cu_sx : hxy;
-        const unsigned gmask = (L1 > 11 && b == 0) ? half : 0xfu;
         const float4* q = str_wait(ring, cslot);
+        if (L1 > 11 && b == 0) {  // half a block
+          if ((base >> 12) & 1u) {
 #pragma unroll
-        for (int g = 0; g < 4; ++g)
-          if ((gmask >> g) & 1u) xs[g] = f4fma(wg, q[g * NT], xs[g]);
+            for (int g = 0; g < 2; ++g) xs[g] = f4fma(wg, q[g * NT], xs[g]);
+          } else {
+#pragma unroll
+            for (int g = 2; g < 4; ++g) xs[g] = f4fma(wg, q[g * NT], xs[g]);
+          }
+        } else {
+#pragma unroll
+          for (int g = 0; g < 4; ++g) xs[g] = f4fma(wg, q[g * NT], xs[g]);
+        }
         str_issue_next(c, S, iu, ring, islot);
         cslot = (cslot + 1 == kStrDepth) ? 0 : cslot + 1;
       }
