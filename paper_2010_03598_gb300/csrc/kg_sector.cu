@@ -179,6 +179,7 @@ struct SectorParams {
   unsigned maskL1, hc_mask;
   double qz, hc_amp, dt, bd_tol;
   double wa, wb;                 // weights of lists A and B
+  float wa_f, wb_f, dt_f, bd_tol_f;  // the same, dt and the breakdown tolerance rounded to FP32
   const unsigned* tab_g;         // [na2][rows] list A, [groups] meta words (sec_meta_*), list B
   const unsigned* states;        // [D] s_r of the kernel's row r
   const unsigned short* perm;    // [D] basis index of the kernel's row r
@@ -387,11 +388,13 @@ __device__ __forceinline__ float sec_times(const SecSmem& sm, int which, int n, 
   const float2 q = sm.diag_ff[which];
   return fmaf(q.x, (float)n, q.y * (float)n);
 }
-// The weights of lists A (2) and B (3) in the vectors' real type.  Complex64: converted from the
-// parameters, which the compiler does once; float-float and complex128: from shared memory, as their
-// conversion or constant operand in the loop costs FP64 issue (2 and 7 % at D = 2445).
+// The weights of lists A (2) and B (3) in the vectors' real type.  Complex64: rounded by the host (the
+// conversion of an FP64 parameter is an FP64 instruction, which every warp of every step repeated: D = 511 63.0 us a slice instead of 61.7, one
+// pulse at D = 110 16.3 instead of 15.3);
+// float-float and complex128: from shared memory, as their conversion or constant operand in the
+// loop costs FP64 issue (2 and 7 % at D = 2445).
 __device__ __forceinline__ float sec_weight(const SectorParams& p, const SecSmem&, int which, float) {
-  return (float)(which == 2 ? p.wa : p.wb);
+  return which == 2 ? p.wa_f : p.wb_f;
 }
 __device__ __forceinline__ FFR sec_weight(const SectorParams&, const SecSmem& sm, int which, FFR) {
   return FFR(sm.diag_ff[which].x, sm.diag_ff[which].y);
@@ -638,7 +641,7 @@ __device__ __forceinline__ void sec_coefficients(const SectorParams& p, SecSmem&
   // The exponential takes ceil(||tau T|| / 4) sub-steps: refuse a T whose Gershgorin bound is not a
   // finite, sane number (it would come from corrupted coefficients) instead of looping on it.
   float row = 0.f;
-  if (k < meff) row = (float)p.dt * (fabsf(sm.alpha_f[k]) + (k >= 1 ? sm.beta_f[k] : 0.f) + (k + 1 < meff ? sm.beta_f[k + 1] : 0.f));
+  if (k < meff) row = p.dt_f * (fabsf(sm.alpha_f[k]) + (k >= 1 ? sm.beta_f[k] : 0.f) + (k + 1 < meff ? sm.beta_f[k + 1] : 0.f));
   row = (row == row) ? row : 3.0e38f;  // NaN -> refused
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) row = fmaxf(row, __shfl_xor_sync(0xffffffffu, row, o));
@@ -747,7 +750,7 @@ __device__ __forceinline__ bool sec_slice(const SectorParams& p, SecSmem& sm, in
   bool broke = false;
   R alpha = 0, bk = 0, ib = 0;
   float amax = 0.f, bmax = 0.f, beta_m = 0.f;
-  const float tol = (float)p.bd_tol;
+  const float tol = p.bd_tol_f;
   for (int k = 0; k < meff; ++k) {
     const bool last = (k == m - 1);
     sec_sync();  // v_k is in shared memory
@@ -1712,6 +1715,10 @@ kg_status kg_sector_evaluate(kg_sector_handle* h, const double* u, const void* p
   p.dt = o.dt;
   p.bd_tol = o.breakdown_tol;
   list_weights(&s, p.wa, p.wb);
+  p.wa_f = (float)p.wa;
+  p.wb_f = (float)p.wb;
+  p.dt_f = (float)p.dt;
+  p.bd_tol_f = (float)p.bd_tol;
   char* ws = h->ws;
   p.tab_g = (const unsigned*)(ws + h->lay.tab);
   p.states = (const unsigned*)(ws + h->lay.states);
