@@ -55,9 +55,8 @@ namespace kg {
 // and the arithmetic on it is FP32 with error-free transformations (Knuth's TwoSum, the FMA
 // TwoProduct: ff_add, ff_mul), so that the rounding of the Krylov vectors -- what limits the
 // complex64 path over the 2 x 4D slices of Sec. 3.2's pulses -- shrinks by about 2^20 without one
-// FP64 instruction (1/64 of the FP32 rate on this GPU) per amplitude.  The scalars that steer the
-// recurrence (alpha, b, norms, overlaps) come from FP64 block sums of the float-float partials,
-// as on the complex128 path.
+// FP64 instruction (1/64 of the FP32 rate on this GPU) per amplitude.  alpha and b stay float-float too; the
+// norms and overlaps of a slice, T and its exponential are FP64, as on the complex128 path.
 struct FFR {
   float hi, lo;
   FFR() = default;
@@ -389,10 +388,9 @@ __device__ __forceinline__ float sec_times(const SecSmem& sm, int which, int n, 
   return fmaf(q.x, (float)n, q.y * (float)n);
 }
 // The weights of lists A (2) and B (3) in the vectors' real type.  Complex64: rounded by the host (the
-// conversion of an FP64 parameter is an FP64 instruction, which every warp of every step repeated: D = 511 63.0 us a slice instead of 61.7, one
-// pulse at D = 110 16.3 instead of 15.3);
-// float-float and complex128: from shared memory, as their conversion or constant operand in the
-// loop costs FP64 issue (2 and 7 % at D = 2445).
+// conversion of an FP64 parameter is an FP64 instruction, which every warp of every step repeated: D = 511
+// 63.0 us a slice instead of 61.7, one pulse at D = 110 16.3 instead of 15.3); float-float and complex128: from
+// shared memory, as their conversion or constant operand in the loop costs FP64 issue (2 and 7 % at D = 2445).
 __device__ __forceinline__ float sec_weight(const SectorParams& p, const SecSmem&, int which, float) {
   return which == 2 ? p.wa_f : p.wb_f;
 }
