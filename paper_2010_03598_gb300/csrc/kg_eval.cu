@@ -2857,16 +2857,24 @@ struct KernelChoice {
   const void* fn;
   size_t smem;
   int threads;
+  size_t smem_max;  // of any tile size: the kernel's limit, the same whichever call sets it (threads)
 };
+
+static cudaError_t set_smem_limit(const KernelChoice& k) {
+  return cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem_max);
+}
 
 template <class V, class A, int APT, int TPC, bool RES, int MODE>
 static KernelChoice choice(int t_bits) {
   constexpr int NB = RES ? TPC : 1;
   // complex64 streaming: two v_k tiles for the stencil plus the per-thread copy ring
-  const size_t smem = (MODE == kModeStream64)      ? kStrSmemBytes
-                      : (MODE == kModeResident64b) ? kRes64bSmemBytes
-                                                   : (size_t)(RES ? 3 : 2) * NB * ((size_t)1 << t_bits) * sizeof(V);
-  return {(const void*)kg_eval_kernel<V, A, APT, TPC, RES, MODE>, smem, eval_threads(MODE)};
+  auto bytes = [](size_t tile) {
+    return (MODE == kModeStream64)      ? (size_t)kStrSmemBytes
+           : (MODE == kModeResident64b) ? (size_t)kRes64bSmemBytes
+                                        : (size_t)(RES ? 3 : 2) * NB * tile * sizeof(V);
+  };
+  return {(const void*)kg_eval_kernel<V, A, APT, TPC, RES, MODE>, bytes((size_t)1 << t_bits), eval_threads(MODE),
+          bytes((size_t)kThreads * APT)};
 }
 
 // Variants: complex64 resident with full 4096-amplitude tiles (specialised loop), complex64
@@ -2889,7 +2897,7 @@ int resident_tiles_per_cta(int prec) { return prec == KG_PREC_C128 ? 0 : 2; }
 
 cudaError_t launch_eval_kernel(int prec, int variant, const EvalParams& p, int ctas, cudaStream_t stream) {
   KernelChoice k = pick(prec, variant, p.t_bits);
-  cudaError_t err = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+  cudaError_t err = set_smem_limit(k);
   if (err != cudaSuccess) return err;
   EvalParams pc = p;
   void* args[] = {&pc};
@@ -2898,7 +2906,7 @@ cudaError_t launch_eval_kernel(int prec, int variant, const EvalParams& p, int c
 
 cudaError_t eval_kernel_max_ctas(int prec, int variant, int t_bits, int* out) {
   KernelChoice k = pick(prec, variant, t_bits);
-  cudaError_t err = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+  cudaError_t err = set_smem_limit(k);
   if (err != cudaSuccess) return err;
   int per_sm = 0;
   err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, k.smem);

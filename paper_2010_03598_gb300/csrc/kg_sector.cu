@@ -1231,6 +1231,10 @@ static SecKernel sec_pick(int prec, int D, int nt = 0) {
 }
 
 constexpr int kSecMaxRows = 4096;  // 512 threads x 8 rows
+// Dynamic shared memory of the largest subspace taken (sector_fits; 202 KB is the most any needs), and
+// every kernel's limit: one value, so that no call can lower it between another host thread's setting and
+// launch.
+constexpr size_t kSecMaxSmem = 216 * 1024;
 
 size_t sector_smem_bytes(int prec, int D, int words) {
   const size_t vb = (prec == KG_PREC_C64_F64REC) ? 8 : 16;
@@ -1241,7 +1245,7 @@ cudaError_t sector_kernel_max_ctas(int prec, int D, int words, int nt, int* out)
   const SecKernel k = sec_pick(prec, D, nt);
   if (!k.fn) return cudaErrorInvalidValue;
   const size_t smem = sector_smem_bytes(prec, D, words);
-  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSecMaxSmem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1258,7 +1262,7 @@ cudaError_t launch_sector_kernel(int prec, const SectorParams& p, int ctas, int 
   const SecKernel k = sec_pick(prec, p.D, nt);
   if (!k.fn) return cudaErrorInvalidValue;
   const size_t smem = sector_smem_bytes(prec, p.D, p.words);
-  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSecMaxSmem);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<SectorParams*>(&p)};
   return cudaLaunchKernel(k.fn, dim3(ctas), dim3(k.threads), args, smem, stream);
@@ -1487,12 +1491,13 @@ kg_status check_sector_opts(const kg_options* o, int B) {
 }
 
 // Whether a subspace is taken: two vectors and one 16-bit column per row and antiparallel bond within
-// 200 KB (the split lists, which pad and double some entries, then stay below 224 KB).
+// 200 KB (the split lists, which pad and double some entries, then take at most 202 KB: L = 14, K = 7 without
+// parity).
 bool sector_fits(const kg_options* o, const SectorBasis& b) {
   const size_t vb = (o->prec == KG_PREC_C64_F64REC) ? 8 : 16;
   const size_t Dp = ((size_t)b.D + 15) & ~(size_t)15;
   return 2 * Dp * vb + (size_t)b.bonds * b.D * 2 <= 200 * 1024 &&
-         kg::sector_smem_bytes(o->prec, b.D, b.words()) <= 224 * 1024;
+         kg::sector_smem_bytes(o->prec, b.D, b.words()) <= kg::kSecMaxSmem;
 }
 
 // Grid for B pulses: every CTA that fits co-resident, at most B, at most opts->ctas.

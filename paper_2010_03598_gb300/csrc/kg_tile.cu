@@ -1366,9 +1366,16 @@ struct TileKernel {
   const void* fn = nullptr;    // one problem (EvalParams by value)
   const void* list = nullptr;  // complex64: a list of problems
   int threads = 0, tile_bits = 0;
-  size_t smem = 0;
+  size_t smem = 0;      // of this call (a basis in shared memory grows with m)
+  size_t smem_max = 0;  // of any call
   int ctas = 1;
 };
+
+// A kernel's limit is shared by the whole process: every call sets the same one, so that none can lower
+// it between another host thread's setting and launch.
+cudaError_t set_smem_limit(const void* fn, const TileKernel& k) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem_max);
+}
 
 // Basis in shared memory up to this size.
 constexpr size_t kTileSmemBasis = 100 * 1024;
@@ -1376,7 +1383,7 @@ constexpr size_t kTileSmemBasis = 100 * 1024;
 template <class V, int NT, int APT, bool SB>
 TileKernel tile_choice(size_t smem) {
   TileKernel k{reinterpret_cast<const void*>(&kg_tile_kernel<V, NT, APT, SB, false>), nullptr, NT,
-               __builtin_ctz(NT * APT), smem};
+               __builtin_ctz(NT * APT), smem, SB ? kTileSmemBasis : smem};
   if constexpr (sizeof(V) == 8) k.list = reinterpret_cast<const void*>(&kg_tile_list_kernel<V, NT, APT, SB>);
   return k;
 }
@@ -1393,8 +1400,9 @@ template <class V, int NT, int APT>
 TileKernel tile_multi(int L) {
   using TileT = Tile<V, NT, APT, false, true>;
   const int t = __builtin_ctz(NT * APT);
-  return {reinterpret_cast<const void*>(&kg_tile_kernel<V, NT, APT, false, true>), nullptr, NT + 32, t,
-          (size_t)(2 + (sizeof(V) == 16 ? TileT::RD : 0)) * TileT::T * sizeof(V), 1 << (L - t)};
+  const size_t smem = (size_t)(2 + (sizeof(V) == 16 ? TileT::RD : 0)) * TileT::T * sizeof(V);
+  return {reinterpret_cast<const void*>(&kg_tile_kernel<V, NT, APT, false, true>), nullptr, NT + 32, t, smem, smem,
+          1 << (L - t)};
 }
 
 // Threads x amplitudes by chain length.  More threads shorten every thread's chain of shared-memory
@@ -1450,7 +1458,7 @@ bool tile_kernel_covers(int prec, int L) {
   if (!k.fn || k.ctas == 1) return k.fn != nullptr;
   // the CTAs of a group wait for one another: all of them have to be resident at once
   int per_sm = 0, dev = 0, sms = 0;
-  if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) != cudaSuccess ||
+  if (set_smem_limit(k.fn, k) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, k.smem) != cudaSuccess ||
       cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -1468,7 +1476,7 @@ size_t tile_kernel_clear_bytes(int prec, int L) {
 cudaError_t launch_tile_kernel(int prec, const EvalParams& p, cudaStream_t stream) {
   const TileKernel k = pick_tile(prec, p.L, p.m);
   if (!k.fn) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+  cudaError_t e = set_smem_limit(k.fn, k);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<EvalParams*>(&p)};
   if (k.ctas > 1) return cudaLaunchCooperativeKernel(k.fn, dim3(k.ctas), dim3(k.threads), args, k.smem, stream);
@@ -1478,7 +1486,7 @@ cudaError_t launch_tile_kernel(int prec, const EvalParams& p, cudaStream_t strea
 cudaError_t launch_tile_list(int L, int m, const EvalParams* list, int n, cudaStream_t stream) {
   const TileKernel k = pick_tile(KG_PREC_C64_F64REC, L, m);
   if (!k.list) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k.list, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+  cudaError_t e = set_smem_limit(k.list, k);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<EvalParams**>(&list)};
   return cudaLaunchKernel(k.list, dim3(n), dim3(k.threads), args, k.smem, stream);
