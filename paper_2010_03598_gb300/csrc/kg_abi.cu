@@ -835,18 +835,29 @@ kg_status kg_batch_launch(kg_batch* b) {
   if (!b->classes.empty()) {
     const size_t n = b->classes.size();
     if (n > 1 && (e = cudaEventRecord(b->fork, b->stream)) != cudaSuccess) return cuda_fail(e, "cudaEventRecord(batch)");
-    for (size_t i = 0; i < n; ++i) {
+    const char* what = "";
+    size_t forked = 1;  // streams that wait for the fork so far, the caller's among them
+    for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
       const BatchClass& c = b->classes[i];
       cudaStream_t s = (i == 0) ? b->stream : b->streams[i - 1];
-      if (i > 0 && (e = cudaStreamWaitEvent(s, b->fork, 0)) != cudaSuccess) return cuda_fail(e, "cudaStreamWaitEvent(batch)");
+      what = "cudaStreamWaitEvent(batch)";
+      if (i > 0 && (e = cudaStreamWaitEvent(s, b->fork, 0)) != cudaSuccess) break;
+      forked = i + 1;
       const kg::EvalParams* list = b->bp.probs + c.first;
+      what = "launch of a batch class";
       e = (c.size == 0) ? kg::launch_tile_list(c.L, b->opts.m, list, c.n, s) : kg::launch_cluster_list(c.size, list, c.n, s);
-      if (e != cudaSuccess) return cuda_fail(e, "launch of a batch class");
-      if (i > 0 && ((e = cudaEventRecord(b->done[i - 1], s)) != cudaSuccess ||
-                    (e = cudaStreamWaitEvent(b->stream, b->done[i - 1], 0)) != cudaSuccess))
-        return cuda_fail(e, "join of a batch class");
     }
-    return KG_OK;
+    // Joined whatever happened: the classes launched before a failure still write the caller's buffers and
+    // the workspace, and a capture has to get its streams back.
+    for (size_t i = 1; i < forked; ++i) {
+      cudaError_t je = cudaEventRecord(b->done[i - 1], b->streams[i - 1]);
+      if (je == cudaSuccess) je = cudaStreamWaitEvent(b->stream, b->done[i - 1], 0);
+      if (je != cudaSuccess && e == cudaSuccess) {
+        e = je;
+        what = "join of a batch class";
+      }
+    }
+    return e == cudaSuccess ? KG_OK : cuda_fail(e, what);
   }
   e = kg::launch_batch_kernel(b->bp, b->ctas, b->stream);
   if (e != cudaSuccess) return cuda_fail(e, "cooperative launch of the batch kernel");

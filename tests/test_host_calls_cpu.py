@@ -155,3 +155,30 @@ def test_a_kernels_shared_memory_limit_does_not_depend_on_the_call(fake):
             assert int(c[2]) <= min(limit[c[1]]), c
     assert launched >= n > 100
     assert all(len(v) == 1 for v in limit.values()), {k: sorted(v) for k, v in limit.items() if len(v) > 1}
+
+
+BATCH = r"""
+B = 6
+cs = (a.KgChain * B)(*[chain(L) for L in (6, 9, 10, 13, 14, 16)])
+ptrs = (ctypes.c_void_p * B)(*[1 << 20] * B)
+h = ctypes.c_void_p()
+o = opts()
+a.check(lib.kg_batch_create(ctypes.byref(h), B, cs, o, None, ptrs, ptrs, ptrs, P, ptrs, WS, 1 << 50, ctypes.c_void_p(0x77)), "batch")
+print(json.dumps(lib.kg_batch_launch(h)))
+"""
+
+
+@pytest.mark.parametrize("fail", [None, 0, 1, 3, 5])
+def test_a_batch_joins_its_streams_even_if_a_launch_fails(fake, fail):
+    # One launch per chain length on a stream each; `fail` is the launch that the runtime refuses.  Whatever was
+    # launched on a side stream has to be waited for by the caller's stream: it writes the caller's buffers.
+    status, calls = fake(BATCH, fail)
+    assert status == (_abi.KG_OK if fail is None else _abi.KG_ERR_CUDA)
+    caller = "0x77"
+    started = {c[3] for c in calls if c[0] == "launch" and c[4] == "0"}
+    assert len(started) == (6 if fail is None else fail)
+    forked = {c[1] for c in calls if c[0] == "wait" and c[1] != caller}
+    for s in (started | forked) - {caller}:
+        last = max(i for i, c in enumerate(calls) if (c[0] == "launch" and c[3] == s) or (c[0] == "wait" and c[1] == s))
+        events = {c[1]: i for i, c in enumerate(calls) if c[0] == "record" and c[2] == s and i > last}
+        assert any(c[0] == "wait" and c[1] == caller and i > events.get(c[2], len(calls)) for i, c in enumerate(calls)), s
