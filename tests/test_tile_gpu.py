@@ -181,3 +181,18 @@ def test_subspace_norm_does_not_drift_in_complex64(dt):
     assert rep["status"] == 0
     assert abs(rep["norm_final"] - 1.0) <= 4 * 6e-8 * np.sqrt(N) + 1e-7
     eng.close()
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("L", [6, 9, 12, 14, 18])
+@pytest.mark.parametrize("norm", [2.2, 4.2])
+def test_checkpoints_are_bitwise_equal_for_any_norm(prec, L, norm):
+    # The recomputed first slice starts from 1 / ||psi_0|| as the forward sweep took it: at these norms the
+    # reciprocal of the stored norm rounds differently.
+    rng = np.random.default_rng(int(norm))
+    psi0 = rng.standard_normal(1 << L) + 1j * rng.standard_normal(1 << L)
+    psi0 *= norm / np.linalg.norm(psi0)
+    u, _, f, spec, _ = problem(L, 8, 3, 0)
+    full = evaluate(spec, dict(N=8, dt=0.05, m=10, prec=prec, grad="centered"), u, psi0, f)
+    ckpt = evaluate(spec, dict(N=8, dt=0.05, m=10, prec=prec, grad="centered", ckpt_every=3), u, psi0, f)
+    assert full[0] == ckpt[0] and np.array_equal(full[1], ckpt[1])
