@@ -8,7 +8,8 @@ Three searches, each keyed by (GPU name, kind, the problem's size, m, precision,
   tiles, streaming) and the CTAs how the tiles are dealt.
 * ``tune_sector``: threads per CTA of the parity-excitation subspace kernel
   (``SectorSpec.block_threads``) and its grid (``Options.ctas``: CTAs, i.e. pulses in flight).
-* ``tune_batch``: CTAs of the batched launch and tiles per CTA.
+* ``tune_batch``: the library's own batch schedule (one launch per chain length), or one cooperative launch
+  with so many CTAs and tiles per CTA.
 
 Every candidate computes the same quantity; schedules that change the tiling sum in another
 order, so results agree to rounding (and bitwise where only the grid of the same loop changes).
@@ -178,6 +179,7 @@ def signature(chains, opts: api.Options) -> str:
 
 
 def batch_candidates(sms: int) -> list[dict]:
+    """Cooperative launches: CTAs x tiles per CTA."""
     out = []
     for ctas in sorted({sms, (sms // 8) * 8, sms // 2}, reverse=True):
         for tpc in (2, 1):
@@ -188,7 +190,8 @@ def batch_candidates(sms: int) -> list[dict]:
 def tune_batch(chains, opts: api.Options, u, psi0, target, device=None, repeats: int = 2,
                cache_path: str | None = None, force: bool = False, timer=None, gpu: str | None = None,
                sms: int | None = None) -> dict:
-    """Fastest schedule {ctas, tiles_per_cta, ms} for this batch (cached by the batch's signature)."""
+    """Fastest schedule {ctas, tiles_per_cta, ms} for this batch (cached by the batch's signature); both 0: the
+    library's own."""
     if timer is None:
         dev, gpu, sms = _gpu(device)
 
@@ -201,4 +204,5 @@ def tune_batch(chains, opts: api.Options, u, psi0, target, device=None, repeats:
             finally:
                 b.close()
     key = cache_key(gpu or "gpu", "batch", sig=signature(chains, opts))
-    return search(key, batch_candidates(sms or 152), timer, cache_path, force)
+    candidates = [dict(ctas=0, tiles_per_cta=0)] + batch_candidates(sms or 152)
+    return search(key, candidates, timer, cache_path, force)
