@@ -1,7 +1,8 @@
 """Schedule autotuner: times candidate launch schedules through the C ABI on the current GPU and
 caches the fastest in a JSON file (``$KG_TUNE_CACHE``, default ``~/.cache/kgrape_tune.json``).
 
-Three searches, each keyed by (GPU name, kind, the problem's size, m, precision, gradient mode):
+Three searches, each keyed by (GPU name, version of the library's sources, kind, the problem's size, m,
+precision, gradient mode):
 
 * ``tune_single``: tile size x CTAs of a single-problem engine (``Options.tile_bits``, ``ctas``);
   the tile size decides the loop (resident pairs of 4096-amplitude tiles, resident smaller
@@ -19,12 +20,14 @@ candidate and returns milliseconds), which lets the search and the cache be chec
 from __future__ import annotations
 
 import dataclasses
+import functools
 import hashlib
 import json
 import os
 
 from . import _abi, api
 
+SOURCES = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc")
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "kgrape_tune.json")
 
 
@@ -45,9 +48,22 @@ def _store(path, cache):
         pass
 
 
+@functools.lru_cache(maxsize=None)
+def library_version() -> str:
+    """Hash of the kernels' and the launch code's sources (of the built library where they are missing): what
+    runs under a schedule changes with them."""
+    names = os.listdir(SOURCES) if os.path.isdir(SOURCES) else []
+    paths = sorted(os.path.join(SOURCES, f) for f in names if f.endswith((".cu", ".cuh", ".h"))) or [_abi.LIB_PATH]
+    h = hashlib.sha256()
+    for path in paths:
+        with open(path, "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()[:12]
+
+
 def cache_key(gpu: str, kind: str, **size) -> str:
-    """`gpu|kind|k=v,...` over the sorted size fields (e.g. L, m, prec, grad)."""
-    return f"{gpu}|{kind}|" + ",".join(f"{k}={size[k]}" for k in sorted(size))
+    """`gpu|version|kind|k=v,...` over the sorted size fields (e.g. L, m, prec, grad)."""
+    return f"{gpu}|{library_version()}|{kind}|" + ",".join(f"{k}={size[k]}" for k in sorted(size))
 
 
 def search(key: str, candidates: list[dict], measure, cache_path: str | None = None, force: bool = False) -> dict:
