@@ -18,6 +18,7 @@ constexpr size_t kCtrlBytes = 256; // control block cleared before each launch: 
 // Scalars kept in the workspace (float64 unless stated).
 enum ScalarIdx {
   kScBetaRe = 0, kScBetaIm = 1, kScErrMax = 2, kScNormFinal = 3, kScBreakdowns = 4,
+  kScInv0 = 5,  // register-tile kernel, complex64: 1 / ||psi_0|| as the first slice took it
   kScCount = 8
 };
 

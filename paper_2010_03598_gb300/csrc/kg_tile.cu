@@ -147,7 +147,6 @@ struct TileSmem {
   double coef_re[3][kMaxM], coef_im[3][kMaxM];
   float coef_re_f[3][kMaxM], coef_im_f[3][kMaxM];
   float2 tau_ff[3];          // complex64: dt and the interior quadrature nodes s_a, s_b of a slice
-  double inv0;               // 1 / ||psi_0|| as the first slice took it (in R)
   float err_max;
   int breakdowns;
   int cmd, ok;               // control warp: hand-over and answer
@@ -1027,7 +1026,7 @@ struct Tile {
       const double n = sqrt(fmax(o[0], 0.0));
       nrm = sfrom(n, S());
       inv = (n > 0.0) ? (R)(1.0 / n) : (R)0;
-      if (tid == 0) sm.inv0 = (double)inv;
+      if (F32 && rank == 0 && tid == 0) p.scal[kScInv0] = (double)inv;
     }
     const bool lead = (rank == 0 && tid == 0);
     if (lead) p.nrm[0] = spack(nrm);
@@ -1110,7 +1109,7 @@ struct Tile {
         sync();
         load_state(seg_slot(a, a));
         nrm = sunpack(__ldcg(p.nrm + a), S());
-        inv = (a == 0) ? (R)sm.inv0 : sinv(nrm);  // psi_0's was rounded once, from FP64
+        inv = (F32 && a == 0) ? (R)__ldcg(p.scal + kScInv0) : sinv(nrm);  // psi_0's was rounded once, from FP64
         sync();
         kind = kRecompute;
         j = a + 1;
