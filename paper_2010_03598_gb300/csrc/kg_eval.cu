@@ -796,7 +796,7 @@ __device__ __forceinline__ bool finish_slice(Ctx<V>& c, const V* src, double nrm
       // a-posteriori indicator ||psi|| b_m |c_{m-1}| (= b_m |coef_{m-1}| for m > 1), in FP32;
       // where the Taylor series stopped before index m-1, ||psi|| b_m ||tau T||^(m-1)/(m-1)!
       // bounds it instead
-      float cm = sqrtf(ss.coef_re_f[tid] * ss.coef_re_f[tid] + ss.coef_im_f[tid] * ss.coef_im_f[tid]);
+      float cm = hypotf(ss.coef_re_f[tid], ss.coef_im_f[tid]);  // the squares may underflow
       if (tid == 0) cm *= ss.f_bk0;
       if (cm == 0.f && !broke) {
         cm = ss.f_bk0;

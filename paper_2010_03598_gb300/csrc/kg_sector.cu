@@ -685,7 +685,7 @@ __device__ __forceinline__ void sec_coefficients(const SectorParams& p, SecSmem&
     n0 = (float)nrm;
   }
   if (w == 0 && k == meff - 1) {  // a-posteriori indicator ||x|| b_m |c_{m-1}| (0 after a breakdown)
-    float cm = sqrtf(cre * cre + cim * cim);
+    float cm = hypotf(cre, cim);  // the squares may underflow
     if (cm == 0.f && !broke) {
       cm = n0;
       for (int i = 1; i < meff; ++i) cm *= tnorm * kInvFF[i].x;

@@ -906,7 +906,7 @@ struct Tile {
         // m - 1, ||x|| b_m ||tau T||^(m-1)/(m-1)! bounds it
         const float n0 = (float)sround(nrm);
         const float re = (float)cr, im = (float)ci;
-        float cm = sqrtf(re * re + im * im);
+        float cm = hypotf(re, im);  // the squares may underflow
         if (lane == 0) cm *= n0;
         if (cm == 0.f) {
           cm = n0;
