@@ -1391,9 +1391,13 @@ TileKernel tile_choice(size_t smem) {
 template <class V, int NT, int APT>
 TileKernel tile_single(int m) {
   constexpr size_t vec = (size_t)NT * APT * sizeof(V);
-  if constexpr (APT < 16)
-    if (m * vec <= kTileSmemBasis) return tile_choice<V, NT, APT, true>(m * vec);
-  return tile_choice<V, NT, APT, false>(2 * vec);
+  if constexpr (APT < 16 && kMaxM * vec <= kTileSmemBasis) {  // whatever m
+    return tile_choice<V, NT, APT, true>(m * vec);
+  } else {
+    if constexpr (APT < 16)
+      if (m * vec <= kTileSmemBasis) return tile_choice<V, NT, APT, true>(m * vec);
+    return tile_choice<V, NT, APT, false>(2 * vec);
+  }
 }
 
 // One of several CTAs: two W_k buffers and (complex128) the ring of partner blocks.
