@@ -52,9 +52,22 @@ typedef enum kg_status {
 } kg_status;
 
 typedef enum kg_precision {
-  KG_PREC_C128 = 0,        /* complex128 vectors, FP64 arithmetic throughout */
-  KG_PREC_C64_F64REC = 1,  /* complex64 vectors and H*v in FP32; alpha/beta recurrences,
-                              norms, the m x m exponential and <f|psi_N> in FP64 */
+  KG_PREC_C128 = 0,        /* complex128 vectors, FP64 arithmetic throughout; only the error
+                              indicator and (chains up to 18 spins by default, subspaces) the
+                              breakdown test's comparison are FP32 */
+  KG_PREC_C64_F64REC = 1,  /* complex64 vectors and H*v in FP32.  Sums: FP32 within a warp, float-
+                              float (hi + lo FP32, about 44 bits) over warps and CTAs.  alpha, b,
+                              the tridiagonal, the norms and the overlaps G_j follow from them in
+                              float-float (chains of up to 18 spins with the schedule left to the
+                              library, batches likewise on single CTAs, subspaces) or in FP64
+                              (elsewhere); the m x m exponential is float-float, and the factors
+                              that multiply vectors are rounded to FP32.  FP64: ||psi_0||, ||chi_N||
+                              and <f|psi_N> (their sums over several CTAs float-float on the
+                              default path up to 18 spins).  Both forms are at the rounding of the
+                              complex64 vectors: mean gradient error 1.2e-7 to 1.8e-7 with float-
+                              float scalars, 1.7e-7 to 2.1e-7 with FP64 ones (14 to 18 spins, N =
+                              24, m = 16); 200 slices of 16 spins: F 1.4e-6, gradient 1.0e-6 and
+                              F 1.7e-6, gradient 1.3e-6 */
   KG_PREC_FF = 2           /* float-float vectors: each real part and imaginary part is the
                               unevaluated sum hi + lo of two FP32 numbers (about 44 significant
                               bits), H*v, the Lanczos updates, the recombination and the Lanczos
@@ -125,7 +138,17 @@ typedef struct kg_options {
   int32_t tile_bits;       /* 0 = automatic; else amplitudes per tile = 2^tile_bits (6..13) */
   int32_t ctas;            /* 0 = automatic; else CTAs cooperating on the problem.  With both 0, chains
                               of up to 18 spins run with one tile in the registers of each CTA
-                              (complex64 one CTA up to 12 spins, complex128 up to 8) */
+                              (complex64 one CTA up to 12 spins, complex128 up to 8).  That is the
+                              schedule of least latency for one evaluation: its CTAs (kg_report.ctas,
+                              up to 128) take an SM each.  More engines side by side on streams of
+                              their own than the SMs hold wait for each other, and from about 15
+                              spins on they finish more per second with fewer CTAs: complex64
+                              tile_bits = 12, ctas = 2^(L-13); complex128 of 14 spins tile_bits = 11.
+                              16 engines, N = 12, m = 16, ms an evaluation, default / so: 14 spins
+                              0.15 / 0.22, 15 spins 0.34 / 0.23, 16 spins 0.74 / 0.25, 17 spins
+                              1.60 / 0.49, 18 spins 2.08 / 0.99 (one engine: 1.4 to 2.1 / 3.4 to
+                              3.7); complex128, N = 6, m = 12: 14 spins 0.68 / 0.44, the default
+                              ahead at the other lengths.  Pulses known together: kg_batch_* */
   int32_t flags;           /* KG_FLAG_* */
   double dt;               /* slice length, dt > 0 */
   double breakdown_tol;    /* <= 0: 1e-12 (C128) or 1e-5 (C64); Lanczos stops when

@@ -42,15 +42,15 @@ class Options:
     N: int
     dt: float
     m: int
-    prec: str = "c64"         # "c64" (complex64 state, FP64 recurrences), "c128", or "ff" (float-float
-                              # vectors; subspace engines only)
+    prec: str = "c64"         # "c64" (complex64 state, recurrences in FP64 or float-float: see kgrape.h),
+                              # "c128", or "ff" (float-float vectors; subspace engines only)
     grad: str = "centered"    # "none", "centered", "zeroth", "exact" (Gauss-Lobatto over each slice),
                               # "taylor1", "taylor2" (App. B's hierarchy; subspace engines only)
     ckpt_every: int = 0       # 0: keep every psi_j; C > 0: checkpoint every C slices; -1 (KG_CKPT_AUTO):
                               # every psi_j if the workspace fits mem_budget, else every ceil(sqrt(N))
     mem_budget: int = 0       # bytes for KG_CKPT_AUTO (0: 90 % of the device's free memory)
-    tile_bits: int = 0
-    ctas: int = 0
+    tile_bits: int = 0        # both 0: least latency for one evaluation; for many engines side by side on
+    ctas: int = 0             # streams of their own tile_bits=12, ctas=2**(L - 13) (c64, 15 to 18 spins)
     host_staging: bool = False
     phase_timing: bool = False
     breakdown_tol: float = 0.0

@@ -772,7 +772,7 @@ __device__ __forceinline__ bool finish_slice(Ctx<V>& c, const V* src, double nrm
       }
     }
   }
-  // ---- small exponential and recombination coefficients (warp 0, FP64)
+  // ---- small exponential and recombination coefficients (warp 0; complex64: T in FP64, series in float-float)
   if (tid < 32) {
     const bool broke = ss.broke != 0;
     double cr = 0.0, ci = 0.0;

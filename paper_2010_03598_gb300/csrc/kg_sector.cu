@@ -32,9 +32,10 @@
 //   alpha_k = <v_k|w>,  b_{k+1}^2 = ||w||^2 - 2 alpha_k <v_k|w> + alpha_k^2 ||v_k||^2   (one block reduction)
 //   v_{k+1} = (w - alpha_k v_k) / b_{k+1}               (into shared memory and the basis)
 // with two block barriers: every warp adds up the warps' partial sums and forms the scalars for itself.
-// Complex64 path: vectors and partial sums in FP32, cross-warp sums, the tridiagonal T and its
-// exponential in float-float (warp 0, once per slice): no FP64 instruction between the first slice and
-// the last.  Complex128 path: FP64 throughout.
+// Complex64 path: vectors and partial sums in FP32, cross-warp sums, the tridiagonal T, its exponential and the
+// norms between slices in float-float (warp 0, once per slice): a step has no FP64 instruction, a slice only
+// the conversion of its control.  Complex128 path: FP64 throughout (the error indicator and the breakdown
+// test, a comparison with a tolerance, in FP32).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -5,16 +5,16 @@
 // each) an evaluation is a chain of short Krylov steps, whose cost is latency: block
 // barriers, warp sums, the recurrence's scalars and the small exponential.  This kernel is laid out
 // for that chain.  A CTA has as many threads as its tile needs (a thread owns APT amplitudes
-// li = tid + NT j), one barrier per Lanczos step, and no FP64 instruction on the complex64 path
-// between the first slice and the last: one FP64 instruction occupies a quarter of the SM's FP64
-// unit for 64 cycles whatever the number of active lanes, so padding warps and scalar chains in
-// FP64 are what small chains spend their time on otherwise.
+// li = tid + NT j), two block barriers per Lanczos step, and on the complex64 path a step has no FP64
+// instruction (a slice has a few: the conversions and prefactors of set_control): one FP64 instruction
+// occupies a quarter of the SM's FP64 unit for 64 cycles whatever the number of active lanes, so padding
+// warps and scalar chains in FP64 are what small chains spend their time on otherwise.
 //
 // One Lanczos step (App. A, Alg. "Lanczos", Paige's order), v_k in shared memory for the neighbours:
 //   W_{k+1} = H v_k - b_k v_{k-1},   H v = diag v + (Jxy/2) sum_{antiparallel bonds} v[partner] (+ control)
 //   alpha_k = <v_k|W_{k+1}>,  b_{k+1}^2 = ||W_{k+1}||^2 - 2 alpha_k <v_k|W_{k+1}> + alpha_k^2 ||v_k||^2
 //   v_{k+1} = (W_{k+1} - alpha_k v_k) / b_{k+1}
-// with two block barriers (the sums, v_{k+1}); every warp adds up the warps' partial sums and forms the
+// with the two block barriers (the sums, v_{k+1}); every warp adds up the warps' partial sums and forms the
 // scalars for itself.  v_{k-1}, v_k and W stay in registers; the basis holds the v_k (shared memory if
 // it fits, else global).
 //
@@ -1419,7 +1419,7 @@ TileKernel tile_multi(int L) {
 // costs 2.3 (8 CTAs) to 5.3 us (128), nearly all of it the exchange, so the tiles are as large as the
 // registers let them be cheap:
 //   13: 128 x 8 40.0;  14: 45.7;  15: 56.9;  16: 59.4;  17: 128 x 8 68.4, 256 x 8 81.4;  18: 256 x 8 89.5.
-// At L = 19 the resident loop is the faster one (139 against 171, both before the exchange by messages).
+// At L = 19 the resident loop is the faster one (m = 20: 154.5 us a slice; 128 CTAs of 512 x 8 198.1).
 // The kernels that ran these chains before took 100 (L = 5) to 148 us (L = 11), 77 us (L = 12) and, two
 // 4096-amplitude tiles per CTA, 128 (L = 13) to 164 us (L = 18).
 // complex128 is bound by the FP64 units, one quarter in each quarter of the SM: one warp per quarter
